@@ -109,10 +109,11 @@ typedef struct {
  *   L         pool size, 1 <= L <= ANN_MAX_L; the maximum when d_L is given
  *   W         pool entries expanded per step, 1..ANN_MAX_W, W*degree <= 128
  *   hash_bits log2 of the per-query shared-memory visited-table capacity,
- *             0 = chosen from L; 8..15; -1 = no shared table (the visited set
- *             lives in the global spill tables from the first step)
+ *             0 = chosen: the largest up to 32 KB that leaves every SM its
+ *             share of the queries, else none; 8..15; -1 = no shared table (the
+ *             visited set lives in the global spill tables from the first step)
  *   stage_rows neighbour rows gathered into shared memory per round, 0 =
- *             chosen from the row size; 1..32.  hash_bits and stage_rows change
+ *             chosen from the row size and nq; 1..32.  hash_bits and stage_rows change
  *             speed only, never results (see ann_autotune)
  *   team      lanes that compute one distance together (the warp evaluates
  *             32/team staged rows at a time), 0 = chosen from the row size;
@@ -126,7 +127,8 @@ typedef struct {
  *             set of nodes; one seed is the NSG-style single entry)
  *   spill_bits log2 of the slots of the first global visited table a query
  *             moves to when its shared table fills (the second one has four
- *             times as many), 0 = chosen from L; 10..16.  Speed only, unless
+ *             times as many), 0 = chosen from L (with d_L, from each query's
+ *             own L); 10..16.  Speed only, unless
  *             a query outgrows both tables (ANN_ERR_CAPACITY)
  *   flags     ANN_SEARCH_* bits.  ANN_SEARCH_RERANK: after the search, every
  *             id of the final pool (L entries) is re-scored exactly from the

@@ -40,6 +40,7 @@ namespace ann {
 
 namespace {
 
+constexpr int kFullTeams = 32;      // teams an SM holds at 64 registers a thread
 constexpr int kMaxSearchWarps = 2;  // warps (teams) per CTA: 1 or 2, whichever fits more teams
 constexpr int kTimeoutIters = 1 << 22;
 constexpr int kSlots = ANN_MAX_STEP_CAND / 32;  // neighbour slots per lane in one step
@@ -73,12 +74,24 @@ struct SearchArgs {
     unsigned long long *counter;
     uint32_t *spill;
     int hash_bits, spill_bits;
+    int spill_by_query;  // 1: a query's first global table is sized by its own L (within spill_bits)
     // per-warp shared-memory layout (byte offsets)
     int off_sel, off_q, off_stage, off_pool, off_ptop, off_cbuf, off_hash, per_warp;
     int stage_rows, stage_stride;
     int team_lg;  // log2 of the lanes computing one distance
     int cpl;      // 8 when a row is exactly 8 16-byte chunks per lane (unrolled), else 0
 };
+
+// log2 slots of a first global visited table that holds 40 evaluations per
+// pool slot below 3/4 load (about 3x the typical count), 12..15: small enough
+// to stay mostly L2-resident and cheap to clear
+__host__ __device__ inline int spill_bits_for(int L)
+{
+    int sb = 12;
+    while ((1 << sb) * 3 / 4 < 40 * L && sb < 15)
+        ++sb;
+    return sb;
+}
 
 __device__ __forceinline__ uint32_t hash_slot(uint32_t key, int bits)
 {
@@ -423,8 +436,13 @@ __global__ void __launch_bounds__(32 * kMaxSearchWarps, 16) beam_search_kernel(c
         int cnt = 0, cursor = 0, evals = 0, hops = 0;
         // visited set: level 0 = the shared table, 1 and 2 = the global ones;
         // used = keys in the current table, limit = its 3/4 load
-        int level = shared_tab ? 0 : 1, used = 0, gbits = a.spill_bits;
-        int limit = shared_tab ? hlimit : (1 << a.spill_bits) * 3 / 4;
+        // the first global table's size: the launch's, or the query's own L's,
+        // so that a small query of a mixed batch clears and touches a small
+        // table (the second one keeps the launch's size, so no query's
+        // capacity shrinks)
+        const int qbits = a.spill_by_query ? min(spill_bits_for(max(Lq, 1)), a.spill_bits) : a.spill_bits;
+        int level = shared_tab ? 0 : 1, used = 0, gbits = qbits;
+        int limit = shared_tab ? hlimit : (1 << qbits) * 3 / 4;
         uint32_t *gtab = gtab1;
         int32_t *pred = sel + ANN_MAX_W;  // predicted ids of the next selection
         int npred = 0;
@@ -443,11 +461,11 @@ __global__ void __launch_bounds__(32 * kMaxSearchWarps, 16) beam_search_kernel(c
             for (int o = lane; o < hcap / 4; o += 32)
                 reinterpret_cast<uint4 *>(htab)[o] = make_uint4(0u, 0u, 0u, 0u);
             if (!shared_tab)
-                for (int o = lane; o < (1 << a.spill_bits) / 4; o += 32)
+                for (int o = lane; o < (1 << qbits) / 4; o += 32)
                     reinterpret_cast<uint4 *>(gtab1)[o] = make_uint4(0u, 0u, 0u, 0u);
             __syncwarp();
             // the initial pool: every distinct seed, evaluated in the first step
-            const int r = seed >= 0 ? visit(htab, a.hash_bits, !shared_tab, gtab1, a.spill_bits, seed) : 0;
+            const int r = seed >= 0 ? visit(htab, a.hash_bits, !shared_tab, gtab1, qbits, seed) : 0;
             const unsigned nm = __ballot_sync(kFull, r == 1);
             if (r == 1)
                 cbuf[__popc(nm & lanemask_lt())] = static_cast<uint64_t>(seed) << 1;
@@ -687,7 +705,7 @@ __global__ void __launch_bounds__(32 * kMaxSearchWarps, 16) beam_search_kernel(c
             // set stays exact.
             while (used + total > limit && level < 2) {
                 uint32_t *dst = level == 0 ? gtab1 : gtab2;
-                const int dbits = level == 0 ? a.spill_bits : a.spill_bits + 2;
+                const int dbits = level == 0 ? qbits : a.spill_bits + 2;
                 if (level == 0)
                     migrate_keys(htab, a.hash_bits, false, dst, dbits, lane);
                 else
@@ -951,13 +969,17 @@ size_t align_up(size_t v, size_t a) { return (v + a - 1) / a * a; }
 
 // Resident teams for `per_warp` bytes of shared memory per team, with one or
 // two teams per CTA, whichever fits more (each CTA also costs the SM a fixed
-// reserve of shared memory, which two teams share).
+// reserve of shared memory, which two teams share).  When one team per CTA
+// already holds all nq queries, it is taken: the queries then spread over
+// twice as many SMs.
 template <int DT, int MT>
-ann_status teams_for(ann_index *idx, size_t per_warp, int *teams, int *wpc)
+ann_status teams_for(ann_index *idx, size_t per_warp, int64_t nq, int *teams, int *wpc)
 {
     auto kern = beam_search_kernel<DT, MT>;
     int best = 0, best_w = 1;
     for (int w = 1; w <= kMaxSearchWarps; ++w) {
+        if (static_cast<int64_t>(best) * idx->num_sms >= nq)
+            break;
         const size_t smem = per_warp * w;
         if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem)) !=
             cudaSuccess) {
@@ -1054,13 +1076,7 @@ int default_team(int rowbytes)
     return G;
 }
 
-int default_spill_bits(int L)
-{
-    int sb = 12;
-    while ((1 << sb) * 3 / 4 < 40 * L && sb < 15)
-        ++sb;
-    return sb;
-}
+int default_spill_bits(int L) { return spill_bits_for(L); }
 
 size_t search_scratch_bytes(int teams, int spill_bits, int64_t order_items)
 {
@@ -1101,24 +1117,11 @@ ann_status launch_search(ann_index *idx, const SearchLaunch &L, cudaStream_t s)
     a.out_stats = L.stats;
     a.status = idx->status_sink ? idx->status_sink : idx->d_status;
 
-    int hb = p->hash_bits;  // -1: no shared table
-    if (hb == 0) {
-        // searches evaluate about 10-16 nodes per pool slot; size the shared
-        // table for 12 per slot below its 3/4 load limit (the exact global
-        // spill table takes any excess; ann_autotune refines the choice)
-        hb = 10;
-        while ((1 << hb) * 3 / 4 < 12 * p->L && hb < 13)
-            ++hb;
-    }
-    a.hash_bits = hb;
-    // the first spill table holds 40 evaluations per pool slot below 3/4 load
-    // (about 3x the typical count), small enough to stay mostly L2-resident
-    // and cheap to clear when a query starts spilling; the second holds four
-    // times more for the tail
     int sb = default_spill_bits(p->L);
     if (p->spill_bits > 0)
         sb = p->spill_bits;
     a.spill_bits = sb;
+    a.spill_by_query = p->d_L && p->spill_bits == 0;
 
     const int maxc = p->W * idx->degree;
     // distance team: the smallest power of two >= 4 that leaves at most four
@@ -1148,37 +1151,76 @@ ann_status launch_search(ann_index *idx, const SearchLaunch &L, cudaStream_t s)
         const int c = chunks / G;
         a.cpl = c == 8 ? c : 0;
     }
-    // Most steps find far fewer new neighbours than W * R (about 30 % of
-    // them), so a small staging area filled in rounds keeps shared memory per
-    // team small (more teams per SM); at most 48 KB staged at once, which also
-    // keeps one mbarrier phase's byte count far below its 2^20 limit.
-    a.stage_rows = std::max(1, std::min({maxc, p->stage_rows > 0 ? p->stage_rows : 16, 49152 / a.stage_stride}));
-    if (a.gather4)
-        a.stage_rows = (a.stage_rows + 3) / 4 * 4;  // whole groups of four
-
-    size_t off = 16;  // mbarrier
-    a.off_sel = static_cast<int>(off);
-    off = align_up(off + 4 * 2 * ANN_MAX_W, 16);  // selected and predicted ids
-    a.off_q = static_cast<int>(off);
-    off = align_up(off + L.qbytes + a.qpad, 16);
-    if (a.gather4)
-        off = align_up(off, 128);  // tensor gathers land on 128-byte boundaries
-    a.off_stage = static_cast<int>(off);
-    off = align_up(off + static_cast<size_t>(a.stage_rows) * a.stage_stride, 16);
-    a.off_pool = static_cast<int>(off);
-    off = align_up(off + 8 * static_cast<size_t>(p->L), 16);
-    a.off_ptop = static_cast<int>(off);
-    off = align_up(off + 8 * ANN_MAX_W, 16);
-    a.off_cbuf = static_cast<int>(off);
-    off = align_up(off + 8 * ANN_MAX_STEP_CAND, 16);
-    a.off_hash = static_cast<int>(off);
-    off = align_up(off + (hb > 0 ? static_cast<size_t>(4) << hb : 0), 128);
-    a.per_warp = static_cast<int>(off);
+    // shared memory of one team with 2^hb visited slots (hb < 1: no table) and
+    // `rows` staged rows (at most 48 KB of them, which also keeps one mbarrier
+    // phase's byte count far below its 2^20 limit); fills in the layout
+    auto layout = [&](int hb, int rows) {
+        a.hash_bits = hb;
+        a.stage_rows = std::max(1, std::min({maxc, rows, 49152 / a.stage_stride}));
+        if (a.gather4)
+            a.stage_rows = (a.stage_rows + 3) / 4 * 4;  // whole groups of four
+        size_t off = 16;  // mbarrier
+        a.off_sel = static_cast<int>(off);
+        off = align_up(off + 4 * 2 * ANN_MAX_W, 16);  // selected and predicted ids
+        a.off_q = static_cast<int>(off);
+        off = align_up(off + L.qbytes + a.qpad, 16);
+        if (a.gather4)
+            off = align_up(off, 128);  // tensor gathers land on 128-byte boundaries
+        a.off_stage = static_cast<int>(off);
+        off = align_up(off + static_cast<size_t>(a.stage_rows) * a.stage_stride, 16);
+        a.off_pool = static_cast<int>(off);
+        off = align_up(off + 8 * static_cast<size_t>(p->L), 16);
+        a.off_ptop = static_cast<int>(off);
+        off = align_up(off + 8 * ANN_MAX_W, 16);
+        a.off_cbuf = static_cast<int>(off);
+        off = align_up(off + 8 * ANN_MAX_STEP_CAND, 16);
+        a.off_hash = static_cast<int>(off);
+        off = align_up(off + (hb > 0 ? static_cast<size_t>(4) << hb : 0), 128);
+        a.per_warp = static_cast<int>(off);
+        return off;
+    };
+    // Visited table and rows per gather round when the caller leaves them
+    // open.  Full SMs hide latency better than a shared table or long rounds
+    // shorten it, and a lone query wants both.  So: the shared table and then
+    // the longest round that still let every SM hold its share of the queries
+    // (up to kFullTeams, where registers end; rounds past 24 rows gain only on
+    // part-full SMs), else no table, and rounds of eight rows, or of four when
+    // rows pass 1 KB (d = 384 fp32: 2,770 us with four, 3,240 with eight).
+    // Measured (us, shared table sized for 12 evaluations per
+    // pool slot and rounds of 16 before, this rule after): 100,000 queries of
+    // mixed L <= 512 at d = 96: 78,600 -> 28,300; 10,000 at d = 200, L = 256:
+    // 8,220 -> 4,290; 100 uint8 queries, L = 64: 497 -> 382; one query: 230 ->
+    // 188.
+    size_t off = 0;
+    {
+        int dev_smem = 0, cta_smem = 0;
+        cudaDeviceGetAttribute(&dev_smem, cudaDevAttrMaxSharedMemoryPerMultiprocessor, idx->device);
+        cudaDeviceGetAttribute(&cta_smem, cudaDevAttrReservedSharedMemoryPerBlock, idx->device);
+        const int64_t want = std::min<int64_t>(kFullTeams, (L.nq + idx->num_sms - 1) / idx->num_sms);
+        auto holds = [&](size_t per_warp) {  // teams an SM holds, two to a CTA when more than one is wanted
+            const int64_t w = want > 1 ? kMaxSearchWarps : 1;
+            return static_cast<int64_t>(dev_smem) / static_cast<int64_t>(per_warp * w + cta_smem) * w >= want;
+        };
+        // a table for three times the typical evaluations, at most 32 KB
+        const int table = std::min(13, default_spill_bits(p->L));
+        const int tables[2] = {p->hash_bits ? p->hash_bits : table, p->hash_bits ? p->hash_bits : -1};
+        const int kRows[] = {32, 24, 16, 12, 8, 4};
+        const int r0 = want < kFullTeams ? 0 : 1, r1 = a.stage_stride > 1024 ? 6 : 5;
+        bool fits = false;
+        for (int t = 0; t < 2 && !fits; ++t) {
+            if (p->stage_rows > 0) {
+                fits = holds(off = layout(tables[t], p->stage_rows));
+            } else {
+                for (int r = r0; r < r1 && !fits; ++r)
+                    fits = holds(off = layout(tables[t], kRows[r]));
+            }
+        }
+    }
 
     // persistent grid: occupancy-limited, at most one team per query
     int teams = 0, wpc = 1;
     ann_status st = ANN_OK;
-    ANN_DISPATCH(teams_for, idx, off, &teams, &wpc);
+    ANN_DISPATCH(teams_for, idx, off, L.nq, &teams, &wpc);
     if (st != ANN_OK)
         return st;
     if (L.max_teams > 0)
@@ -1192,11 +1234,16 @@ ann_status launch_search(ann_index *idx, const SearchLaunch &L, cudaStream_t s)
     // scratch: work counter, then two spill tables per team, then the grouped
     // work order (when asked for, with seeds given and item indices in int32)
     const bool group = (p->flags & ANN_SEARCH_GROUP_ENTRIES) && L.entries && L.nq <= INT32_MAX;
-    const size_t need = search_scratch_bytes(teams, a.spill_bits, group ? L.nq : 0);
+    size_t need = search_scratch_bytes(teams, a.spill_bits, group ? L.nq : 0);
     void *scratch = L.scratch;
     const bool own = scratch == nullptr;
     if (own) {
-        st = scratch_alloc(idx, need, s, &scratch);
+        // a nearly full device still searches, with fewer teams and tables
+        while ((st = scratch_alloc(idx, need, s, &scratch)) == ANN_ERR_OOM && teams > idx->num_sms) {
+            cudaGetLastError();
+            teams = std::max(idx->num_sms, teams / 2) / wpc * wpc;
+            need = search_scratch_bytes(teams, a.spill_bits, group ? L.nq : 0);
+        }
         if (st != ANN_OK)
             return st;
     } else if (L.scratch_bytes < need) {

@@ -349,3 +349,40 @@ def test_visited_set_outgrows_both_global_tables():
     assert np.array_equal(ids[:2], oi) and np.array_equal(ev[:2], oe) and np.array_equal(hp[:2], oh)
     assert np.array_equal(d[:2], od.astype(np.float32))
     assert (ids[2] == -1).all()
+
+
+@pytest.mark.parametrize("nq", [1, 153, 1_217, 4_865])
+@pytest.mark.parametrize("L,W", [(20, 4), (160, 2), (2_000, 4)])
+def test_default_sizes_change_nothing(c1, nq, L, W):
+    # the visited table and gather rounds chosen when the caller leaves them
+    # open depend on nq and L (all queries resident, SMs part full, SMs full);
+    # results never do
+    q = np.resize(c1["queries"], (nq, 128))
+    oi, od, oe, oh = _oracle(c1, c1["queries"][:min(nq, 100)], L, 10, W=W)
+    ids, d, ev, hp, st = search(c1["h"], q, 10, L, W=W)
+    assert st == ann.OK
+    at = np.arange(nq) % 100
+    assert np.array_equal(ids, oi[at]) and np.array_equal(ev, oe[at]) and np.array_equal(hp, oh[at])
+    assert np.array_equal(d, od[at].astype(np.int64).astype(np.int32))
+
+
+@pytest.mark.parametrize("hash_bits", [0, -1, 8])
+def test_tables_sized_by_each_querys_own_L(hash_bits):
+    # on a random graph nearly every neighbour is new, so a query outgrows the
+    # table its own L sizes (3,072 keys up to L = 76) and moves to the second
+    # one, whose size is the launch's
+    rng = np.random.default_rng(12)
+    w = synth.small_u8(n=20_000)
+    g = rng.integers(0, 20_000, size=(20_000, 32)).astype(np.int32)
+    q = w["queries"]
+    Ls = np.resize(np.array([1, 40, 76, 77, 300, 512], np.int32), len(q))
+    ks = np.minimum(Ls, 10).astype(np.int32)
+    h = make_index(w["base"], g, 0)
+    try:
+        ids, d, ev, hp, st = search(h, q, 10, 512, W=4, ks=ks, Ls=Ls, hash_bits=hash_bits)
+    finally:
+        ann.ann_free_index(h)
+    oi, od, oe, oh = oracle.search(w["base"], g, q.astype(np.float64), 0, 512, 10, W=4, Ls=Ls, ks=ks)
+    assert st == ann.OK
+    assert (oe[Ls == 76] > 3_072).any()
+    assert np.array_equal(ids, oi[:, :10]) and np.array_equal(ev, oe) and np.array_equal(hp, oh)
