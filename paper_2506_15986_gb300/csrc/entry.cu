@@ -48,9 +48,7 @@ struct TowerArgs {
     int64_t nq;
     float *qhat;                // [nq][64] optional
     __nv_bfloat16 *qhat_bf;     // [nq][64] optional
-    float *z1;                  // [nq][256] optional (training)
-    __nv_bfloat16 *a1;          // [nq][256] optional (training)
-    float *nrm;                 // [nq] optional (training)
+    TowerTrain train;           // training outputs (train.zmask null: none)
     int *status;
 };
 
@@ -103,23 +101,26 @@ __global__ void __launch_bounds__(128) tower_forward_kernel(const TowerArgs t)
 #pragma unroll
             for (int j = 0; j < 32; ++j)
                 v[j] += t.b1[c0 + j];
-            if (t.z1 && live) {
-                float4 *dst = reinterpret_cast<float4 *>(t.z1 + row * 256 + c0);
-#pragma unroll
-                for (int j = 0; j < 8; ++j)
-                    dst[j] = make_float4(v[4 * j], v[4 * j + 1], v[4 * j + 2], v[4 * j + 3]);
-            }
+            uint32_t active = 0;
 #pragma unroll
             for (int j = 0; j < 32; j += 8) {
                 float a[8];
 #pragma unroll
-                for (int u = 0; u < 8; ++u)
+                for (int u = 0; u < 8; ++u) {
                     a[u] = fmaxf(v[j + u], 0.f);
+                    active |= (v[j + u] > 0.f ? 1u : 0u) << (j + u);
+                }
                 const uint4 pk = pack8_bf16(a);
                 *reinterpret_cast<uint4 *>(sH + canon_off(m, c0 + j, 32)) = pk;
-                if (t.a1 && live)
-                    *reinterpret_cast<uint4 *>(t.a1 + row * 256 + c0 + j) = pk;
+                if (t.train.zmask && live) {
+                    const __nv_bfloat16 *h = reinterpret_cast<const __nv_bfloat16 *>(&pk);
+#pragma unroll
+                    for (int u = 0; u < 8; ++u)
+                        t.train.a1T[(c0 + j + u) * t.train.ld + row] = h[u];
+                }
             }
+            if (t.train.zmask && live)
+                t.train.zmask[(c0 / 32) * t.train.ld + row] = active;
         }
         // GEMM 2: [128 x 256] x [256 x 64]; W2t staged whole (64 rows x 256 k)
         const Operand W2{t.W2t, OP_BF16, 256, 1, 64, 256, nullptr};
@@ -156,11 +157,15 @@ __global__ void __launch_bounds__(128) tower_forward_kernel(const TowerArgs t)
         const float nrm = sqrtf(ss);
         const float inv = nrm > 0.f ? 1.0f / nrm : 0.f;
         if (live) {
-            if (t.nrm)
-                t.nrm[row] = nrm;
 #pragma unroll
             for (int j = 0; j < 64; ++j)
                 z[j] *= inv;
+            if (t.train.zmask) {
+                t.train.nrm[row] = nrm;
+#pragma unroll
+                for (int j = 0; j < 64; ++j)
+                    t.train.qT[j * t.train.ld + row] = __float2bfloat16_rn(z[j]);
+            }
             if (t.qhat) {
                 float4 *dst = reinterpret_cast<float4 *>(t.qhat + row * 64);
 #pragma unroll
@@ -585,30 +590,72 @@ __global__ void pack_canonical_kernel(const __nv_bfloat16 *src, int64_t rows, in
     }
 }
 
-// BF16 transposed weight copies for K-major B operands, and normalised hub
-// embeddings (FP32 and BF16)
-__global__ void prepare_model_kernel(const float *W1, const float *W2, const float *E, int in_dim, int H,
-                                     __nv_bfloat16 *W1t, __nv_bfloat16 *W2t, float *En, __nv_bfloat16 *Eb)
+// BF16 weight copies for K-major B operands, and normalised hub embeddings
+// (FP32 and BF16; transposed BF16 and the norms too for training models).
+// Blocks take 32 x 32 tiles of W1, then of W2, then 64 hubs each; everything
+// goes through shared memory so that both sides move in whole lines.  (One
+// thread per weight read down a column and one thread per hub walked its row:
+// 51 us at 128 inputs and 1,024 hubs, 7.5 us here; bounded by latency.)
+__global__ void __launch_bounds__(256)
+    prepare_model_kernel(const float *W1, const float *W2, const float *E, int in_dim, int H, __nv_bfloat16 *W1t,
+                         __nv_bfloat16 *W2t, float *En, __nv_bfloat16 *Eb, float *Enrm, __nv_bfloat16 *W2b,
+                         __nv_bfloat16 *EnT, int64_t ldE)
 {
-    const int64_t tid = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x;
-    const int64_t n1 = static_cast<int64_t>(in_dim) * 256, n2 = 256 * 64;
-    if (tid < n1) {
-        const int n = static_cast<int>(tid / in_dim), k = static_cast<int>(tid % in_dim);
-        W1t[tid] = __float2bfloat16_rn(W1[static_cast<int64_t>(k) * 256 + n]);
-    } else if (tid < n1 + n2) {
-        const int64_t i = tid - n1;
-        const int n = static_cast<int>(i / 256), k = static_cast<int>(i % 256);
-        W2t[i] = __float2bfloat16_rn(W2[k * 64 + n]);
-    } else if (tid < n1 + n2 + H) {
-        const int64_t h = tid - n1 - n2;
+    __shared__ float t[64][65];
+    __shared__ float scale[64];
+    const int tid = threadIdx.x;
+    const int k1 = (in_dim + 31) / 32, n1 = k1 * 8, n2 = 8 * 2;
+    int b = blockIdx.x;
+    if (b < n1 + n2) {
+        // dst[n][k] = src[k][n], a tile of 32 k x 32 n
+        const bool first = b < n1;
+        const float *src = first ? W1 : W2;
+        const int K = first ? in_dim : 256, N = first ? 256 : 64;
+        if (!first)
+            b -= n1;
+        const int k0 = b % ((K + 31) / 32) * 32, c0 = b / ((K + 31) / 32) * 32;
+        for (int i = tid; i < 1024; i += 256) {
+            const int k = k0 + i / 32, n = c0 + i % 32;
+            const float v = k < K ? src[static_cast<int64_t>(k) * N + n] : 0.f;
+            t[i / 32][i % 32] = v;
+            if (!first && W2b && k < K)
+                W2b[k * N + n] = __float2bfloat16_rn(v);
+        }
+        __syncthreads();
+        __nv_bfloat16 *dst = first ? W1t : W2t;
+        for (int i = tid; i < 1024; i += 256) {
+            const int n = c0 + i / 32, k = k0 + i % 32;
+            if (k < K)
+                dst[static_cast<int64_t>(n) * K + k] = __float2bfloat16_rn(t[i % 32][i / 32]);
+        }
+        return;
+    }
+    const int64_t h0 = static_cast<int64_t>(b - n1 - n2) * 64;
+    for (int i = tid; i < 64 * 64; i += 256)
+        t[i / 64][i % 64] = h0 + i / 64 < H ? E[h0 * 64 + i] : 0.f;
+    __syncthreads();
+    if (tid < 64) {
         float ss = 0.f;
         for (int j = 0; j < 64; ++j)
-            ss = fmaf(E[h * 64 + j], E[h * 64 + j], ss);
-        const float inv = ss > 0.f ? rsqrtf(ss) : 0.f;
-        for (int j = 0; j < 64; ++j) {
-            const float v = E[h * 64 + j] * inv;
-            En[h * 64 + j] = v;
-            Eb[h * 64 + j] = __float2bfloat16_rn(v);
+            ss = fmaf(t[tid][j], t[tid][j], ss);
+        scale[tid] = ss > 0.f ? rsqrtf(ss) : 0.f;
+        if (Enrm && h0 + tid < H)
+            Enrm[h0 + tid] = sqrtf(ss);
+    }
+    __syncthreads();
+    for (int i = tid; i < 64 * 64; i += 256) {
+        const int r = i / 64;
+        if (h0 + r < H) {
+            const float v = t[r][i % 64] * scale[r];
+            En[h0 * 64 + i] = v;
+            Eb[h0 * 64 + i] = __float2bfloat16_rn(v);
+        }
+    }
+    if (EnT) {
+        for (int i = tid; i < 64 * 64; i += 256) {
+            const int r = i % 64, c = i / 64;
+            if (h0 + r < H)
+                EnT[c * ldE + h0 + r] = __float2bfloat16_rn(t[r][c] * scale[r]);
         }
     }
 }
@@ -962,9 +1009,9 @@ size_t packed_model_bytes(int in_dim, int H)
 
 ann_status prepare_model(ann_entry_model *m, cudaStream_t s)
 {
-    const int64_t total = static_cast<int64_t>(m->in_dim) * 256 + 256 * 64 + m->H;
-    prepare_model_kernel<<<static_cast<unsigned>((total + 255) / 256), 256, 0, s>>>(
-        m->W1, m->W2, m->E, m->in_dim, m->H, m->W1t, m->W2t, m->En, m->Eb);
+    const int blocks = (m->in_dim + 31) / 32 * 8 + 16 + (m->H + 63) / 64;
+    prepare_model_kernel<<<blocks, 256, 0, s>>>(m->W1, m->W2, m->E, m->in_dim, m->H, m->W1t, m->W2t, m->En, m->Eb,
+                                                m->Enrm, m->W2b, m->EnT, m->ldE);
     cudaError_t e = cudaGetLastError();
     if (e == cudaSuccess && m->packed) {
         // W1^T in 64-wide k chunks of 256 rows, W2^T (64 rows x 256), the
@@ -981,8 +1028,7 @@ ann_status prepare_model(ann_entry_model *m, cudaStream_t s)
 }
 
 ann_status launch_tower(const ann_entry_model *m, const Operand &X, int64_t nq, float *qhat,
-                        __nv_bfloat16 *qhat_bf, float *z1, __nv_bfloat16 *a1, float *nrm, int *status,
-                        cudaStream_t s)
+                        __nv_bfloat16 *qhat_bf, const TowerTrain *train, int *status, cudaStream_t s)
 {
     if (nq == 0)
         return ANN_OK;
@@ -996,9 +1042,8 @@ ann_status launch_tower(const ann_entry_model *m, const Operand &X, int64_t nq, 
     t.nq = nq;
     t.qhat = qhat;
     t.qhat_bf = qhat_bf;
-    t.z1 = z1;
-    t.a1 = a1;
-    t.nrm = nrm;
+    if (train)
+        t.train = *train;
     t.status = status;
     cudaError_t e = cudaFuncSetAttribute(tower_forward_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          kTowerSmem);
@@ -1433,7 +1478,7 @@ ann_status ann_select_entries(ann_index *idx, const void *d_queries, int64_t nq,
     __nv_bfloat16 *qbf = reinterpret_cast<__nv_bfloat16 *>(static_cast<uint8_t *>(scr) + qf);
     int32_t *hid = reinterpret_cast<int32_t *>(static_cast<uint8_t *>(scr) + qf + qb);
     float *hsc = reinterpret_cast<float *>(static_cast<uint8_t *>(scr) + qf + qb + hb);
-    st = launch_tower(m, X, nq, qhat, qbf, nullptr, nullptr, nullptr, idx->d_status, s);
+    st = launch_tower(m, X, nq, qhat, qbf, nullptr, idx->d_status, s);
     if (st == ANN_OK && one_launch) {
         const int bm_words = (m->H + 127) / 128 * 4;
         const size_t per_warp = 256 + 128 + 4 * static_cast<size_t>(bm_words);

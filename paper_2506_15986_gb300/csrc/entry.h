@@ -19,6 +19,11 @@ struct ann_entry_model {
     __nv_bfloat16 *W1t = nullptr;            // [256][in_dim]
     __nv_bfloat16 *W2t = nullptr;            // [64][256]
     __nv_bfloat16 *Eb = nullptr;             // normalised, BF16 [H][64]
+    // training models only (a trainer owns them):
+    float *Enrm = nullptr;                   // |e_v| [H]
+    __nv_bfloat16 *W2b = nullptr;            // W2 as it is, BF16 [256][64]
+    __nv_bfloat16 *EnT = nullptr;            // normalised, BF16, transposed [64][ldE]
+    int64_t ldE = 0;
     // index models only: the operands of the exhaustive entry kernel as the
     // 32 KB canonical shared-memory images its bulk copies load (W1 in
     // 64-wide k chunks, then W2, then the hubs in tiles of 256 rows)
@@ -44,9 +49,18 @@ size_t packed_model_bytes(int in_dim, int H);
 ann_status prepare_model(ann_entry_model *m, cudaStream_t s);
 ann_status build_hub_index(ann_index *idx, ann_entry_model *m, const int32_t *hub_graph, int32_t hub_entry,
                            cudaStream_t s);
+// What the backward pass needs of a forward pass, laid out as it reads it
+// (batch along the rows, so that a warp's lanes, one query each, write
+// consecutive elements).
+struct TowerTrain {
+    uint32_t *zmask;      // [8][ld]: bit j of word c: hidden unit 32 c + j is active (Z1 > 0)
+    __nv_bfloat16 *a1T;   // [256][ld] ReLU(Z1)
+    __nv_bfloat16 *qT;    // [64][ld] q_hat
+    float *nrm;           // [nq] |Z2|
+    int64_t ld;
+};
 ann_status launch_tower(const ann_entry_model *m, const Operand &X, int64_t nq, float *qhat,
-                        __nv_bfloat16 *qhat_bf, float *z1, __nv_bfloat16 *a1, float *nrm, int *status,
-                        cudaStream_t s);
+                        __nv_bfloat16 *qhat_bf, const TowerTrain *train, int *status, cudaStream_t s);
 // Exhaustive entry selection in one kernel: the query tower, every hub's
 // score and the topm (1..8) best hubs' nodes per query (nq x topm, best
 // first); qhat (optional) receives the fp32 query embeddings.

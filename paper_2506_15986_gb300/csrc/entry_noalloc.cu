@@ -99,7 +99,7 @@ ann_status ann_select_entry_noalloc(ann_index *idx, const void *d_queries, int64
         cudaStream_t s = static_cast<cudaStream_t>(stream);
         const ann_entry_model *m = idx->model;
         const Operand X{d_queries, idx->dtype == ANN_U8 ? OP_U8 : OP_F32, idx->dim, 1, nq, idx->dim, nullptr};
-        st = launch_tower(m, X, nq, d_qhat, qbf, nullptr, nullptr, nullptr, idx->d_status, s);
+        st = launch_tower(m, X, nq, d_qhat, qbf, nullptr, idx->d_status, s);
         if (st == ANN_OK) {
             const Operand Q{qbf, OP_BF16, 64, 1, nq, 64, nullptr};
             st = launch_hub_argmax(m, Q, nq, d_entry, hub, score, idx->d_status, s);

@@ -12,9 +12,11 @@
 //             through the normalisations, dZ2 -> dW2 = A1^T dZ2, db2,
 //             dZ1 = (dZ2 W2^T) * [Z1 > 0] -> dW1 = X^T dZ1, db1 (tcgen05 GEMMs)
 //   update    Adam with bias correction on W1, b1, W2, b2, E     (adam_kernel)
-// Every GEMM runs BF16 x BF16 -> FP32 on the tensor cores; operands that a
-// GEMM reads K-major from a row-major matrix's columns are transposed into
-// BF16 scratch first.
+// Every GEMM runs BF16 x BF16 -> FP32 on the tensor cores.  Whatever produces
+// an operand writes it as BF16 in the layouts its GEMMs read (row-major, and
+// transposed where a GEMM reduces over the batch), so that a step moves each
+// matrix about once: the tower leaves A1^T, q_hat^T and the ReLU mask, the
+// loss kernel dS, the dZ1 GEMM's epilogue dZ1^T and db1's partial sums.
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 #include <math.h>
@@ -38,46 +40,75 @@ constexpr int kMaxTrainHubs = 65536;
 
 // ---- generic tensor-core GEMM ------------------------------------------------
 
-enum Epi { EPI_STORE = 0, EPI_RELU_MASK = 1 };
+enum Epi { EPI_STORE = 0, EPI_HIDDEN = 1 };
+
+// A BF16 matrix read along its rows (K): element (r, k) = p[r * ld + k], zero
+// outside rows x K; ld a multiple of 8 and p 16-byte aligned.
+struct Mat {
+    const __nv_bfloat16 *p;
+    int64_t ld, rows;
+};
 
 struct GemmArgs {
-    Operand A, B;      // A: M x K, B: N x K (both read K-major)
+    Mat A, B;               // A: M x K, B: N x K
     int64_t M, N, K;
     float alpha;            // out = alpha * scale[0] * acc (scale may be null)
     const float *scale;
-    int epi;
-    const float *aux;       // EPI_RELU_MASK: out *= (aux[r*ldo + c] > 0)
-    float *out;
+    float *out;             // EPI_STORE
     int64_t ldo;
+    // EPI_HIDDEN: x = alpha * acc where the row's mask bit is set, else 0;
+    // outT[c * ldt + r] = bf16(x), part[warp][c] = sum of the warp's 32 rows
+    const uint32_t *mask;   // [N / 32][ldt]
+    __nv_bfloat16 *outT;
+    int64_t ldt;
+    float *part;            // [M / 32, rounded up to 4][256]
     int *status;
     int64_t ksplit;         // > 0: blockIdx.z takes K range [z*ksplit, (z+1)*ksplit) and adds into out
+    int stages;             // ring of operand stages, 1 to kGemmStages
 };
 
-// the operand seen from column k0 on (k0 a multiple of 64: 16-byte alignment kept)
-__device__ __forceinline__ Operand op_from_k(const Operand &o, int64_t k0)
+constexpr int kGemmStages = 4;
+
+// Rows [r0, r0 + ROWS) x k [k0, k0 + 64) of m into a canonical K-major tile by
+// 16-byte asynchronous copies (chunk c holds row (c / 64) * 8 + c % 8, k-chunk
+// (c / 8) % 8); what lies past the matrix is filled with zeros.
+template <int ROWS>
+__device__ __forceinline__ void load_tile(uint8_t *tile, const Mat &m, int64_t r0, int64_t k0, int64_t K)
 {
-    Operand r = o;
-    const int es = o.type == OP_F32 ? 4 : (o.type == OP_BF16 ? 2 : 1);
-    r.p = static_cast<const uint8_t *>(o.p) + k0 * o.sk * es;
-    r.cols = o.cols - k0;
-    return r;
+    const uint32_t to = smem_addr(tile);
+#pragma unroll
+    for (int i = 0; i < ROWS * 8 / 128; ++i) {
+        const int c = i * 128 + static_cast<int>(threadIdx.x);
+        const int64_t r = r0 + (c >> 6) * 8 + (c & 7), k = k0 + ((c >> 3) & 7) * 8;
+        const int64_t left = r < m.rows ? K - k : 0;
+        const int bytes = left >= 8 ? 16 : left > 0 ? static_cast<int>(left) * 2 : 0;
+        const __nv_bfloat16 *src = bytes ? m.p + r * m.ld + k : m.p;
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(to + c * 16), "l"(src), "r"(bytes)
+                     : "memory");
+    }
 }
 
+// One 128 x BN tile of out = A B^T (or its share of K).  The operands stream
+// through a ring of 64-wide K stages filled by asynchronous copies up to
+// three stages ahead, thread 0 issues each stage's four MMAs as it lands, and
+// the epilogue goes through shared memory so that whole lines are written.
+// Staging each K chunk, waiting for its MMAs and storing a row per lane took
+// 339 us for the six GEMMs of a step (8,192 rows, 1,024 hubs); 108 us here,
+// bounded by load latency and, for the logits, by the 34 MB they write.
 template <int BN>
-__global__ void __launch_bounds__(128) gemm_kernel(const GemmArgs g)
+__global__ void __launch_bounds__(128) gemm_kernel(const GemmArgs g, const int epi)
 {
     extern __shared__ __align__(1024) uint8_t smem[];
-    uint8_t *sA = smem;
-    uint8_t *sB = smem + 16384;
-    uint64_t *bar = reinterpret_cast<uint64_t *>(smem + 16384 + BN * 128);
-    uint32_t *slot = reinterpret_cast<uint32_t *>(smem + 16384 + BN * 128 + 8);
+    constexpr int kStage = 16384 + BN * 128;
+    uint64_t *bar = reinterpret_cast<uint64_t *>(smem + g.stages * kStage);
+    uint32_t *slot = reinterpret_cast<uint32_t *>(bar + kGemmStages);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int64_t r0 = static_cast<int64_t>(blockIdx.x) * 128;
     const int64_t c0 = static_cast<int64_t>(blockIdx.y) * BN;
-    const int64_t row = r0 + warp * 32 + lane;
     constexpr uint32_t NCOL = BN < 32 ? 32 : BN;
     if (threadIdx.x == 0) {
-        mbar_init(bar, 1);
+        for (int i = 0; i < kGemmStages; ++i)
+            mbar_init(bar + i, 1);
         fence_mbar_init();
     }
     if (warp == 0)
@@ -86,32 +117,94 @@ __global__ void __launch_bounds__(128) gemm_kernel(const GemmArgs g)
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = *slot;
-    uint32_t phase = 0;
     const int64_t kb = g.ksplit > 0 ? static_cast<int64_t>(blockIdx.z) * g.ksplit : 0;
-    const int64_t kl = g.ksplit > 0 ? min(g.ksplit, g.K - kb) : g.K;
-    const bool ok = tc_gemm_tile<BN>(kb ? op_from_k(g.A, kb) : g.A, r0, kb ? op_from_k(g.B, kb) : g.B, c0, kl, sA,
-                                     sB, bar, phase, tmem);
+    const int64_t ke = g.ksplit > 0 ? min(kb + g.ksplit, g.K) : g.K;
+    const int nc = static_cast<int>((ke - kb + 63) / 64), S = g.stages;
+    auto load = [&](int c) {
+        if (c < nc) {
+            uint8_t *st = smem + (c % S) * kStage;
+            load_tile<128>(st, g.A, r0, kb + static_cast<int64_t>(c) * 64, ke);
+            load_tile<BN>(st + 16384, g.B, c0, kb + static_cast<int64_t>(c) * 64, ke);
+        }
+        asm volatile("cp.async.commit_group;" ::: "memory");
+    };
+    constexpr uint32_t IDESC = idesc_bf16_f32(128, BN);
+    bool ok = true;
+    for (int c = 0; c < kGemmStages - 1; ++c)
+        if (c < S)
+            load(c);
+        else
+            asm volatile("cp.async.commit_group;" ::: "memory");
+    // (S < kGemmStages only when all nc chunks fit the ring: nothing is refilled)
+    for (int c = 0; c < nc; ++c) {
+        asm volatile("cp.async.wait_group %0;" ::"n"(kGemmStages - 2) : "memory");
+        fence_proxy_async_smem();
+        tc_fence_before();
+        __syncthreads();
+        if (threadIdx.x == 0) {
+            tc_fence_after();
+            const uint8_t *sA = smem + (c % S) * kStage, *sB = sA + 16384;
+#pragma unroll
+            for (int kk = 0; kk < 4; ++kk)
+                tc_mma(tmem, smem_desc(sA + kk * 256, 128, 1024), smem_desc(sB + kk * 256, 128, 1024), IDESC,
+                       (c > 0 || kk > 0) ? 1u : 0u);
+            tc_commit(bar + c % S);
+        }
+        const int next = c + kGemmStages - 1;
+        if (next < nc && c > 0) {
+            // the stage to refill was read by the previous chunk's MMAs
+            uint32_t phase = static_cast<uint32_t>((c - 1) / S) & 1u;
+            if (!(ok = tc_wait(bar + (c - 1) % S, phase)))
+                break;
+        }
+        load(next);
+    }
+    asm volatile("cp.async.wait_group 0;" ::: "memory");
+    if (ok) {
+        uint32_t phase = static_cast<uint32_t>((nc - 1) / S) & 1u;
+        ok = tc_wait(bar + (nc - 1) % S, phase);
+    }
     if (ok) {
         const float a = g.alpha * (g.scale ? g.scale[0] : 1.f);
         const uint32_t my_lane = tmem + (static_cast<uint32_t>(warp * 32) << 16);
-        for (int cc = 0; cc < BN; cc += 32) {
+        const int64_t row = r0 + warp * 32 + lane;
+        float *tw = reinterpret_cast<float *>(smem) + warp * (32 * 33);  // the operands are read
+        for (int cc = 0; cc < BN && c0 + cc < g.N; cc += 32) {
             float v[32];
             tmem_ld32(my_lane + cc, v);
-            if (row < g.M) {
+            if (epi == EPI_HIDDEN) {
+                const uint32_t mask = row < g.M ? g.mask[((c0 + cc) >> 5) * g.ldt + row] : 0u;
 #pragma unroll
                 for (int j = 0; j < 32; ++j) {
-                    const int64_t col = c0 + cc + j;
-                    if (col < g.N) {
-                        float x = a * v[j];
-                        if (g.epi == EPI_RELU_MASK && !(g.aux[row * g.ldo + col] > 0.f))
-                            x = 0.f;
+                    const float x = (mask >> j) & 1u ? a * v[j] : 0.f;
+                    tw[lane * 33 + j] = x;
+                    if (row < g.M)
+                        g.outT[(c0 + cc + j) * g.ldt + row] = __float2bfloat16_rn(x);
+                }
+                __syncwarp();
+                float sum = 0.f;
+#pragma unroll
+                for (int r = 0; r < 32; ++r)
+                    sum += tw[r * 33 + lane];
+                g.part[(static_cast<int64_t>(blockIdx.x) * 4 + warp) * 256 + c0 + cc + lane] = sum;
+            } else {
+#pragma unroll
+                for (int j = 0; j < 32; ++j)
+                    tw[lane * 33 + j] = a * v[j];
+                __syncwarp();
+                const int64_t col = c0 + cc + lane;
+                const int rows = static_cast<int>(min(static_cast<int64_t>(32), g.M - r0 - warp * 32));
+                if (col < g.N) {
+                    float *o = g.out + (r0 + warp * 32) * g.ldo + col;
+                    for (int r = 0; r < rows; ++r) {
                         if (g.ksplit > 0)
-                            atomicAdd(g.out + row * g.ldo + col, x);  // a partial sum over its K range
+                            atomicAdd(o + r * g.ldo, tw[r * 33 + lane]);  // a partial sum over its K range
                         else
-                            g.out[row * g.ldo + col] = x;
+                            o[r * g.ldo] = tw[r * 33 + lane];
                     }
                 }
             }
+            __syncwarp();
         }
     } else if (threadIdx.x == 0) {
         atomicOr(g.status, kStatusTimeoutBit);
@@ -124,80 +217,123 @@ __global__ void __launch_bounds__(128) gemm_kernel(const GemmArgs g)
     }
 }
 
+// Queues one GEMM.  With EPI_STORE and few output tiles over a long reduction
+// K is split over CTAs that add into `out`, which the caller has zeroed.
 template <int BN>
-ann_status gemm(const GemmArgs &g, cudaStream_t s)
+ann_status gemm(const GemmArgs &g, cudaStream_t s, int epi = EPI_STORE)
 {
-    // at least 100 KB: at most two CTAs, so at most 2 x 256 TMEM columns, per SM
-    const int smem = std::max(16384 + BN * 128 + 64, 100 * 1024);
-    cudaError_t e = cudaFuncSetAttribute(gemm_kernel<BN>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-    if (e != cudaSuccess)
-        return cuda_status(e);
     dim3 grid(static_cast<unsigned>((g.M + 127) / 128), static_cast<unsigned>((g.N + BN - 1) / BN));
-    // few output tiles over a long reduction: split K over CTAs (linear
-    // epilogue only), at least 512 columns each, up to about two CTAs per SM
+    // at least 512 columns of K each, up to about two CTAs per SM
     GemmArgs h = g;
     h.ksplit = 0;
     const int64_t tiles = static_cast<int64_t>(grid.x) * grid.y;
-    if (g.epi == EPI_STORE && tiles < 128 && g.K >= 1024) {
+    if (epi == EPI_STORE && tiles < 128 && g.K >= 1024) {
         const int64_t want = std::min<int64_t>(g.K / 512, std::max<int64_t>(1, 256 / tiles));
         if (want > 1) {
             h.ksplit = ((g.K + want - 1) / want + 63) / 64 * 64;
             grid.z = static_cast<unsigned>((g.K + h.ksplit - 1) / h.ksplit);
-            // the partial sums add into a zeroed M x N block (rows ldo apart)
-            e = cudaMemset2DAsync(g.out, static_cast<size_t>(g.ldo) * 4, 0, static_cast<size_t>(g.N) * 4,
-                                  static_cast<size_t>(g.M), s);
-            if (e != cudaSuccess)
-                return cuda_status(e);
         }
     }
-    gemm_kernel<BN><<<grid, 128, smem, s>>>(h);
+    const int64_t chunks = ((h.ksplit ? h.ksplit : g.K) + 63) / 64;
+    h.stages = static_cast<int>(std::min<int64_t>(kGemmStages, chunks));
+    // at most 512 / BN CTAs fit an SM's 228 KB, so that they never ask for
+    // more than its 512 TMEM columns
+    const int smem = std::max(h.stages * (16384 + BN * 128) + 64, 228 * 1024 / (512 / BN + 1) + 1);
+    cudaError_t e = cudaFuncSetAttribute(gemm_kernel<BN>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    if (e != cudaSuccess)
+        return cuda_status(e);
+    gemm_kernel<BN><<<grid, 128, smem, s>>>(h, epi);
     return cuda_status(cudaGetLastError());
 }
 
 // ---- elementwise / row kernels --------------------------------------------
 
-// dst[c][r] = bf16(src(r, c)) for r < rows, c < cols; src row r read through rowmap
-__global__ void transpose_bf16(const Operand src, int64_t rows, int64_t cols, __nv_bfloat16 *dst)
+// The two transposes over the batch that no producer can write itself, in
+// 64 x 64 tiles: blockIdx.z = 0: dst[c][r] = dS(r, c), BF16 both; 1: xT[c][r] =
+// bf16(X(row r of the batch, c)).
+struct TransposeArgs {
+    const __nv_bfloat16 *dS;
+    int64_t ldS;
+    int H;
+    __nv_bfloat16 *dST;
+    const float *X;
+    const int32_t *rowmap;
+    int D;
+    __nv_bfloat16 *xT;
+    int64_t B, ldB;
+};
+
+__global__ void __launch_bounds__(256) transpose_kernel(const TransposeArgs a)
 {
-    __shared__ float tile[32][33];
-    const int64_t r0 = static_cast<int64_t>(blockIdx.y) * 32, c0 = static_cast<int64_t>(blockIdx.x) * 32;
-    for (int i = threadIdx.y; i < 32; i += blockDim.y) {
-        const int64_t r = r0 + i, c = c0 + threadIdx.x;
-        float v = 0.f;
-        if (r < rows && c < cols)
-            v = op_at(src, src.rowmap ? src.rowmap[r] : r, c);
-        tile[i][threadIdx.x] = v;
+    __shared__ __nv_bfloat16 tile[64][66];
+    const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
+    const int64_t c0 = static_cast<int64_t>(blockIdx.x) * 64, r0 = static_cast<int64_t>(blockIdx.y) * 64;
+    const bool logits = blockIdx.z == 0;
+    const int cols = logits ? a.H : a.D;
+    if (c0 >= cols)
+        return;
+    for (int i = ty; i < 64; i += 8) {
+        const int64_t r = r0 + i;
+        __nv_bfloat162 v;
+        v.x = v.y = __float2bfloat16_rn(0.f);
+        const int64_t c = c0 + 2 * tx;
+        if (r < a.B) {
+            if (logits) {
+                // pairs are 4-byte aligned (ldS even); past H the row's padding is read, never used
+                if (c < a.ldS)
+                    v = *reinterpret_cast<const __nv_bfloat162 *>(a.dS + r * a.ldS + c);
+            } else {
+                const float *x = a.X + static_cast<int64_t>(a.rowmap ? a.rowmap[r] : r) * a.D;
+                if (c < cols)
+                    v.x = __float2bfloat16_rn(x[c]);
+                if (c + 1 < cols)
+                    v.y = __float2bfloat16_rn(x[c + 1]);
+            }
+        }
+        *reinterpret_cast<__nv_bfloat162 *>(&tile[i][2 * tx]) = v;
     }
     __syncthreads();
-    for (int i = threadIdx.y; i < 32; i += blockDim.y) {
-        const int64_t c = c0 + i, r = r0 + threadIdx.x;
-        if (r < rows && c < cols)
-            dst[c * rows + r] = __float2bfloat16_rn(tile[threadIdx.x][i]);
+    __nv_bfloat16 *dst = logits ? a.dST : a.xT;
+    for (int i = ty; i < 64; i += 8) {
+        const int64_t c = c0 + i, r = r0 + 2 * tx;
+        if (c >= cols || r >= a.B)
+            continue;
+        if (r + 1 < a.B) {
+            __nv_bfloat162 v;
+            v.x = tile[2 * tx][i];
+            v.y = tile[2 * tx + 1][i];
+            *reinterpret_cast<__nv_bfloat162 *>(dst + c * a.ldB + r) = v;  // ldB and r are even
+        } else {
+            dst[c * a.ldB + r] = tile[2 * tx][i];
+        }
     }
 }
 
-// Sum (or maximum) over the block of one value per thread; every thread gets
-// the result.  red holds 32 slots; blockDim.x is a multiple of 32.
+// The block's sum of b and its maximum (MAX) or sum of a, one value of each per
+// thread; every thread gets both.  red holds 64 slots; blockDim.x is a multiple
+// of 32.
 template <bool MAX>
-__device__ __forceinline__ float block_reduce(float v, float *red)
+__device__ __forceinline__ void block_reduce2(float &a, float &b, float *red)
 {
+    auto warp = [&]() {
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        const float w = __shfl_xor_sync(kFull, v, o);
-        v = MAX ? fmaxf(v, w) : v + w;
-    }
+        for (int o = 16; o > 0; o >>= 1) {
+            const float w = __shfl_xor_sync(kFull, a, o);
+            a = MAX ? fmaxf(a, w) : a + w;
+            b += __shfl_xor_sync(kFull, b, o);
+        }
+    };
+    warp();
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
     __syncthreads();  // red is free again
-    if (lane == 0)
-        red[wid] = v;
-    __syncthreads();
-    v = lane < nw ? red[lane] : (MAX ? -INFINITY : 0.f);
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        const float w = __shfl_xor_sync(kFull, v, o);
-        v = MAX ? fmaxf(v, w) : v + w;
+    if (lane == 0) {
+        red[wid] = a;
+        red[32 + wid] = b;
     }
-    return v;
+    __syncthreads();
+    a = lane < nw ? red[lane] : (MAX ? -INFINITY : 0.f);
+    b = lane < nw ? red[32 + lane] : 0.f;
+    warp();
 }
 
 // One block per batch row: masked multi-positive InfoNCE over the labelled
@@ -205,12 +341,13 @@ __device__ __forceinline__ float block_reduce(float v, float *red)
 // not listed is a negative, so the row's H labels are first laid out in
 // shared memory (all -1, then the listed ones).  Writes the row loss, a
 // validity flag (|P| > 0) and the unscaled gradient softmax_{P u N}(S) -
-// 1[P]/|P| (0 outside P u N and on invalid rows).
+// 1[P]/|P| (0 outside P u N and on invalid rows), rounded to BF16 as the GEMMs
+// that read it need it.
 __global__ void infonce_kernel(const float *S, int64_t B, int H, const int32_t *cand, const int8_t *lab, int M,
-                               const int32_t *rowmap, float *dS, float *row_loss, int *valid)
+                               const int32_t *rowmap, __nv_bfloat16 *dS, int64_t ldS, float *row_loss, int *valid)
 {
     extern __shared__ int8_t lrow[];
-    __shared__ float red[32];
+    __shared__ float red[64];
     const int64_t r = blockIdx.x;
     const int64_t mr = rowmap ? rowmap[r] : r;
     for (int c = threadIdx.x; c < H; c += blockDim.x)
@@ -229,8 +366,8 @@ __global__ void infonce_kernel(const float *S, int64_t B, int H, const int32_t *
             mx = fmaxf(mx, s[c]);
         np += lrow[c] > 0 ? 1.f : 0.f;
     }
-    mx = block_reduce<true>(mx, red);
-    const int npos = static_cast<int>(block_reduce<false>(np, red));
+    block_reduce2<true>(mx, np, red);
+    const int npos = static_cast<int>(np);
     float z = 0.f, sp = 0.f;
     for (int c = threadIdx.x; c < H; c += blockDim.x) {
         if (lrow[c] != 0)
@@ -238,8 +375,7 @@ __global__ void infonce_kernel(const float *S, int64_t B, int H, const int32_t *
         if (lrow[c] > 0)
             sp += s[c];
     }
-    z = block_reduce<false>(z, red);
-    sp = block_reduce<false>(sp, red);
+    block_reduce2<false>(z, sp, red);
     const float lse = mx + logf(z);
     const bool ok = npos > 0;
     const float inv_np = ok ? 1.f / static_cast<float>(npos) : 0.f;
@@ -247,7 +383,7 @@ __global__ void infonce_kernel(const float *S, int64_t B, int H, const int32_t *
         float g = 0.f;
         if (ok && lrow[c] != 0)
             g = expf(s[c] - lse) - (lrow[c] > 0 ? inv_np : 0.f);
-        dS[r * H + c] = g;
+        dS[r * ldS + c] = __float2bfloat16_rn(g);
     }
     if (threadIdx.x == 0) {
         row_loss[r] = ok ? -(sp - npos * lse) * inv_np : 0.f;
@@ -259,8 +395,8 @@ __global__ void infonce_kernel(const float *S, int64_t B, int H, const int32_t *
 __global__ void finalize_loss_kernel(const float *row_loss, const int *valid, int64_t B, float tau, float *loss,
                                      float *scale)
 {
-    __shared__ float sl[256];
-    __shared__ int sv[256];
+    __shared__ float sl[1024];
+    __shared__ int sv[1024];
     float l = 0.f;
     int v = 0;
     for (int64_t i = threadIdx.x; i < B; i += blockDim.x) {
@@ -303,26 +439,77 @@ __global__ void norm_backward_kernel(const float *Y, const float *n, const float
         dZ[r * W + c] = (dY[r * W + c] - Y[r * W + c] * dot) * inv;
 }
 
-__global__ void colsum_kernel(const float *X, int64_t rows, int cols, float *out)
+// norm_backward_kernel for the queries (64 columns), 32 rows per block, with
+// what the next GEMMs read: dZ2 in BF16, by rows and transposed, and the
+// block's column sums (db2's partial sums).
+__global__ void __launch_bounds__(256)
+    query_backward_kernel(const float *Y, const float *n, const float *dY, int64_t rows, __nv_bfloat16 *dZ,
+                          __nv_bfloat16 *dZT, int64_t ld, float *part)
 {
-    const int c = blockIdx.x * blockDim.x + threadIdx.x;
-    if (c >= cols)
-        return;
-    float s = 0.f;
-    for (int64_t r = 0; r < rows; ++r)
-        s += X[r * cols + c];
-    out[c] = s;
+    __shared__ float dz[32][65];
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const int64_t r0 = static_cast<int64_t>(blockIdx.x) * 32;
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        const int64_t r = r0 + 4 * w + i;
+        float z0 = 0.f, z1 = 0.f;
+        if (r < rows) {
+            const float y0 = Y[r * 64 + lane], y1 = Y[r * 64 + 32 + lane];
+            const float g0 = dY[r * 64 + lane], g1 = dY[r * 64 + 32 + lane];
+            float dot = fmaf(y1, g1, fmaf(y0, g0, 0.f));
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1)
+                dot += __shfl_xor_sync(kFull, dot, o);
+            const float inv = n[r] > 0.f ? 1.f / n[r] : 0.f;
+            z0 = (g0 - y0 * dot) * inv;
+            z1 = (g1 - y1 * dot) * inv;
+            dZ[r * 64 + lane] = __float2bfloat16_rn(z0);
+            dZ[r * 64 + 32 + lane] = __float2bfloat16_rn(z1);
+        }
+        dz[4 * w + i][lane] = z0;
+        dz[4 * w + i][32 + lane] = z1;
+    }
+    __syncthreads();
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+        const int c = w + 8 * i;
+        const float v = dz[lane][c];
+        if (r0 + lane < rows)
+            dZT[c * ld + r0 + lane] = __float2bfloat16_rn(v);
+        float sum = v;
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1)
+            sum += __shfl_xor_sync(kFull, sum, o);
+        if (lane == 0)
+            part[static_cast<int64_t>(blockIdx.x) * 64 + c] = sum;
+    }
 }
 
-__global__ void row_norms_kernel(const float *E, int64_t rows, int W, float *n)
+// db1 and db2 from their partial sums, 32 columns per block (blocks 0..7: db1,
+// 8 and 9: db2), in a fixed order.  (One block that walked all rows took
+// 230 us per bias.)
+__global__ void __launch_bounds__(1024)
+    bias_sum_kernel(const float *part1, int64_t n1, const float *part2, int64_t n2, float *b1, float *b2)
 {
-    const int64_t r = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x;
-    if (r >= rows)
-        return;
-    float ss = 0.f;
-    for (int c = 0; c < W; ++c)
-        ss = fmaf(E[r * W + c], E[r * W + c], ss);
-    n[r] = sqrtf(ss);
+    __shared__ float sh[32][33];
+    const bool first = blockIdx.x < 8;
+    const float *part = first ? part1 : part2;
+    const int64_t n = first ? n1 : n2;
+    const int width = first ? 256 : 64, c0 = static_cast<int>(first ? blockIdx.x : blockIdx.x - 8) * 32;
+    const int lane = threadIdx.x & 31, g = threadIdx.x >> 5;
+    float s = 0.f;
+#pragma unroll 4
+    for (int64_t p = g; p < n; p += 32)
+        s += part[p * width + c0 + lane];
+    sh[g][lane] = s;
+    __syncthreads();
+    if (g == 0) {
+        float t = 0.f;
+#pragma unroll
+        for (int i = 0; i < 32; ++i)
+            t += sh[i][lane];
+        (first ? b1 : b2)[c0 + lane] = t;
+    }
 }
 
 // Adam with bias correction (Kingma & Ba), fp32 state
@@ -360,12 +547,14 @@ struct ann_trainer {
     float *params = nullptr, *grads = nullptr, *m = nullptr, *v = nullptr;
     ann_entry_model model;  // views into params + BF16 copies
     // scratch
-    float *z1 = nullptr, *qhat = nullptr, *nrm = nullptr, *S = nullptr, *dS = nullptr, *row_loss = nullptr;
-    float *dQ = nullptr, *dEh = nullptr, *dZ2 = nullptr, *dZ1 = nullptr, *Enrm = nullptr;
+    float *qhat = nullptr, *S = nullptr, *row_loss = nullptr;
+    float *dQ = nullptr, *dEh = nullptr, *part1 = nullptr, *part2 = nullptr;
     float *loss = nullptr, *scale = nullptr;
     int *valid = nullptr, *status = nullptr;
-    __nv_bfloat16 *a1 = nullptr, *qbf = nullptr, *EnT = nullptr, *dST = nullptr, *qT = nullptr, *a1T = nullptr,
-                  *dZ2T = nullptr, *xT = nullptr, *dZ1T = nullptr;
+    int64_t ldB = 0, ldH = 0;  // batch and hubs rounded up to whole 16-byte pieces
+    TowerTrain tower{};
+    __nv_bfloat16 *qbf = nullptr, *dS = nullptr, *dST = nullptr, *dZ2 = nullptr, *dZ2T = nullptr, *xT = nullptr,
+                  *dZ1T = nullptr;
     std::vector<void *> owned;
     ann::Fusion *fu = nullptr;  // topology-aware hub tower: hub rows are E + F
 };
@@ -443,17 +632,18 @@ ann_status trainer_grads(ann_trainer *t, const float *d_queries, const int32_t *
     M.E = t->params + o.E;
     if (st != ANN_OK)
         return st;
-    const float *Erows = t->fu ? t->fu->Eeff : M.E;
-    row_norms_kernel<<<blocks_for(H, 256), 256, 0, s>>>(Erows, H, 64, t->Enrm);
     const Operand X{d_queries, OP_F32, D, 1, B, D, rows};
-    st = launch_tower(&M, X, B, t->qhat, t->qbf, t->z1, t->a1, t->nrm, t->status, s);
-    if (st != ANN_OK)
+    if ((st = launch_tower(&M, X, B, t->qhat, t->qbf, &t->tower, t->status, s)) != ANN_OK)
         return st;
+    // what split GEMMs add into: the weight gradients, de_hat and dq_hat lie together
+    cudaError_t e = cudaMemsetAsync(t->grads, 0, static_cast<size_t>(o.total + (H + B) * 64) * 4, s);
+    if (e != cudaSuccess)
+        return cuda_status(e);
     // logits
     GemmArgs g{};
     g.status = t->status;
-    g.A = Operand{t->qbf, OP_BF16, 64, 1, B, 64, nullptr};
-    g.B = Operand{M.Eb, OP_BF16, 64, 1, H, 64, nullptr};
+    g.A = Mat{t->qbf, 64, B};
+    g.B = Mat{M.Eb, 64, H};
     g.M = B;
     g.N = H;
     g.K = 64;
@@ -462,16 +652,14 @@ ann_status trainer_grads(ann_trainer *t, const float *d_queries, const int32_t *
     g.ldo = H;
     if ((st = gemm<128>(g, s)) != ANN_OK)
         return st;
-    infonce_kernel<<<static_cast<unsigned>(B), 256, H, s>>>(t->S, B, H, d_cand, d_lab, n_listed, rows, t->dS,
+    infonce_kernel<<<static_cast<unsigned>(B), 256, H, s>>>(t->S, B, H, d_cand, d_lab, n_listed, rows, t->dS, t->ldH,
                                                              t->row_loss, t->valid);
-    finalize_loss_kernel<<<1, 256, 0, s>>>(t->row_loss, t->valid, B, t->tau, t->loss, t->scale);
+    finalize_loss_kernel<<<1, 1024, 0, s>>>(t->row_loss, t->valid, B, t->tau, t->loss, t->scale);
     // dq_hat = scale * dS e_hat  (B x 64, K = H)
-    transpose_bf16<<<dim3(blocks_for(64, 32), blocks_for(H, 32)), dim3(32, 8), 0, s>>>(
-        Operand{M.En, OP_F32, 64, 1, H, 64, nullptr}, H, 64, t->EnT);
     g = GemmArgs{};
     g.status = t->status;
-    g.A = Operand{t->dS, OP_F32, H, 1, B, H, nullptr};
-    g.B = Operand{t->EnT, OP_BF16, H, 1, 64, H, nullptr};
+    g.A = Mat{t->dS, t->ldH, B};
+    g.B = Mat{M.EnT, M.ldE, 64};
     g.M = B;
     g.N = 64;
     g.K = H;
@@ -482,12 +670,10 @@ ann_status trainer_grads(ann_trainer *t, const float *d_queries, const int32_t *
     if ((st = gemm<64>(g, s)) != ANN_OK)
         return st;
     // de_hat = scale * dS^T q_hat  (H x 64, K = B)
-    transpose_bf16<<<dim3(blocks_for(H, 32), blocks_for(B, 32)), dim3(32, 8), 0, s>>>(
-        Operand{t->dS, OP_F32, H, 1, B, H, nullptr}, B, H, t->dST);
-    transpose_bf16<<<dim3(blocks_for(64, 32), blocks_for(B, 32)), dim3(32, 8), 0, s>>>(
-        Operand{t->qhat, OP_F32, 64, 1, B, 64, nullptr}, B, 64, t->qT);
-    g.A = Operand{t->dST, OP_BF16, B, 1, H, B, nullptr};
-    g.B = Operand{t->qT, OP_BF16, B, 1, 64, B, nullptr};
+    const TransposeArgs ta{t->dS, t->ldH, H, t->dST, d_queries, rows, D, t->xT, B, t->ldB};
+    transpose_kernel<<<dim3(blocks_for(std::max(H, D), 64), blocks_for(B, 64), 2), 256, 0, s>>>(ta);
+    g.A = Mat{t->dST, t->ldB, H};
+    g.B = Mat{t->tower.qT, t->ldB, 64};
     g.M = H;
     g.N = 64;
     g.K = B;
@@ -495,21 +681,18 @@ ann_status trainer_grads(ann_trainer *t, const float *d_queries, const int32_t *
     if ((st = gemm<64>(g, s)) != ANN_OK)
         return st;
     // through the normalisations
-    norm_backward_kernel<<<blocks_for(B * 32, 256), 256, 0, s>>>(t->qhat, t->nrm, t->dQ, B, 64, t->dZ2);
-    norm_backward_kernel<<<blocks_for(static_cast<int64_t>(H) * 32, 256), 256, 0, s>>>(M.En, t->Enrm, t->dEh, H, 64,
+    query_backward_kernel<<<blocks_for(B, 32), 256, 0, s>>>(t->qhat, t->tower.nrm, t->dQ, B, t->dZ2, t->dZ2T, t->ldB,
+                                                            t->part2);
+    norm_backward_kernel<<<blocks_for(static_cast<int64_t>(H) * 32, 256), 256, 0, s>>>(M.En, M.Enrm, t->dEh, H, 64,
                                                                                       t->grads + o.E);
     // dL/dF = dL/d(E + F) = dL/dE
     if (t->fu && (st = fusion_backward(t->fu, t->grads + o.E, s)) != ANN_OK)
         return st;
-    // dW2 = A1^T dZ2 (256 x 64, K = B); db2
-    transpose_bf16<<<dim3(blocks_for(256, 32), blocks_for(B, 32)), dim3(32, 8), 0, s>>>(
-        Operand{t->a1, OP_BF16, 256, 1, B, 256, nullptr}, B, 256, t->a1T);
-    transpose_bf16<<<dim3(blocks_for(64, 32), blocks_for(B, 32)), dim3(32, 8), 0, s>>>(
-        Operand{t->dZ2, OP_F32, 64, 1, B, 64, nullptr}, B, 64, t->dZ2T);
+    // dW2 = A1^T dZ2 (256 x 64, K = B)
     g = GemmArgs{};
     g.status = t->status;
-    g.A = Operand{t->a1T, OP_BF16, B, 1, 256, B, nullptr};
-    g.B = Operand{t->dZ2T, OP_BF16, B, 1, 64, B, nullptr};
+    g.A = Mat{t->tower.a1T, t->ldB, 256};
+    g.B = Mat{t->dZ2T, t->ldB, 64};
     g.M = 256;
     g.N = 64;
     g.K = B;
@@ -518,28 +701,28 @@ ann_status trainer_grads(ann_trainer *t, const float *d_queries, const int32_t *
     g.ldo = 64;
     if ((st = gemm<64>(g, s)) != ANN_OK)
         return st;
-    colsum_kernel<<<1, 64, 0, s>>>(t->dZ2, B, 64, t->grads + o.b2);
-    // dZ1 = (dZ2 W2^T) * [Z1 > 0]  (B x 256, K = 64): B operand row n = W2[n][:]
-    g.A = Operand{t->dZ2, OP_F32, 64, 1, B, 64, nullptr};
-    g.B = Operand{M.W2, OP_F32, 64, 1, 256, 64, nullptr};
+    // dZ1 = (dZ2 W2^T) * [Z1 > 0]  (B x 256, K = 64), written transposed, with db1's partial sums
+    g = GemmArgs{};
+    g.status = t->status;
+    g.A = Mat{t->dZ2, 64, B};
+    g.B = Mat{M.W2b, 64, 256};
     g.M = B;
     g.N = 256;
     g.K = 64;
-    g.epi = EPI_RELU_MASK;
-    g.aux = t->z1;
-    g.out = t->dZ1;
-    g.ldo = 256;
-    if ((st = gemm<256>(g, s)) != ANN_OK)
+    g.alpha = 1.f;
+    g.mask = t->tower.zmask;
+    g.outT = t->dZ1T;
+    g.ldt = t->ldB;
+    g.part = t->part1;
+    if ((st = gemm<256>(g, s, EPI_HIDDEN)) != ANN_OK)
         return st;
-    colsum_kernel<<<1, 256, 0, s>>>(t->dZ1, B, 256, t->grads + o.b1);
+    bias_sum_kernel<<<10, 1024, 0, s>>>(t->part1, (B + 127) / 128 * 4, t->part2, (B + 31) / 32, t->grads + o.b1,
+                                        t->grads + o.b2);
     // dW1 = X^T dZ1  (D x 256, K = B)
-    transpose_bf16<<<dim3(blocks_for(D, 32), blocks_for(B, 32)), dim3(32, 8), 0, s>>>(X, B, D, t->xT);
-    transpose_bf16<<<dim3(blocks_for(256, 32), blocks_for(B, 32)), dim3(32, 8), 0, s>>>(
-        Operand{t->dZ1, OP_F32, 256, 1, B, 256, nullptr}, B, 256, t->dZ1T);
     g = GemmArgs{};
     g.status = t->status;
-    g.A = Operand{t->xT, OP_BF16, B, 1, D, B, nullptr};
-    g.B = Operand{t->dZ1T, OP_BF16, B, 1, 256, B, nullptr};
+    g.A = Mat{t->xT, t->ldB, D};
+    g.B = Mat{t->dZ1T, t->ldB, 256};
     g.M = D;
     g.N = 256;
     g.K = B;
@@ -587,33 +770,34 @@ ann_status ann_trainer_create(int device, int32_t in_dim, int32_t n_hubs, const 
     const int64_t B = max_batch, H = n_hubs;
     cudaError_t e = cudaSuccess;
     t->params = talloc<float>(t, o.total, e);
-    t->grads = talloc<float>(t, o.total, e);
+    t->grads = talloc<float>(t, o.total + (H + B) * 64, e);
+    t->dEh = t->grads + o.total;
+    t->dQ = t->dEh + H * 64;
     t->m = talloc<float>(t, o.total, e);
     t->v = talloc<float>(t, o.total, e);
-    t->z1 = talloc<float>(t, B * 256, e);
-    t->a1 = talloc<__nv_bfloat16>(t, B * 256, e);
+    t->ldB = (B + 7) / 8 * 8;
+    t->ldH = (H + 7) / 8 * 8;
+    t->tower.ld = t->ldB;
+    t->tower.zmask = talloc<uint32_t>(t, 8 * t->ldB, e);
+    t->tower.a1T = talloc<__nv_bfloat16>(t, 256 * t->ldB, e);
+    t->tower.qT = talloc<__nv_bfloat16>(t, 64 * t->ldB, e);
+    t->tower.nrm = talloc<float>(t, B, e);
     t->qhat = talloc<float>(t, B * 64, e);
     t->qbf = talloc<__nv_bfloat16>(t, B * 64, e);
-    t->nrm = talloc<float>(t, B, e);
     t->S = talloc<float>(t, B * H, e);
-    t->dS = talloc<float>(t, B * H, e);
+    t->dS = talloc<__nv_bfloat16>(t, B * t->ldH, e);
+    t->dST = talloc<__nv_bfloat16>(t, H * t->ldB, e);
     t->row_loss = talloc<float>(t, B, e);
     t->valid = talloc<int>(t, B, e);
-    t->dQ = talloc<float>(t, B * 64, e);
-    t->dEh = talloc<float>(t, H * 64, e);
-    t->dZ2 = talloc<float>(t, B * 64, e);
-    t->dZ1 = talloc<float>(t, B * 256, e);
-    t->Enrm = talloc<float>(t, H, e);
+    t->part1 = talloc<float>(t, (B + 127) / 128 * 4 * 256, e);
+    t->part2 = talloc<float>(t, (B + 31) / 32 * 64, e);
     t->loss = talloc<float>(t, 2, e);
     t->scale = talloc<float>(t, 2, e);
     t->status = talloc<int>(t, 4, e);
-    t->EnT = talloc<__nv_bfloat16>(t, H * 64, e);
-    t->dST = talloc<__nv_bfloat16>(t, B * H, e);
-    t->qT = talloc<__nv_bfloat16>(t, B * 64, e);
-    t->a1T = talloc<__nv_bfloat16>(t, B * 256, e);
-    t->dZ2T = talloc<__nv_bfloat16>(t, B * 64, e);
-    t->xT = talloc<__nv_bfloat16>(t, B * in_dim, e);
-    t->dZ1T = talloc<__nv_bfloat16>(t, B * 256, e);
+    t->dZ2 = talloc<__nv_bfloat16>(t, B * 64, e);
+    t->dZ2T = talloc<__nv_bfloat16>(t, 64 * t->ldB, e);
+    t->xT = talloc<__nv_bfloat16>(t, in_dim * t->ldB, e);
+    t->dZ1T = talloc<__nv_bfloat16>(t, 256 * t->ldB, e);
     ann_entry_model &M = t->model;
     M.in_dim = in_dim;
     M.H = n_hubs;
@@ -621,6 +805,10 @@ ann_status ann_trainer_create(int device, int32_t in_dim, int32_t n_hubs, const 
     M.W2t = talloc<__nv_bfloat16>(t, 256 * 64, e);
     M.En = talloc<float>(t, H * 64, e);
     M.Eb = talloc<__nv_bfloat16>(t, H * 64, e);
+    M.Enrm = talloc<float>(t, H, e);
+    M.W2b = talloc<__nv_bfloat16>(t, 256 * 64, e);
+    M.EnT = talloc<__nv_bfloat16>(t, 64 * t->ldH, e);
+    M.ldE = t->ldH;
     if (e == cudaSuccess) {
         M.W1 = t->params + o.W1;
         M.b1 = t->params + o.b1;

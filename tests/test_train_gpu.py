@@ -137,3 +137,25 @@ def test_listed_labels_train_like_their_dense_matrix():
     assert out[0][0] == out[1][0]
     # the reductions over the batch may add partial sums in another order
     assert _rel(out[0][1], out[1][1]) <= 1e-5
+
+
+@pytest.mark.parametrize("B,D,H", [(641, 33, 67), (2049, 512, 1_025)])
+def test_gradients_match_oracle_at_ragged_sizes(B, D, H):
+    # batches, widths and hub counts that are no multiple of a 16-byte piece, a
+    # 64-wide K chunk or a 128-row tile: the operands' last pieces are cut
+    X, W1, b1, W2, b2, E, mask, rows = _problem(B=B, D=D, H=H, seed=B)
+    t = ann.ann_trainer_create(D, W1, b1, W2, b2, E, B, tau=0.1, lr=1e-3)
+    try:
+        loss = ann.ann_trainer_step(t, torch.from_numpy(X).to(DEV), torch.from_numpy(rows).to(DEV), len(rows),
+                                    *dense_as_listed(mask), apply_update=False)
+        g = {k: np.zeros_like(v) for k, v in dict(W1=W1, b1=b1, W2=W2, b2=b2, E=E).items()}
+        ann.ann_trainer_get(t, g["W1"], g["b1"], g["W2"], g["b2"], g["E"], gradients=True)
+    finally:
+        ann.ann_trainer_free(t)
+    bf = ot.bf16_round
+    ref_loss, ref = ot.loss_and_grads(bf(X[rows]), bf(W1), b1.astype(np.float64), bf(W2), b2.astype(np.float64),
+                                      E.astype(np.float64), mask[rows], 0.1)
+    assert abs(loss - ref_loss) <= 1e-4 * abs(ref_loss)
+    for k in ("W1", "b1", "W2", "b2", "E"):
+        assert _rel(g[k], ref[k]) <= 8e-3, (k, _rel(g[k], ref[k]))
+        assert _cos(g[k], ref[k]) >= 0.99995, (k, _cos(g[k], ref[k]))
