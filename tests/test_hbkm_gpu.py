@@ -101,3 +101,15 @@ def test_full_size_invariants():
         np.testing.assert_allclose(cent[c], xd.mean(0), rtol=1e-3, atol=1e-3)
         d = ((xd - cent[c].astype(np.float64)) ** 2).sum(1)
         assert d[mem == hubs[c]][0] <= d.min() * (1 + 1e-4) + 1e-5
+
+
+@pytest.mark.parametrize("n,dim,k,levels,lam", [
+    (8_192, 36, 32, 2, 1.0), (8_193, 100, 3, 2, 50.0), (9_215, 4, 32, 1, 1e9), (33_000, 132, 3, 2, 0.3)])
+def test_visits_by_rounds(n, dim, k, levels, lam):
+    # clusters just above the size from which the visit goes 512 members at a
+    # time (a full and a partial last round, 32-member blocks of one member,
+    # ragged coordinate slices), on small whole numbers: many equal distances,
+    # so ties between children and uncertain members are frequent
+    rng = np.random.default_rng(n)
+    x = rng.integers(0, 3, size=(n, dim)).astype(np.float32)
+    _same(x, k, levels, lam, 3, synth.hbkm_keys(n, seed=5))
