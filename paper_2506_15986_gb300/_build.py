@@ -2,7 +2,7 @@
 
 Each translation unit is compiled in parallel (one nvcc process per file),
 then linked into ``paper_2506_15986_gb300/libann.so`` against the shared CUDA
-runtime and cuBLAS.  The object files go to ``paper_2506_15986_gb300/_build/``.
+runtime.  The object files go to ``paper_2506_15986_gb300/_build/``.
 """
 from __future__ import annotations
 
@@ -81,7 +81,7 @@ def build(verbose: bool = False, force: bool = False) -> str:
     if not os.path.isdir(libdir):
         libdir = os.path.join(cuda, "lib")
     cmd = [nvcc, *ARCH, "-shared", "-cudart", "shared", "-o", tmp, *objs,
-           "-L", libdir, "-lcublas", "-Xlinker", f"-rpath,{libdir}"]
+           "-L", libdir, "-Xlinker", f"-rpath,{libdir}"]
     r = subprocess.run(cmd, capture_output=True, text=True)
     if r.returncode != 0:
         raise RuntimeError(f"link failed:\n{r.stdout}\n{r.stderr}")

@@ -1,14 +1,7 @@
-// build.cu -- offline index construction on the GPU: exact k-NN (also the
-// ground truth of recall@k), the proximity graph of Sec. 2.1 Def. 1 (K-NN
-// candidates, relative-neighbourhood pruning, reachability repair from the
-// navigating node) and the navigating node (medoid).
-//
-// k-NN: candidate scores come from a plain cuBLAS SGEMM (x.y per query chunk);
-// a warp per row keeps the best KP = k + margin keys by the expanded distance
-// |y|^2 - 2 x.y with a threshold filter, then the KP candidates are re-scored
-// exactly (direct differences: int32 for uint8, fp32 otherwise) and sorted by
-// (distance, id).
-#include <cublas_v2.h>
+// build.cu -- offline index construction on the GPU: the proximity graph of
+// Sec. 2.1 Def. 1 (exact K-NN candidates from knn.cu, relative-neighbourhood
+// pruning, reachability repair from the navigating node) and the navigating
+// node (medoid).
 #include <cuda_runtime.h>
 #include <stdint.h>
 
@@ -20,129 +13,6 @@
 
 namespace ann {
 namespace {
-
-constexpr int kSelWarps = 4;
-
-__global__ void u8_to_f32(const uint8_t *x, float *y, int64_t count)
-{
-    for (int64_t i = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x; i < count;
-         i += static_cast<int64_t>(gridDim.x) * blockDim.x)
-        y[i] = static_cast<float>(x[i]);
-}
-
-// squared norms of fp32 rows (exact integers for uint8-valued rows)
-__global__ void row_norms(const float *x, int64_t n, int dim, float *out)
-{
-    const int lane = threadIdx.x & 31;
-    const int64_t row = (blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x) >> 5;
-    if (row >= n)
-        return;
-    float s = 0.f;
-    for (int c = lane; c < dim; c += 32) {
-        const float v = x[row * dim + c];
-        s = fmaf(v, v, s);
-    }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1)
-        s += __shfl_xor_sync(kFull, s, o);
-    if (lane == 0)
-        out[row] = s;
-}
-
-// Per row of a chunk of scores S (rows x ld, row-major): keep the KP = 32*KPL
-// smallest keys (expanded distance, column id).  L2: key distance =
-// ny[j] - 2 S[r][j]; IP: -S[r][j].  Column self0 + r is skipped when
-// exclude_self.  Output: KP candidate ids per row, best first.
-template <int KPL>
-__global__ void __launch_bounds__(32 * kSelWarps)
-    select_topk(const float *S, int64_t ld, int64_t N, int rows, const float *ny, int metric,
-                int64_t self0, int exclude_self, int32_t *out)
-{
-    constexpr int KP = 32 * KPL;
-    constexpr int BCAP = 256;
-    __shared__ uint64_t sh_top[kSelWarps][2][KP];
-    __shared__ uint64_t sh_buf[kSelWarps][BCAP];
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    const int r = blockIdx.x * kSelWarps + w;
-    if (r >= rows)
-        return;
-    uint64_t *T = sh_top[w][0];
-    uint64_t *Tn = sh_top[w][1];
-    uint64_t *B = sh_buf[w];
-    for (int i = lane; i < KP; i += 32)
-        T[i] = kKeyMax;
-    __syncwarp();
-    uint64_t thr = kKeyMax;
-    int nb = 0;
-    const float *row = S + static_cast<int64_t>(r) * ld;
-    const int64_t self = exclude_self ? self0 + r : -1;
-
-    auto flush = [&]() {
-        // sort the buffer (pad to 256 with max keys) ...
-        uint64_t k[8];
-#pragma unroll
-        for (int t = 0; t < 8; ++t) {
-            const int e = t * 32 + lane;
-            k[t] = e < nb ? B[e] : kKeyMax;
-        }
-        warp_sort_n<8>(k, lane);
-        __syncwarp();
-#pragma unroll
-        for (int t = 0; t < 8; ++t)
-            B[t * 32 + lane] = k[t];
-        __syncwarp();
-        // ... and merge it with the kept list by rank
-        for (int i = lane; i < KP; i += 32) {
-            const uint64_t v = T[i];
-            const int pos = i + count_less_raw(B, nb, v);
-            if (pos < KP)
-                Tn[pos] = v;
-        }
-        for (int j = lane; j < nb; j += 32) {
-            const uint64_t v = B[j];
-            const int pos = j + count_less_raw(T, KP, v);
-            if (pos < KP)
-                Tn[pos] = v;
-        }
-        __syncwarp();
-        uint64_t *t = T;
-        T = Tn;
-        Tn = t;
-        thr = T[KP - 1];
-        nb = 0;
-    };
-
-    for (int64_t j0 = 0; j0 < N; j0 += 128) {
-        const int64_t j = j0 + 4 * lane;
-        float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
-        if (j < N)
-            v = *reinterpret_cast<const float4 *>(row + j);  // ld % 4 == 0, padded columns exist
-        const float vs[4] = {v.x, v.y, v.z, v.w};
-#pragma unroll
-        for (int t = 0; t < 4; ++t) {
-            const int64_t c = j + t;
-            uint64_t key = kKeyMax;
-            if (c < N && c != self) {
-                const float d = metric == ANN_L2 ? fmaf(-2.f, vs[t], ny[c]) : -vs[t];
-                key = make_key(f32_to_ord(d), static_cast<int32_t>(c)) >> 1;  // id in low 31 bits
-            }
-            const bool pass = key < thr;
-            const unsigned m = __ballot_sync(kFull, pass);
-            if (pass)
-                B[nb + __popc(m & lanemask_lt())] = key;
-            nb += __popc(m);
-        }
-        __syncwarp();
-        if (nb >= BCAP - 128)
-            flush();
-    }
-    if (nb > 0)
-        flush();
-    for (int i = lane; i < KP; i += 32) {
-        const uint64_t v = T[i];
-        out[static_cast<int64_t>(r) * KP + i] = v == kKeyMax ? -1 : static_cast<int32_t>(v & 0x7fffffffu);
-    }
-}
 
 // exact distance between a base row and a query row (uint8: int32 squared L2)
 template <int DT, int MT>
@@ -180,43 +50,6 @@ __device__ __forceinline__ uint32_t exact_dist_bits(const uint8_t *x, const uint
         if constexpr (MT == ANN_IP)
             s = -s;
         return f32_to_ord(s);
-    }
-}
-
-// Re-score the KP candidates of each query exactly, sort by (distance, id),
-// write the best k ids and distances (int32 for uint8, fp32 otherwise).
-template <int DT, int MT, int KPL>
-__global__ void rescore_topk(const uint8_t *base, int rowbytes, const uint8_t *queries, int qbytes,
-                             int dim, int64_t nq, const int32_t *cand, int k, int32_t *out_ids,
-                             void *out_dists)
-{
-    constexpr int KP = 32 * KPL;
-    const int lane = threadIdx.x & 31;
-    const int64_t r = (blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x) >> 5;
-    if (r >= nq)
-        return;
-    const uint8_t *q = queries + r * qbytes;
-    uint64_t key[KPL];
-#pragma unroll
-    for (int t = 0; t < KPL; ++t) {
-        const int32_t id = cand[r * KP + t * 32 + lane];
-        key[t] = id < 0 ? kKeyMax
-                        : make_key(exact_dist_bits<DT, MT>(base + static_cast<int64_t>(id) * rowbytes, q, dim), id);
-    }
-    warp_sort_n<KPL>(key, lane);
-#pragma unroll
-    for (int t = 0; t < KPL; ++t) {
-        const int e = t * 32 + lane;
-        if (e < k) {
-            const uint64_t v = key[t];
-            const bool ok = v != kKeyMax;
-            out_ids[r * k + e] = ok ? key_id(v) : -1;
-            const uint32_t db = static_cast<uint32_t>(v >> 32);
-            if constexpr (DT == ANN_U8)
-                reinterpret_cast<int32_t *>(out_dists)[r * k + e] = ok ? static_cast<int32_t>(db) : INT32_MAX;
-            else
-                reinterpret_cast<float *>(out_dists)[r * k + e] = ok ? ord_to_f32(db) : __int_as_float(0x7f800000);
-        }
     }
 }
 
@@ -410,15 +243,6 @@ __global__ void set_flags(uint8_t *flags, const int32_t *ids, int count, uint8_t
         flags[ids[i]] = v;
 }
 
-struct Cublas {
-    cublasHandle_t h = nullptr;
-    ~Cublas()
-    {
-        if (h)
-            cublasDestroy(h);
-    }
-};
-
 template <typename T>
 struct DevBuf {
     T *p = nullptr;
@@ -442,82 +266,7 @@ struct DevBuf {
             return cuda_status(e_);          \
     } while (0)
 
-size_t kp_for(int k) { return k <= 32 ? 64 : 128; }
-
 }  // namespace
-
-// Exact k-NN of nq query rows among n base rows (see file comment).
-ann_status knn_exact(const void *d_base, int64_t n, int dim, int dtype, int metric, const void *d_queries,
-                     int64_t nq, int k, bool exclude_self, int32_t *d_ids, void *d_dists, cudaStream_t s)
-{
-    const int es = elem_size(dtype);
-    const int rowbytes = dim * es;
-    const int qbytes = dtype == ANN_U8 ? dim : dim * 4;
-    const int KP = static_cast<int>(kp_for(k));
-    // fp32 views of base and queries for the GEMM
-    DevBuf<float> bf, qf, ny, Sbuf;
-    DevBuf<int32_t> cand;
-    const float *B = static_cast<const float *>(d_base);
-    const float *Q = static_cast<const float *>(d_queries);
-    if (dtype == ANN_U8) {
-        CK(bf.alloc(static_cast<size_t>(n) * dim, s));
-        u8_to_f32<<<2048, 256, 0, s>>>(static_cast<const uint8_t *>(d_base), bf.p, n * dim);
-        B = bf.p;
-        if (d_queries == d_base) {
-            Q = bf.p;
-        } else {
-            CK(qf.alloc(static_cast<size_t>(nq) * dim, s));
-            u8_to_f32<<<2048, 256, 0, s>>>(static_cast<const uint8_t *>(d_queries), qf.p, nq * dim);
-            Q = qf.p;
-        }
-    } else if (dtype != ANN_F32) {
-        return ANN_ERR_UNSUPPORTED;
-    }
-    CK(ny.alloc(n, s));
-    row_norms<<<static_cast<unsigned>((n * 32 + 255) / 256), 256, 0, s>>>(B, n, dim, ny.p);
-    const int64_t ld = (n + 3) / 4 * 4;
-    const size_t budget = static_cast<size_t>(4) << 30;  // bytes of scores per chunk
-    int64_t qc = std::max<int64_t>(1, std::min<int64_t>(nq, static_cast<int64_t>(budget / (4 * ld))));
-    CK(Sbuf.alloc(static_cast<size_t>(qc) * ld, s));
-    CK(cand.alloc(static_cast<size_t>(qc) * KP, s));
-    Cublas cb;
-    if (cublasCreate(&cb.h) != CUBLAS_STATUS_SUCCESS)
-        return ANN_ERR_CUDA;
-    cublasSetStream(cb.h, s);
-    cublasSetMathMode(cb.h, CUBLAS_PEDANTIC_MATH);  // true fp32, no reduced-precision modes
-    const float one = 1.f, zero = 0.f;
-    for (int64_t q0 = 0; q0 < nq; q0 += qc) {
-        const int rows = static_cast<int>(std::min<int64_t>(qc, nq - q0));
-        // S (rows x n, row-major, ld) = Q[q0:q0+rows] . B^T
-        if (cublasSgemm(cb.h, CUBLAS_OP_T, CUBLAS_OP_N, static_cast<int>(n), rows, dim, &one, B, dim,
-                        Q + q0 * dim, dim, &zero, Sbuf.p, static_cast<int>(ld)) != CUBLAS_STATUS_SUCCESS)
-            return ANN_ERR_CUDA;
-        const unsigned grid = (rows + kSelWarps - 1) / kSelWarps;
-        if (KP == 64)
-            select_topk<2><<<grid, 32 * kSelWarps, 0, s>>>(Sbuf.p, ld, n, rows, ny.p, metric, q0,
-                                                           exclude_self ? 1 : 0, cand.p);
-        else
-            select_topk<4><<<grid, 32 * kSelWarps, 0, s>>>(Sbuf.p, ld, n, rows, ny.p, metric, q0,
-                                                           exclude_self ? 1 : 0, cand.p);
-        CK(cudaGetLastError());
-        const uint8_t *qb = static_cast<const uint8_t *>(d_queries) + q0 * qbytes;
-        const unsigned rgrid = static_cast<unsigned>((rows * 32 + 127) / 128);
-        int32_t *oi = d_ids + q0 * k;
-        void *od = static_cast<uint8_t *>(d_dists) + q0 * k * 4;
-        const uint8_t *bb = static_cast<const uint8_t *>(d_base);
-#define RESCORE(DT, MT, KPL) \
-    rescore_topk<DT, MT, KPL><<<rgrid, 128, 0, s>>>(bb, rowbytes, qb, qbytes, dim, rows, cand.p, k, oi, od)
-        if (dtype == ANN_U8)
-            KP == 64 ? RESCORE(ANN_U8, ANN_L2, 2) : RESCORE(ANN_U8, ANN_L2, 4);
-        else if (metric == ANN_L2)
-            KP == 64 ? RESCORE(ANN_F32, ANN_L2, 2) : RESCORE(ANN_F32, ANN_L2, 4);
-        else
-            KP == 64 ? RESCORE(ANN_F32, ANN_IP, 2) : RESCORE(ANN_F32, ANN_IP, 4);
-#undef RESCORE
-        CK(cudaGetLastError());
-    }
-    return ANN_OK;
-}
 
 ann_status medoid_gpu(const void *d_base, int64_t n, int dim, int dtype, cudaStream_t s, int32_t *out)
 {

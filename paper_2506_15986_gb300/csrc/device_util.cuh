@@ -233,6 +233,42 @@ __device__ __forceinline__ void warp_sort_n(uint64_t (&k)[NPL], int lane)
     }
 }
 
+// warp_sort_n with rolled stage loops: a few dozen instructions instead of
+// hundreds, for kernels whose warps run out of step and share one instruction
+// cache.  NPL is 2 or 4.
+template <int NPL>
+__device__ __forceinline__ void warp_sort_rolled(uint64_t (&k)[NPL], int lane)
+{
+    auto exchange = [&](int r, int rj, int kk) {
+        const bool asc = ((r * 32 + lane) & kk) == 0;
+        const uint64_t a = k[r], b = k[r | rj];
+        k[r] = asc ? kmin(a, b) : kmax(a, b);
+        k[r | rj] = asc ? kmax(a, b) : kmin(a, b);
+    };
+#pragma unroll 1
+    for (int kk = 2; kk <= 32 * NPL; kk <<= 1) {
+#pragma unroll 1
+        for (int j = kk >> 1; j > 0; j >>= 1) {
+            if (NPL == 4 && j == 64) {
+                exchange(0, NPL / 2, kk);
+                exchange(1, NPL / 2, kk);
+            } else if (j == 32) {
+                exchange(0, 1, kk);
+                if (NPL == 4)
+                    exchange(NPL - 2, 1, kk);
+            } else {
+                const bool lower = (lane & j) == 0;
+#pragma unroll
+                for (int r = 0; r < NPL; ++r) {
+                    const uint64_t o = __shfl_xor_sync(kFull, k[r], j);
+                    const bool asc = ((r * 32 + lane) & kk) == 0;
+                    k[r] = (lower == asc) ? kmin(k[r], o) : kmax(k[r], o);
+                }
+            }
+        }
+    }
+}
+
 // number of entries of the sorted array a[0..len) whose plain key is < v
 __device__ __forceinline__ int count_less(const uint64_t *a, int len, uint64_t v)
 {

@@ -82,7 +82,8 @@ int default_spill_bits(int L);
 // (order_items: work items of a grouped work order, 0 without one).
 size_t search_scratch_bytes(int teams, int spill_bits, int64_t order_items);
 
-// Exact k-NN (build.cu): candidates from an fp32 GEMM, exact re-scoring.
+// Exact k-NN (knn.cu): candidates from tensor-core scores, exact re-scoring.
+// Waits for the stream.
 ann_status knn_exact(const void *d_base, int64_t n, int dim, int dtype, int metric, const void *d_queries,
                      int64_t nq, int k, bool exclude_self, int32_t *d_ids, void *d_dists, cudaStream_t s);
 

@@ -143,3 +143,30 @@ def test_insertion_graph_builder():
     assert rec[0] >= rec[1] - 0.02, rec
     with pytest.raises(ann.AnnError):
         ann.ann_build_graph_insert(x, n, d, ann.F32, 64, 48, 1.0, 15000, 15000, g_in)  # R > 32
+
+
+@pytest.mark.parametrize("n,nq,d,k,dtype,metric,self_", [
+    (1, 1, 4, 1, "f32", "l2", False), (127, 3, 64, 32, "f32", "l2", False), (128, 128, 60, 33, "f32", "ip", False),
+    (129, 129, 128, 100, "f32", "l2", True), (4_099, 130, 132, 10, "f32", "l2", False),
+    (1_000, 257, 200, 128, "f32", "ip", False), (3_000, 50, 960, 64, "f32", "l2", False),
+    (700, 9, 1_028, 1, "f32", "l2", False), (20_000, 20_001, 16, 1, "f32", "l2", False),
+    (130, 130, 16, 128, "u8", "l2", True), (5_000, 300, 128, 32, "u8", "l2", False),
+    (5_000, 300, 528, 10, "u8", "l2", False)])
+def test_knn_edges_exact(n, nq, d, k, dtype, metric, self_):
+    # whole numbers: every distance is exact in fp32, many are equal, and ties go
+    # to the smaller id, so ids must agree one by one.  Tiles of 128 rows and
+    # columns, part-filled; one to nine 128-coordinate phases; K chunks resident
+    # and streamed; lists of 64 and 128, one row to a CTA and shared
+    rng = np.random.default_rng(n + d)
+    if dtype == "u8":
+        base = rng.integers(0, 256, size=(n, d)).astype(np.uint8)
+        base[n // 2:] = base[:n - n // 2]  # every row twice
+        q = base if self_ else rng.integers(0, 256, size=(nq, d)).astype(np.uint8)
+    else:
+        base = rng.integers(-3, 4, size=(n, d)).astype(np.float32)
+        q = base if self_ else rng.integers(-3, 4, size=(nq, d)).astype(np.float32)
+    ids, dd = _knn_gpu(base, q, k, ann.IP if metric == "ip" else ann.L2, self_)
+    oi, od = oracle.knn(base, q.astype(np.float64), k, metric=oracle.IP if metric == "ip" else oracle.L2,
+                        exclude=np.arange(n) if self_ else None)
+    assert np.array_equal(ids, oi)
+    assert np.array_equal(dd.astype(np.float64)[oi >= 0], od[oi >= 0])
