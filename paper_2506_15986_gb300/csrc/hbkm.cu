@@ -526,9 +526,10 @@ __global__ void hb_scatter(int64_t n, int k, const int32_t *perm, const int32_t 
 // here, the mean of all rows among them.
 constexpr int kMeanStages = 8;
 
+template <typename I>
 __global__ void __launch_bounds__(32)
     hb_means(const float *__restrict__ x, int dim, int64_t lists, const int64_t *__restrict__ seg,
-             const int32_t *__restrict__ perm, float *__restrict__ out)
+             const I *__restrict__ perm, float *__restrict__ out)
 {
     __shared__ __align__(16) float ring[kMeanStages][32][32];
     constexpr unsigned kAll = 0xffffffffu;
@@ -541,16 +542,16 @@ __global__ void __launch_bounds__(32)
         if (b == e)
             continue;
         const int64_t stages = (e - b + 31) / 32;
-        int32_t ids = b + lane < e ? perm[b + lane] : -1;  // the next stage's rows
+        I ids = b + lane < e ? perm[b + lane] : -1;  // the next stage's rows
         auto fill = [&](int64_t s) {
             if (s < stages) {
-                const int32_t cur = ids;
+                const I cur = ids;
                 const int64_t nx = b + (s + 1) * 32 + lane;
                 ids = nx < e ? perm[nx] : -1;
                 float *dst = &ring[s % kMeanStages][0][0];
 #pragma unroll
                 for (int r = 0; r < 8; ++r) {
-                    const int32_t row = __shfl_sync(kAll, cur, 4 * r + sub);
+                    const I row = __shfl_sync(kAll, cur, 4 * r + sub);
                     if (row >= 0 && piece < w4) {
                         const unsigned to = static_cast<unsigned>(
                             __cvta_generic_to_shared(dst + (4 * r + sub) * 32 + 4 * piece));
@@ -660,6 +661,12 @@ unsigned grid_for(int64_t items, int per_block)
 
 }  // namespace
 
+void list_means(const float *x, int dim, int64_t lists, const int64_t *seg, const int64_t *list, float *out,
+                cudaStream_t s)
+{
+    hb_means<int64_t><<<means_grid(lists, dim), 32, 0, s>>>(x, dim, lists, seg, list, out);
+}
+
 }  // namespace ann
 
 using namespace ann;
@@ -708,7 +715,7 @@ ann_status ann_hbkm(const float *d_x, int64_t n, int32_t dim, int32_t k, int32_t
     const int64_t seg0[2] = {0, n};
     HB_CK(cudaMemcpyAsync(seg.p, seg0, sizeof(seg0), cudaMemcpyHostToDevice, s));
     auto means = [&](int64_t lists, const Buf &sg, const Buf &list, const Buf &out) {
-        hb_means<<<means_grid(lists, dim), 32, 0, s>>>(d_x, dim, lists, sg.as<int64_t>(), list.as<int32_t>(),
+        hb_means<int32_t><<<means_grid(lists, dim), 32, 0, s>>>(d_x, dim, lists, sg.as<int64_t>(), list.as<int32_t>(),
                                                                 out.as<float>());
     };
     means(1, seg, perm, cent);  // level 0: the mean of all rows

@@ -87,4 +87,10 @@ size_t search_scratch_bytes(int teams, int spill_bits, int64_t order_items);
 ann_status knn_exact(const void *d_base, int64_t n, int dim, int dtype, int metric, const void *d_queries,
                      int64_t nq, int k, bool exclude_self, int32_t *d_ids, void *d_dists, cudaStream_t s);
 
+// Means of lists of fp32 rows (hbkm.cu): list c is list[seg[c] .. seg[c + 1]), added
+// in that order; an empty list leaves out's row as it is.  dim % 4 == 0, x
+// 16-byte aligned.
+void list_means(const float *x, int dim, int64_t lists, const int64_t *seg, const int64_t *list, float *out,
+                cudaStream_t s);
+
 }  // namespace ann

@@ -35,19 +35,124 @@ __global__ void gather_rows(const uint8_t *src, int rowbytes, const int64_t *row
         *reinterpret_cast<uint4 *>(d + o) = *reinterpret_cast<const uint4 *>(s + o);
 }
 
-// centroid j = mean of its members (listed in id order by the host), in fp32
-template <typename T>
-__global__ void centroid_update(const T *x, int dim, const int64_t *order, const int64_t *start, float *cent)
+// ---- members of every centroid in row order: a stable counting sort ----------
+// Blocks of `per` rows count their rows of every centroid (part, [blocks][k]),
+// the counts become first places (down the blocks, then across the centroids),
+// and each block places its rows, 32 at a time in row order.  On the host,
+// between a copy of the assignment and one of the order, this was most of an
+// iteration: 65,536 rows, 1,024 centroids, five iterations and the assignment of
+// 200,000 rows 12.2 ms, 6.2 ms with it here (30 us an iteration).
+constexpr int kSortThreads = 1024;
+
+__global__ void __launch_bounds__(kSortThreads)
+    members_count(const int32_t *asg, int64_t m, int64_t per, int k, int32_t *part)
 {
-    const int j = blockIdx.x;
-    const int64_t a = start[j], b = start[j + 1];
-    if (a == b)
-        return;  // empty: re-seeded by the host
-    for (int c = threadIdx.x; c < dim; c += blockDim.x) {
-        float s = 0.f;
-        for (int64_t i = a; i < b; ++i)
-            s += static_cast<float>(x[order[i] * dim + c]);
-        cent[static_cast<int64_t>(j) * dim + c] = s / static_cast<float>(b - a);
+    const int64_t b = blockIdx.x, end = min(m, (b + 1) * per);
+    for (int64_t i = b * per + threadIdx.x; i < end; i += kSortThreads)
+        if (asg[i] >= 0)
+            atomicAdd(part + b * k + asg[i], 1);
+}
+
+// part[b][j] becomes the number of rows of centroid j in earlier blocks
+__global__ void members_down(int32_t *part, int blocks, int k, int64_t *count)
+{
+    const int j = blockIdx.x * blockDim.x + threadIdx.x;
+    if (j >= k)
+        return;
+    int64_t run = 0;
+#pragma unroll 8
+    for (int b = 0; b < blocks; ++b) {
+        const int32_t c = part[static_cast<int64_t>(b) * k + j];
+        part[static_cast<int64_t>(b) * k + j] = static_cast<int32_t>(run);
+        run += c;
+    }
+    count[j] = run;
+}
+
+// One CTA: start = the exclusive sums of count (start[k] the total), the number
+// of empty centroids, and the sum of the distances.
+struct KmeansState {
+    double objective;
+    int64_t empty;
+};
+
+__global__ void __launch_bounds__(kSortThreads)
+    members_across(const int64_t *count, int k, int64_t *start, const float *dist, int64_t m, KmeansState *st)
+{
+    __shared__ int64_t warp_sum[32];
+    __shared__ double warp_obj[32];
+    __shared__ int64_t warp_empty[32];
+    const int t = threadIdx.x, lane = t & 31, w = t >> 5;
+    int64_t base = 0, empty = 0;
+    for (int j0 = 0; j0 < k; j0 += kSortThreads) {
+        const int j = j0 + t;
+        const int64_t c = j < k ? count[j] : 0;
+        empty += j < k && c == 0;
+        int64_t inc = c;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int64_t u = __shfl_up_sync(kFull, inc, o);
+            inc += lane >= o ? u : 0;
+        }
+        if (lane == 31)
+            warp_sum[w] = inc;
+        __syncthreads();
+        int64_t before = 0, all = 0;
+        for (int i = 0; i < 32; ++i) {
+            before += i < w ? warp_sum[i] : 0;
+            all += warp_sum[i];
+        }
+        if (j < k)
+            start[j] = base + before + inc - c;
+        base += all;
+        __syncthreads();
+    }
+    double obj = 0.0;
+#pragma unroll 8
+    for (int64_t i = t; i < m; i += kSortThreads)
+        obj += dist[i];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        obj += __shfl_xor_sync(kFull, obj, o);
+        empty += __shfl_xor_sync(kFull, empty, o);
+    }
+    if (lane == 0) {
+        warp_obj[w] = obj;
+        warp_empty[w] = empty;
+    }
+    __syncthreads();
+    if (t == 0) {
+        for (int i = 1; i < 32; ++i) {
+            obj += warp_obj[i];
+            empty += warp_empty[i];
+        }
+        start[k] = base;
+        st->objective = obj;
+        st->empty = empty;
+    }
+}
+
+__global__ void __launch_bounds__(kSortThreads)
+    members_place(const int32_t *asg, int64_t m, int64_t per, int k, int32_t *part, const int64_t *start,
+                  int64_t *order)
+{
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const int64_t b = blockIdx.x, end = min(m, (b + 1) * per);
+    for (int64_t i0 = b * per; i0 < end; i0 += kSortThreads) {
+        const int64_t i = i0 + threadIdx.x;
+        const int a = i < end ? asg[i] : -1;
+        const unsigned same = __match_any_sync(kFull, a);
+        for (int v = 0; v < kSortThreads / 32; ++v) {
+            if (v == w && a >= 0) {
+                const int leader = __ffs(same) - 1;
+                int first = 0;
+                if (lane == leader)
+                    first = atomicAdd(part + b * k + a, __popc(same));
+                first = __shfl_sync(same, first, leader);
+                order[start[a] + first + __popc(same & lanemask_lt())] = i;
+            }
+            __syncthreads();
+        }
     }
 }
 
@@ -174,14 +279,21 @@ ann_status ann_kmeans(const void *d_x, int64_t n, int32_t dim, int32_t dtype, co
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     const int rowbytes = dim * es;
     // the sample, as fp32 rows (the k-NN assignment runs on fp32 data)
-    Scoped rows(s), xs(s), xf(s), ids(s), dd(s), ord(s), st(s), which(s), srows(s);
+    Scoped rows(s), xs(s), xf(s), ids(s), dd(s), ord(s), st(s), which(s), srows(s), part(s), cnt(s), state(s);
+    // blocks of the counting sort: at least 1,024 rows, at most 2^24 counters
+    const int64_t max_blocks = std::max<int64_t>(1, (int64_t{1} << 24) / k);
+    const int64_t blocks = std::min<int64_t>((m + kSortThreads - 1) / kSortThreads, max_blocks);
+    const int64_t per = (m + blocks - 1) / blocks;
+    CK(part.alloc(static_cast<size_t>(blocks) * k * 4));
+    CK(cnt.alloc(static_cast<size_t>(k) * 8));
+    CK(state.alloc(sizeof(KmeansState)));
     CK(rows.alloc(m * 8));
     CK(xs.alloc(static_cast<size_t>(m) * rowbytes));
     CK(xf.alloc(static_cast<size_t>(m) * dim * 4));
     CK(ids.alloc(m * 4));
     CK(dd.alloc(m * 4));
     CK(ord.alloc(m * 8));
-    CK(st.alloc((k + 1) * 8));
+    CK(st.alloc((static_cast<size_t>(k) + 1) * 8));
     CK(which.alloc(k * 4));
     CK(srows.alloc(k * 8));
     CK(cudaMemcpyAsync(rows.p, sample_rows, m * 8, cudaMemcpyHostToDevice, s));
@@ -204,42 +316,39 @@ ann_status ann_kmeans(const void *d_x, int64_t n, int32_t dim, int32_t dtype, co
     CK(cudaMemcpyAsync(which.p, wj.data(), k * 4, cudaMemcpyHostToDevice, s));
     set_centroid_rows<float><<<k, 128, 0, s>>>(X, dim, static_cast<int64_t *>(srows.p),
                                                static_cast<int32_t *>(which.p), k, d_centroids);
-    std::vector<int32_t> asg(m);
-    std::vector<float> dist(m);
-    std::vector<int64_t> order(m), start(k + 1);
     for (int it = 0; it < iters; ++it) {
         ann_status r = knn_exact(d_centroids, k, dim, ANN_F32, ANN_L2, X, m, 1, false,
                                  static_cast<int32_t *>(ids.p), dd.p, s);
         if (r != ANN_OK)
             return r;
-        CK(cudaMemcpyAsync(asg.data(), ids.p, m * 4, cudaMemcpyDeviceToHost, s));
-        CK(cudaMemcpyAsync(dist.data(), dd.p, m * 4, cudaMemcpyDeviceToHost, s));
+        const int32_t *asg = static_cast<int32_t *>(ids.p);
+        int32_t *pt = static_cast<int32_t *>(part.p);
+        int64_t *start = static_cast<int64_t *>(st.p), *order = static_cast<int64_t *>(ord.p);
+        KmeansState h{};
+        CK(cudaMemsetAsync(part.p, 0, static_cast<size_t>(blocks) * k * 4, s));
+        members_count<<<static_cast<unsigned>(blocks), kSortThreads, 0, s>>>(asg, m, per, k, pt);
+        members_down<<<(k + 255) / 256, 256, 0, s>>>(pt, static_cast<int>(blocks), k, static_cast<int64_t *>(cnt.p));
+        members_across<<<1, kSortThreads, 0, s>>>(static_cast<int64_t *>(cnt.p), k, start, static_cast<float *>(dd.p),
+                                                  m, static_cast<KmeansState *>(state.p));
+        members_place<<<static_cast<unsigned>(blocks), kSortThreads, 0, s>>>(asg, m, per, k, pt, start, order);
+        list_means(X, dim, k, start, order, d_centroids, s);
+        CK(cudaGetLastError());
+        CK(cudaMemcpyAsync(&h, state.p, sizeof(h), cudaMemcpyDeviceToHost, s));
         CK(cudaStreamSynchronize(s));
-        double obj = 0.0;
-        for (int64_t i = 0; i < m; ++i)
-            obj += dist[i];
         if (objective)
-            objective[it] = obj;
-        // members of each centroid in row order (counting sort)
-        std::fill(start.begin(), start.end(), 0);
-        for (int64_t i = 0; i < m; ++i)
-            start[asg[i] + 1]++;
-        for (int j = 0; j < k; ++j)
-            start[j + 1] += start[j];
-        std::vector<int64_t> fill(start.begin(), start.end() - 1);
-        for (int64_t i = 0; i < m; ++i)
-            order[fill[asg[i]]++] = i;
-        CK(cudaMemcpyAsync(ord.p, order.data(), m * 8, cudaMemcpyHostToDevice, s));
-        CK(cudaMemcpyAsync(st.p, start.data(), (k + 1) * 8, cudaMemcpyHostToDevice, s));
-        centroid_update<float><<<k, 128, 0, s>>>(X, dim, static_cast<int64_t *>(ord.p),
-                                                 static_cast<int64_t *>(st.p), d_centroids);
+            objective[it] = h.objective;
         // empty centroids move onto the rows farthest from their centroid
         // (larger distance first, smaller row on ties), each row used once
-        std::vector<int32_t> empty;
-        for (int j = 0; j < k; ++j)
-            if (start[j] == start[j + 1])
-                empty.push_back(j);
-        if (!empty.empty()) {
+        if (h.empty > 0) {
+            std::vector<float> dist(m);
+            std::vector<int64_t> count(k);
+            CK(cudaMemcpyAsync(dist.data(), dd.p, m * 4, cudaMemcpyDeviceToHost, s));
+            CK(cudaMemcpyAsync(count.data(), cnt.p, static_cast<size_t>(k) * 8, cudaMemcpyDeviceToHost, s));
+            CK(cudaStreamSynchronize(s));
+            std::vector<int32_t> empty;
+            for (int j = 0; j < k; ++j)
+                if (count[j] == 0)
+                    empty.push_back(j);
             std::vector<int64_t> idx(m);
             std::iota(idx.begin(), idx.end(), 0);
             std::stable_sort(idx.begin(), idx.end(), [&](int64_t a, int64_t b) { return dist[a] > dist[b]; });
@@ -250,8 +359,8 @@ ann_status ann_kmeans(const void *d_x, int64_t n, int32_t dim, int32_t dtype, co
             set_centroid_rows<float><<<static_cast<unsigned>(empty.size()), 128, 0, s>>>(
                 X, dim, static_cast<int64_t *>(srows.p), static_cast<int32_t *>(which.p),
                 static_cast<int>(empty.size()), d_centroids);
+            CK(cudaStreamSynchronize(s));  // host vectors are reused next iteration
         }
-        CK(cudaStreamSynchronize(s));  // host vectors are reused next iteration
     }
     CK(cudaStreamSynchronize(s));
     return ANN_OK;
