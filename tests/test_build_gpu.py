@@ -170,3 +170,20 @@ def test_knn_edges_exact(n, nq, d, k, dtype, metric, self_):
                         exclude=np.arange(n) if self_ else None)
     assert np.array_equal(ids, oi)
     assert np.array_equal(dd.astype(np.float64)[oi >= 0], od[oi >= 0])
+
+
+@pytest.mark.parametrize("n,dim,K,R,dtype", [(300, 16, 5, 3, "f32"), (1_001, 384, 64, 64, "f32"), (257, 960, 20, 7, "f32"),
+                                             (2_500, 48, 128, 33, "u8"), (66, 16, 64, 32, "u8")])
+def test_graph_edges_match_oracle(n, dim, K, R, dtype):
+    # candidate counts that are no multiple of four, rows staged and read in
+    # place, and graphs that fall apart (four separated groups), so that the
+    # repair has nodes to attach; whole numbers make every decision exact
+    rng = np.random.default_rng(dim)
+    lo, hi = (0, 40) if dtype == "u8" else (-3, 4)
+    base = rng.integers(lo, hi, size=(n, dim))
+    base[:, 0] += (np.arange(n) % 4) * (50 if dtype == "u8" else 400)
+    base = base.astype(np.uint8 if dtype == "u8" else np.float32)
+    g, med, rep = _graph_gpu(base, K, R)
+    og, orep = oracle.build_graph(base, K=K, R=R, alpha=1.0)
+    assert np.array_equal(g, og) and rep == orep
+    assert med == oracle.medoid(base)
