@@ -146,8 +146,11 @@ def kernel_digest():
     import hashlib
     import re
     h = hashlib.sha1()
-    for rel in ("paper_2506_15986_gb300/csrc/search.cu", "paper_2506_15986_gb300/csrc/device_util.cuh",
-                "paper_2506_15986_gb300/csrc/internal.h", "include/ann.h"):
+    for rel in ("paper_2506_15986_gb300/csrc/search.cu", "paper_2506_15986_gb300/csrc/search_kernel.cuh",
+                "paper_2506_15986_gb300/csrc/device_util.cuh", "paper_2506_15986_gb300/csrc/internal.h",
+                "include/ann.h"):
+        if not os.path.exists(os.path.join(ROOT, rel)):
+            continue
         with open(os.path.join(ROOT, rel), encoding="utf-8") as f:
             src = f.read()
         src = re.sub(r"/\*.*?\*/", " ", src, flags=re.S)

@@ -1,0 +1,10 @@
+// search_f16.cu -- instances of the search kernel (one file per group of storage
+// types, so that they compile side by side).
+#include "search_kernel.cuh"
+
+namespace ann {
+
+ANN_SEARCH_INSTANCE(, ANN_F16, ANN_L2)
+ANN_SEARCH_INSTANCE(, ANN_F16, ANN_IP)
+
+}  // namespace ann

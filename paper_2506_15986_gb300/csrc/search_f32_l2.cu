@@ -1,0 +1,9 @@
+// search_f32_l2.cu -- instances of the search kernel (one file per group of storage
+// types, so that they compile side by side).
+#include "search_kernel.cuh"
+
+namespace ann {
+
+ANN_SEARCH_INSTANCE(, ANN_F32, ANN_L2)
+
+}  // namespace ann

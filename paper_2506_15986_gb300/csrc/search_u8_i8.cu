@@ -1,0 +1,11 @@
+// search_u8_i8.cu -- instances of the search kernel (one file per group of storage
+// types, so that they compile side by side).
+#include "search_kernel.cuh"
+
+namespace ann {
+
+ANN_SEARCH_INSTANCE(, ANN_U8, ANN_L2)
+ANN_SEARCH_INSTANCE(, ANN_I8S, ANN_L2)
+ANN_SEARCH_INSTANCE(, ANN_I8S, ANN_IP)
+
+}  // namespace ann
