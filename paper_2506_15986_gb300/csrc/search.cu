@@ -344,7 +344,7 @@ ann_status launch_search(ann_index *idx, const SearchLaunch &L, cudaStream_t s)
             a.stage_rows = (a.stage_rows + 3) / 4 * 4;  // whole groups of four
         size_t off = 16;  // mbarrier
         a.off_sel = static_cast<int>(off);
-        off = align_up(off + 4 * 2 * ANN_MAX_W, 16);  // selected and predicted ids
+        off = align_up(off + 4 * 3 * ANN_MAX_W, 16);  // the selection: pool indices, ids, sources
         a.off_q = static_cast<int>(off);
         off = align_up(off + L.qbytes + a.qpad, 16);
         if (a.gather4)

@@ -492,7 +492,8 @@ __global__ void __launch_bounds__(32 * kMaxSearchWarps, 16) beam_search_kernel(c
         int level = shared_tab ? 0 : 1, used = 0, gbits = qbits;
         int limit = shared_tab ? hlimit : (1 << qbits) * 3 / 4;
         uint32_t *gtab = gtab1;
-        int32_t *pred = sel + ANN_MAX_W;  // predicted ids of the next selection
+        int32_t *pred = sel + ANN_MAX_W;     // ids of the next selection
+        int32_t *src = sel + 2 * ANN_MAX_W;  // where they come from
         int npred = 0;
         int32_t nxt[NS];  // their adjacency rows, lane-distributed like cur[]
 #pragma unroll
@@ -598,72 +599,99 @@ __global__ void __launch_bounds__(32 * kMaxSearchWarps, 16) beam_search_kernel(c
                 }
                 __syncwarp();
                 if (m > 0) {
-                    if (NS == 1 || m <= 32 || (m <= 64 && nc > 64)) {
-                        // compact the survivors into cbuf[0, m) (a 64-key
-                        // sort of candidates that all sit in slots 0-1 needs
-                        // none: the dropped ones sort to the end)
-                        int base = 0;
+                    // up to 32 survivors: a survivor's place is the number of
+                    // smaller ones, counted over broadcasts that do not wait
+                    // for one another (a bitonic network's stages do)
+                    if (NS == 1) {
+                        int place = 0;
+                        for (unsigned todo = bm[0]; todo; todo &= todo - 1)
+                            place += __shfl_sync(kFull, kk[0], __ffs(todo) - 1) < kk[0];
+                        if (kk[0] != kKeyMax)
+                            cbuf[place] = kk[0];
+                    } else {
+                        if (m <= 32 || (m <= 64 && nc > 64)) {
+                            // compact the survivors into cbuf[0, m) (a 64-key
+                            // sort of candidates that all sit in slots 0-1 needs
+                            // none: the dropped ones sort to the end)
+                            int base = 0;
 #pragma unroll
-                        for (int s = 0; s < NS; ++s) {
-                            if (kk[s] != kKeyMax)
-                                cbuf[base + __popc(bm[s] & lanemask_lt())] = kk[s];
-                            base += __popc(bm[s]);
+                            for (int s = 0; s < NS; ++s) {
+                                if (kk[s] != kKeyMax)
+                                    cbuf[base + __popc(bm[s] & lanemask_lt())] = kk[s];
+                                base += __popc(bm[s]);
+                            }
+                            __syncwarp();
+                            kk[0] = lane < m ? cbuf[lane] : kKeyMax;
+                            if constexpr (NS > 1)
+                                kk[1] = lane + 32 < m ? cbuf[lane + 32] : kKeyMax;
+                            __syncwarp();
                         }
-                        __syncwarp();
-                        kk[0] = lane < m ? cbuf[lane] : kKeyMax;
-                        if constexpr (NS > 1)
-                            kk[1] = lane + 32 < m ? cbuf[lane + 32] : kKeyMax;
-                        __syncwarp();
-                    }
-                    if (NS == 1 || m <= 32) {
-                        // sort over the next power of two only
-                        int width = 1;
-                        while (width < m)
-                            width <<= 1;
-                        kk[0] = warp_sort_lanes(kk[0], lane, width);
-                        cbuf[lane] = kk[0];
-                    } else if constexpr (NS > 1) {
-                        if (NS == 2 || m <= 64) {
-                            uint64_t k2[2] = {kk[0], kk[1]};
-                            warp_sort_rolled<2>(k2, lane);
-                            cbuf[lane] = k2[0];
-                            cbuf[lane + 32] = k2[1];
-                        } else if constexpr (NS == 4) {
-                            warp_sort_rolled<4>(kk, lane);
+                        if (m <= 32) {
+                            int place = 0;
+                            for (int s = 0; s < m; s += 4) {
 #pragma unroll
-                            for (int s = 0; s < NS; ++s)
-                                cbuf[lane + 32 * s] = kk[s];
+                                for (int u = 0; u < 4; ++u)
+                                    place += __shfl_sync(kFull, kk[0], s + u) < kk[0];
+                            }
+                            if (lane < m)
+                                cbuf[place] = kk[0];
+                        } else if constexpr (NS > 1) {
+                            if (NS == 2 || m <= 64) {
+                                uint64_t k2[2] = {kk[0], kk[1]};
+                                warp_sort_rolled<2>(k2, lane);
+                                cbuf[lane] = k2[0];
+                                cbuf[lane + 32] = k2[1];
+                            } else if constexpr (NS == 4) {
+                                warp_sort_rolled<4>(kk, lane);
+#pragma unroll
+                                for (int s = 0; s < NS; ++s)
+                                    cbuf[lane + 32 * s] = kk[s];
+                            }
                         }
                     }
                     __syncwarp();
                 }
             }
 
-            // ---- predict the next selection: the W smallest unexpanded keys
-            // among the pool and the survivors.  Their adjacency rows are
+            // ---- the next selection: the W smallest unexpanded keys among the
+            // pool and the survivors, in order.  Their adjacency rows are
             // loaded now, so the loads overlap the merge.
+            int from = 0;  // lane r < npred: the r-th one's pool index, or ~j for survivor j
             {
                 int nf = 0;
                 for (int i0 = cursor; i0 < cnt && nf < a.W; i0 += 32) {
                     const int i = i0 + lane;
-                    const bool un = i < cnt && !(pool[i] & 1ull);
+                    const uint64_t v = i < cnt ? pool[i] : 1ull;
+                    const bool un = !(v & 1ull);
                     const unsigned um = __ballot_sync(kFull, un);
                     const int g = nf + __popc(um & lanemask_lt());
-                    if (un && g < a.W)
-                        ptop[g] = pool[i];
+                    if (un && g < a.W) {
+                        ptop[g] = v;
+                        sel[g] = i;
+                    }
                     nf = min(a.W, nf + __popc(um));
                 }
                 __syncwarp();
-                const int mw = min(m, a.W);
-                int i = 0, j = 0, np = 0;
-                for (; np < a.W && (i < nf || j < mw); ++np) {
-                    const bool from_pool = j >= mw || (i < nf && ptop[i] < cbuf[j]);
-                    const uint64_t v = from_pool ? ptop[i++] : cbuf[j++];
-                    if (lane == 0)
-                        pred[np] = key_id(v);
+                // lane l < nf places the pool's l-th, lane ANN_MAX_W + j the
+                // survivors' j-th: its own index plus the other side's smaller ones
+                const int mw = min(m, a.W), np = min(a.W, nf + mw);
+                const bool mine = lane < ANN_MAX_W;
+                const int own = mine ? lane : lane - ANN_MAX_W, other = mine ? mw : nf;
+                if (own < (mine ? nf : mw)) {
+                    const uint64_t *theirs = mine ? cbuf : ptop;
+                    const uint64_t v = mine ? ptop[own] : cbuf[own];
+                    int r = own;
+#pragma unroll
+                    for (int j = 0; j < ANN_MAX_W; ++j)
+                        r += j < other && theirs[j] < v;
+                    if (r < a.W) {
+                        pred[r] = key_id(v);
+                        src[r] = mine ? sel[own] : ~own;
+                    }
                 }
                 npred = np;
                 __syncwarp();
+                from = lane < np ? src[lane] : 0;
                 const int tp = npred * a.R;
 #pragma unroll
                 for (int r = 0; r < NS; ++r) {
@@ -677,6 +705,7 @@ __global__ void __launch_bounds__(32 * kMaxSearchWarps, 16) beam_search_kernel(c
             // survivors' ranks come from the unmodified pool; pool entries move
             // right by the number of smaller survivors, 32 at a time from the
             // back, so that none is overwritten before it is read
+            int dst0 = Lq;  // lane j < 32: survivor j's place in the pool
             if (m > 0) {
                 int dst[NS];
 #pragma unroll
@@ -685,6 +714,7 @@ __global__ void __launch_bounds__(32 * kMaxSearchWarps, 16) beam_search_kernel(c
                     dst[r] = j < m ? j + count_less(pool, cnt, cbuf[j]) : Lq;
                 }
                 const int p0 = __shfl_sync(kFull, dst[0], 0);  // rank of the best survivor
+                dst0 = dst[0];
                 __syncwarp();
                 for (int b = cnt > p0 ? p0 + (cnt - 1 - p0) / 32 * 32 : p0 - 32; b >= p0; b -= 32) {
                     const int i = b + lane;
@@ -710,45 +740,27 @@ __global__ void __launch_bounds__(32 * kMaxSearchWarps, 16) beam_search_kernel(c
             if (found)
                 break;
 
-            // ---- select the first W unexpanded pool entries; mark them expanded
-            int ns = 0, first = -1;
-            for (int i0 = cursor; i0 < cnt && ns < a.W; i0 += 32) {
-                const int i = i0 + lane;
-                const bool un = i < cnt && !(pool[i] & 1ull);
-                const unsigned um = __ballot_sync(kFull, un);
-                if (um) {
-                    if (first < 0)
-                        first = i0 + __ffs(um) - 1;
-                    const int g = ns + __popc(um & lanemask_lt());
-                    if (un && g < a.W) {
-                        const uint64_t v = pool[i];
-                        pool[i] = v | 1ull;
-                        sel[g] = key_id(v);
-                    }
-                    ns = min(a.W, ns + __popc(um));
-                }
-            }
-            __syncwarp();
+            // ---- mark the selected entries expanded where they are now: a pool
+            // entry moved right by the survivors before it, all of them selected
+            // too; one that the pool's end cut off takes the later ones with it
+            const unsigned late = __ballot_sync(kFull, lane < npred && from < 0);
+            const int at_dst = __shfl_sync(kFull, dst0, from < 0 ? ~from : 0);
+            const int pos = from < 0 ? at_dst : from + __popc(late & lanemask_lt());
+            const bool take = lane < npred && pos < Lq;
+            if (take)
+                pool[pos] |= 1ull;
+            const int ns = __popc(__ballot_sync(kFull, take));
             if (ns == 0)
                 break;
-            cursor = first;
+            cursor = __shfl_sync(kFull, pos, 0);
             hops += ns;
 
-            // ---- adjacency rows of the selected entries: the predicted ones,
-            // unless truncation to L dropped a predicted entry (then loaded now)
             const int total = ns * a.R;
-            bool hit = ns == npred;
-            for (int s = 0; s < ns && hit; ++s)
-                hit = sel[s] == pred[s];
             int32_t cur[NS];
 #pragma unroll
-            for (int r = 0; r < NS; ++r) {
-                const int t = lane + 32 * r;
-                cur[r] = hit ? nxt[r]
-                             : (t < total ? __ldg(a.graph + static_cast<int64_t>(sel[(t * a.R_inv) >> 16]) * a.R +
-                                                   (t - ((t * a.R_inv) >> 16) * a.R))
-                                          : -1);
-            }
+            for (int r = 0; r < NS; ++r)
+                cur[r] = nxt[r];
+            __syncwarp();
 
             // ---- neighbours of the selected entries: visited test, compaction
             // A table that would pass 3/4 load hands its keys to the next,
