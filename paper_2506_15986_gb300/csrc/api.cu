@@ -6,6 +6,8 @@
 #include <stdio.h>
 #include <string.h>
 
+#include <algorithm>
+#include <mutex>
 #include <new>
 #include <vector>
 
@@ -60,6 +62,53 @@ void scratch_free(ann_index *idx, void *p, cudaStream_t s)
 
 namespace {
 
+constexpr int kMaxDevices = 64;
+constexpr uint64_t kBuilderKeep = uint64_t{1} << 30;  // bytes a builder pool keeps between calls
+std::mutex g_builder_mu;
+cudaMemPool_t g_builder_pool[kMaxDevices] = {};
+
+// the current device's pool, made on first use (null: none can be made)
+cudaMemPool_t builder_pool(bool make)
+{
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices)
+        return nullptr;
+    std::lock_guard<std::mutex> lock(g_builder_mu);
+    if (!g_builder_pool[dev] && make) {
+        cudaMemPoolProps props = {};
+        props.allocType = cudaMemAllocationTypePinned;
+        props.location.type = cudaMemLocationTypeDevice;
+        props.location.id = dev;
+        cudaMemPool_t p = nullptr;
+        uint64_t keep = kBuilderKeep;
+        if (cudaMemPoolCreate(&p, &props) == cudaSuccess) {
+            if (cudaMemPoolSetAttribute(p, cudaMemPoolAttrReleaseThreshold, &keep) == cudaSuccess)
+                g_builder_pool[dev] = p;
+            else
+                cudaMemPoolDestroy(p);
+        }
+        cudaGetLastError();
+    }
+    return g_builder_pool[dev];
+}
+
+}  // namespace
+
+cudaError_t builder_alloc(void **p, size_t bytes, cudaStream_t s)
+{
+    bytes = std::max<size_t>(bytes, 16);
+    cudaMemPool_t pool = builder_pool(true);
+    return pool ? cudaMallocFromPoolAsync(p, bytes, pool, s) : cudaMallocAsync(p, bytes, s);
+}
+
+void builder_trim()
+{
+    if (cudaMemPool_t pool = builder_pool(false))
+        cudaMemPoolTrimTo(pool, 0);
+}
+
+namespace {
+
 __global__ void count_bad_ids(const int32_t *g, int64_t total, int64_t n, unsigned long long *bad)
 {
     for (int64_t i = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x; i < total;
@@ -98,6 +147,7 @@ void destroy(ann_index *idx)
     if (idx->pool)
         cudaMemPoolDestroy(idx->pool);
     delete idx;
+    builder_trim();
 }
 
 // 64-bit FNV-1a

@@ -411,7 +411,7 @@ struct DevBuf {
     cudaError_t alloc(size_t count, cudaStream_t st)
     {
         s = st;
-        return cudaMallocAsync(reinterpret_cast<void **>(&p), count * sizeof(T), st);
+        return builder_alloc(reinterpret_cast<void **>(&p), count * sizeof(T), st);
     }
     ~DevBuf()
     {

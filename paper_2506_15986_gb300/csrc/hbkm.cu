@@ -629,7 +629,7 @@ struct Buf {
     void *p = nullptr;
     cudaStream_t s;
     explicit Buf(cudaStream_t st) : s(st) {}
-    cudaError_t alloc(size_t bytes) { return cudaMallocAsync(&p, std::max<size_t>(bytes, 16), s); }
+    cudaError_t alloc(size_t bytes) { return builder_alloc(&p, bytes, s); }
     template <typename T>
     T *as() const
     {

@@ -875,7 +875,7 @@ struct Scratch {
     void *p = nullptr;
     cudaStream_t s;
     explicit Scratch(cudaStream_t st) : s(st) {}
-    cudaError_t alloc(size_t bytes) { return cudaMallocAsync(&p, std::max<size_t>(bytes, 16), s); }
+    cudaError_t alloc(size_t bytes) { return builder_alloc(&p, bytes, s); }
     template <typename T>
     T *as() const
     {

@@ -247,7 +247,7 @@ struct Scoped {
     void *p = nullptr;
     cudaStream_t s;
     explicit Scoped(cudaStream_t st) : s(st) {}
-    cudaError_t alloc(size_t bytes) { return cudaMallocAsync(&p, std::max<size_t>(bytes, 16), s); }
+    cudaError_t alloc(size_t bytes) { return builder_alloc(&p, bytes, s); }
     ~Scoped()
     {
         if (p)

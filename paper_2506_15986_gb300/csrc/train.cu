@@ -582,6 +582,7 @@ void trainer_free(ann_trainer *t)
         cudaFree(p);
     fusion_free(t->fu);
     delete t;
+    builder_trim();
 }
 
 // one Adam step over every parameter block
