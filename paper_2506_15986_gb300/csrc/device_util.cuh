@@ -137,8 +137,6 @@ __device__ __forceinline__ int32_t key_id(uint64_t k)
     return static_cast<int32_t>((static_cast<uint32_t>(k)) >> 1);
 }
 
-__device__ __forceinline__ uint64_t key_plain(uint64_t k) { return k & ~1ull; }
-
 // ---- warp bitonic sorts (ascending) ------------------------------------------
 
 __device__ __forceinline__ uint64_t kmin(uint64_t a, uint64_t b) { return a < b ? a : b; }
@@ -154,22 +152,6 @@ __device__ __forceinline__ uint64_t warp_sort32(uint64_t k, int lane)
             uint64_t o = __shfl_xor_sync(kFull, k, j);
             bool lower = (lane & j) == 0;
             bool asc = (lane & kk) == 0;
-            k = (lower == asc) ? kmin(k, o) : kmax(k, o);
-        }
-    }
-    return k;
-}
-
-// Keys of lanes [0, width) sorted ascending (width a power of two <= 32);
-// lanes at or above width exchange only among themselves.  The whole warp
-// must call it.
-__device__ __forceinline__ uint64_t warp_sort_lanes(uint64_t k, int lane, int width)
-{
-    for (int kk = 2; kk <= width; kk <<= 1) {
-        for (int j = kk >> 1; j > 0; j >>= 1) {
-            const uint64_t o = __shfl_xor_sync(kFull, k, j);
-            const bool lower = (lane & j) == 0;
-            const bool asc = (lane & kk) == 0;
             k = (lower == asc) ? kmin(k, o) : kmax(k, o);
         }
     }
@@ -200,42 +182,9 @@ __device__ __forceinline__ void warp_sort64(uint64_t &k0, uint64_t &k1, int lane
     }
 }
 
-// NPL*32 keys, NPL per lane: element r*32+lane lives in k[r].  NPL is a power of 2.
-template <int NPL>
-__device__ __forceinline__ void warp_sort_n(uint64_t (&k)[NPL], int lane)
-{
-    constexpr int N = NPL * 32;
-#pragma unroll
-    for (int kk = 2; kk <= N; kk <<= 1) {
-#pragma unroll
-        for (int j = kk >> 1; j > 0; j >>= 1) {
-            if (j >= 32) {
-                const int rj = j >> 5;
-#pragma unroll
-                for (int r = 0; r < NPL; ++r) {
-                    if ((r & rj) == 0) {
-                        const bool asc = ((r * 32 + lane) & kk) == 0;
-                        const uint64_t a = k[r], b = k[r | rj];
-                        k[r] = asc ? kmin(a, b) : kmax(a, b);
-                        k[r | rj] = asc ? kmax(a, b) : kmin(a, b);
-                    }
-                }
-            } else {
-#pragma unroll
-                for (int r = 0; r < NPL; ++r) {
-                    const uint64_t o = __shfl_xor_sync(kFull, k[r], j);
-                    const bool lower = (lane & j) == 0;
-                    const bool asc = ((r * 32 + lane) & kk) == 0;
-                    k[r] = (lower == asc) ? kmin(k[r], o) : kmax(k[r], o);
-                }
-            }
-        }
-    }
-}
-
-// warp_sort_n with rolled stage loops: a few dozen instructions instead of
-// hundreds, for kernels whose warps run out of step and share one instruction
-// cache.  NPL is 2 or 4.
+// NPL*32 keys, NPL (2 or 4) per lane: element r*32+lane lives in k[r].  The
+// stage loops are rolled: a few dozen instructions instead of hundreds, for
+// kernels whose warps run out of step and share one instruction cache.
 template <int NPL>
 __device__ __forceinline__ void warp_sort_rolled(uint64_t (&k)[NPL], int lane)
 {
@@ -269,31 +218,23 @@ __device__ __forceinline__ void warp_sort_rolled(uint64_t (&k)[NPL], int lane)
     }
 }
 
-// number of entries of the sorted array a[0..len) whose plain key is < v
-__device__ __forceinline__ int count_less(const uint64_t *a, int len, uint64_t v)
+// number of entries of the sorted array a[0..len) that are < v, by thirds of
+// three loads that do not wait for one another (a binary search waits for each
+// of its twice as many)
+__device__ __forceinline__ int count_less4(const uint64_t *a, int len, uint64_t v)
 {
-    int lo = 0, hi = len;
-    while (lo < hi) {
-        int mid = (lo + hi) >> 1;
-        if (key_plain(a[mid]) < v)
-            lo = mid + 1;
-        else
-            hi = mid;
+    int lo = 0, n = len;
+    while (n > 3) {
+        const int q = n >> 2;
+        const uint64_t x1 = a[lo + q], x2 = a[lo + 2 * q], x3 = a[lo + 3 * q];
+        const int c = (x1 < v) + (x2 < v) + (x3 < v);
+        // c of the three are below: the count lies after the c-th of them
+        n = c == 0 ? q : c == 3 ? n - 3 * q - 1 : q - 1;
+        lo += c == 0 ? 0 : c * q + 1;
     }
-    return lo;
-}
-
-// number of entries of the sorted array a[0..len) that are < v (full keys)
-__device__ __forceinline__ int count_less_raw(const uint64_t *a, int len, uint64_t v)
-{
-    int lo = 0, hi = len;
-    while (lo < hi) {
-        int mid = (lo + hi) >> 1;
-        if (a[mid] < v)
-            lo = mid + 1;
-        else
-            hi = mid;
-    }
+#pragma unroll
+    for (int i = 0, l = lo; i < 3; ++i)
+        lo += i < n && a[l + i] < v;
     return lo;
 }
 

@@ -386,3 +386,30 @@ def test_tables_sized_by_each_querys_own_L(hash_bits):
     assert st == ann.OK
     assert (oe[Ls == 76] > 3_072).any()
     assert np.array_equal(ids, oi[:, :10]) and np.array_equal(ev, oe) and np.array_equal(hp, oh)
+
+
+@pytest.mark.parametrize("dtype", [np.float32, np.float16])
+@pytest.mark.parametrize("metric", [ann.L2, ann.IP])
+@pytest.mark.parametrize("dim,team", [(72, 0), (104, 0), (128, 0), (136, 0), (200, 0), (256, 0), (256, 8), (128, 4), (256, 32), (8, 0)])
+def test_distance_forms_are_bit_identical(dtype, metric, dim, team):
+    # rows read one by one are summed by fewer lanes than the team has (two or
+    # four members in turn or together, by the row's chunks and the type);
+    # tensor gathers always take one lane a member: the same bits either way,
+    # for every step width and the last, ragged round
+    rng = np.random.default_rng(dim + team)
+    n = 3_000
+    if dtype == np.float16:
+        dim *= 2
+    base = rng.standard_normal((n, dim)).astype(dtype)
+    q = rng.standard_normal((150, dim)).astype(np.float32)
+    g = rng.integers(0, n, size=(n, 29)).astype(np.int32)
+    h = make_index(base, g, 5, metric=metric)
+    try:
+        for W in (1, 2, 4):
+            a = search(h, q, 20, 40, W=W, team=team, gather=1)
+            b = search(h, q, 20, 40, W=W, team=team, gather=4)
+            assert a[4] == b[4] == ann.OK
+            for x, y in zip(a[:4], b[:4]):
+                assert np.array_equal(x.view(np.int32), y.view(np.int32))
+    finally:
+        ann.ann_free_index(h)
