@@ -218,17 +218,18 @@ __global__ void __launch_bounds__(128) gemm_kernel(const GemmArgs g, const int e
 }
 
 // Queues one GEMM.  With EPI_STORE and few output tiles over a long reduction
-// K is split over CTAs that add into `out`, which the caller has zeroed.
+// K is split over CTAs, at least min_k columns each, that add into `out`, which
+// the caller has zeroed.
 template <int BN>
-ann_status gemm(const GemmArgs &g, cudaStream_t s, int epi = EPI_STORE)
+ann_status gemm(const GemmArgs &g, cudaStream_t s, int epi = EPI_STORE, int64_t min_k = 512)
 {
     dim3 grid(static_cast<unsigned>((g.M + 127) / 128), static_cast<unsigned>((g.N + BN - 1) / BN));
-    // at least 512 columns of K each, up to about two CTAs per SM
+    // up to about two CTAs per SM
     GemmArgs h = g;
     h.ksplit = 0;
     const int64_t tiles = static_cast<int64_t>(grid.x) * grid.y;
     if (epi == EPI_STORE && tiles < 128 && g.K >= 1024) {
-        const int64_t want = std::min<int64_t>(g.K / 512, std::max<int64_t>(1, 256 / tiles));
+        const int64_t want = std::min<int64_t>(g.K / min_k, std::max<int64_t>(1, 256 / tiles));
         if (want > 1) {
             h.ksplit = ((g.K + want - 1) / want + 63) / 64 * 64;
             grid.z = static_cast<unsigned>((g.K + h.ksplit - 1) / h.ksplit);
@@ -386,6 +387,111 @@ __global__ void infonce_kernel(const float *S, int64_t B, int H, const int32_t *
         dS[r * ldS + c] = __float2bfloat16_rn(g);
     }
     if (threadIdx.x == 0) {
+        row_loss[r] = ok ? -(sp - npos * lse) * inv_np : 0.f;
+        valid[r] = ok ? 1 : 0;
+    }
+}
+
+// infonce_kernel with a warp per row, for up to kRowHubs hubs: no barriers, and
+// up to 1,024 hubs a row's logits are read once into registers.  Every sum runs
+// as the block's does (its thread t = 32 w + lane adds columns t, t + 256, ...;
+// lanes by xor-shuffles; warps 4 apart, 2 apart, 1 apart), so that the
+// logarithm of the partition sum, which decides how dS rounds to BF16, has the
+// same bits.  8,192 rows x 1,024 hubs: 39 us by blocks, 33 us here.
+constexpr int kRowHubs = 8192;
+constexpr int kRowWarps = 8;
+
+template <bool REG>
+__global__ void __launch_bounds__(32 * kRowWarps)
+    infonce_rows_kernel(const float *S, int64_t B, int H, const int32_t *cand, const int8_t *lab, int M,
+                        const int32_t *rowmap, __nv_bfloat16 *dS, int64_t ldS, float *row_loss, int *valid)
+{
+    extern __shared__ int8_t lrow_all[];
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    const int64_t r = blockIdx.x * static_cast<int64_t>(kRowWarps) + wid;
+    if (r >= B)
+        return;
+    const int hp = (H + 15) / 16 * 16;
+    int8_t *lrow = lrow_all + wid * hp;
+    const int64_t mr = rowmap ? rowmap[r] : r;
+    for (int c = lane; c < hp / 16; c += 32)
+        reinterpret_cast<uint4 *>(lrow)[c] = make_uint4(~0u, ~0u, ~0u, ~0u);
+    __syncwarp();
+    for (int j = lane; j < M; j += 32) {
+        const int32_t h = cand[mr * M + j];
+        if (h >= 0 && h < H)
+            lrow[h] = lab[mr * M + j];
+    }
+    __syncwarp();
+    const float *s = S + r * H;
+    constexpr int kReg = REG ? 32 : 1;
+    float sv[kReg];
+    if constexpr (REG) {
+#pragma unroll
+        for (int i = 0; i < 32; ++i)
+            sv[i] = lane + 32 * i < H ? s[lane + 32 * i] : 0.f;
+    }
+    // f(i, c, logit) over the lane's columns c = lane + 32 i < H, eight i at a time
+    auto each = [&](auto f) {
+        if constexpr (REG) {
+#pragma unroll
+            for (int i = 0; i < 32; ++i)
+                if (lane + 32 * i < H)
+                    f(i & 7, lane + 32 * i, sv[i]);
+        } else {
+            for (int i0 = 0; 32 * i0 < H; i0 += 8) {
+#pragma unroll
+                for (int w = 0; w < 8; ++w) {
+                    const int c = lane + 32 * (i0 + w);
+                    if (c < H)
+                        f(w, c, s[c]);
+                }
+            }
+        }
+    };
+    auto add = [&](float (&v)[8]) {
+#pragma unroll
+        for (int w = 0; w < 8; ++w)
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1)
+                v[w] += __shfl_xor_sync(kFull, v[w], o);
+        return ((v[0] + v[4]) + (v[2] + v[6])) + ((v[1] + v[5]) + (v[3] + v[7]));
+    };
+    float mx = -INFINITY;
+    int npos = 0;
+    each([&](int, int c, float x) {
+        const int8_t l = lrow[c];
+        if (l != 0)
+            mx = fmaxf(mx, x);
+        npos += l > 0;
+    });
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1)
+        mx = fmaxf(mx, __shfl_xor_sync(kFull, mx, o));
+    npos = __reduce_add_sync(kFull, npos);
+    float zs[8], ps[8];
+#pragma unroll
+    for (int w = 0; w < 8; ++w)
+        zs[w] = ps[w] = 0.f;
+    each([&](int w, int c, float x) {
+        const int8_t l = lrow[c];
+        if (l != 0)
+            zs[w] += expf(x - mx);
+        if (l > 0)
+            ps[w] += x;
+    });
+    const float z = add(zs), sp = add(ps);
+    const float lse = mx + logf(z);
+    const bool ok = npos > 0;
+    const float inv_np = ok ? 1.f / static_cast<float>(npos) : 0.f;
+    each([&](int, int c, float x) {
+        const int8_t l = lrow[c];
+        float g = 0.f;
+        if (ok && l != 0)
+            g = expf(x - lse) - (l > 0 ? inv_np : 0.f);
+        dS[r * ldS + c] = __float2bfloat16_rn(g);
+    });
+    if (lane == 0) {
         row_loss[r] = ok ? -(sp - npos * lse) * inv_np : 0.f;
         valid[r] = ok ? 1 : 0;
     }
@@ -653,8 +759,14 @@ ann_status trainer_grads(ann_trainer *t, const float *d_queries, const int32_t *
     g.ldo = H;
     if ((st = gemm<128>(g, s)) != ANN_OK)
         return st;
-    infonce_kernel<<<static_cast<unsigned>(B), 256, H, s>>>(t->S, B, H, d_cand, d_lab, n_listed, rows, t->dS, t->ldH,
-                                                             t->row_loss, t->valid);
+    if (H <= kRowHubs) {
+        auto kern = H <= 1024 ? infonce_rows_kernel<true> : infonce_rows_kernel<false>;
+        kern<<<blocks_for(B, kRowWarps), 32 * kRowWarps, kRowWarps * ((H + 15) / 16 * 16), s>>>(
+            t->S, B, H, d_cand, d_lab, n_listed, rows, t->dS, t->ldH, t->row_loss, t->valid);
+    } else {
+        infonce_kernel<<<static_cast<unsigned>(B), 256, H, s>>>(t->S, B, H, d_cand, d_lab, n_listed, rows, t->dS,
+                                                                 t->ldH, t->row_loss, t->valid);
+    }
     finalize_loss_kernel<<<1, 1024, 0, s>>>(t->row_loss, t->valid, B, t->tau, t->loss, t->scale);
     // dq_hat = scale * dS e_hat  (B x 64, K = H)
     g = GemmArgs{};
@@ -679,7 +791,8 @@ ann_status trainer_grads(ann_trainer *t, const float *d_queries, const int32_t *
     g.N = 64;
     g.K = B;
     g.out = t->dEh;
-    if ((st = gemm<64>(g, s)) != ANN_OK)
+    // (sums that no later rounding to BF16 reads are split further)
+    if ((st = gemm<64>(g, s, EPI_STORE, 256)) != ANN_OK)
         return st;
     // through the normalisations
     query_backward_kernel<<<blocks_for(B, 32), 256, 0, s>>>(t->qhat, t->tower.nrm, t->dQ, B, t->dZ2, t->dZ2T, t->ldB,
@@ -700,7 +813,7 @@ ann_status trainer_grads(ann_trainer *t, const float *d_queries, const int32_t *
     g.alpha = 1.f;
     g.out = t->grads + o.W2;
     g.ldo = 64;
-    if ((st = gemm<64>(g, s)) != ANN_OK)
+    if ((st = gemm<64>(g, s, EPI_STORE, 256)) != ANN_OK)
         return st;
     // dZ1 = (dZ2 W2^T) * [Z1 > 0]  (B x 256, K = 64), written transposed, with db1's partial sums
     g = GemmArgs{};
@@ -730,7 +843,7 @@ ann_status trainer_grads(ann_trainer *t, const float *d_queries, const int32_t *
     g.alpha = 1.f;
     g.out = t->grads + o.W1;
     g.ldo = 256;
-    if ((st = gemm<256>(g, s)) != ANN_OK)
+    if ((st = gemm<256>(g, s, EPI_STORE, 256)) != ANN_OK)
         return st;
     return cuda_status(cudaGetLastError());
 }
@@ -752,7 +865,10 @@ ann_status ann_trainer_create(int device, int32_t in_dim, int32_t n_hubs, const 
     if (cudaGetDeviceCount(&ndev) != cudaSuccess || device < 0 || device >= ndev)
         return ANN_ERR_CUDA;
     cudaSetDevice(device);
-    if (cudaFuncSetAttribute(infonce_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, n_hubs) != cudaSuccess)
+    if (cudaFuncSetAttribute(infonce_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxTrainHubs) !=
+            cudaSuccess ||
+        cudaFuncSetAttribute(infonce_rows_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             kRowWarps * kRowHubs) != cudaSuccess)
         return ANN_ERR_CUDA;
     ann_trainer *t = new (std::nothrow) ann_trainer();
     if (!t)

@@ -159,3 +159,27 @@ def test_gradients_match_oracle_at_ragged_sizes(B, D, H):
     for k in ("W1", "b1", "W2", "b2", "E"):
         assert _rel(g[k], ref[k]) <= 8e-3, (k, _rel(g[k], ref[k]))
         assert _cos(g[k], ref[k]) >= 0.99995, (k, _cos(g[k], ref[k]))
+
+
+@pytest.mark.parametrize("H", [64, 1_024, 8_192, 8_193])
+def test_row_losses_on_both_sides_of_the_hub_limits(H):
+    # a row's logits are read by a warp into registers (to 1,024 hubs) or twice
+    # (to 8,192), by a block above; the last column and the last row of a block
+    # of eight are listed, one row has no positive and one lists nothing
+    X, W1, b1, W2, b2, E, mask, rows = _problem(B=203, D=32, H=H, seed=H)
+    mask[rows[5]] = np.minimum(mask[rows[5]], 0)
+    mask[rows[6]] = 0
+    mask[rows[7], H - 1] = 1
+    t = ann.ann_trainer_create(32, W1, b1, W2, b2, E, 203, tau=0.1, lr=1e-3)
+    try:
+        loss = ann.ann_trainer_step(t, torch.from_numpy(X).to(DEV), torch.from_numpy(rows).to(DEV), len(rows),
+                                    *dense_as_listed(mask), apply_update=False)
+        gE = np.zeros_like(E)
+        ann.ann_trainer_get(t, hub_emb=gE, gradients=True)
+    finally:
+        ann.ann_trainer_free(t)
+    bf = ot.bf16_round
+    ref_loss, ref = ot.loss_and_grads(bf(X[rows]), bf(W1), b1.astype(np.float64), bf(W2), b2.astype(np.float64),
+                                      E.astype(np.float64), mask[rows], 0.1)
+    assert abs(loss - ref_loss) <= 1e-4 * abs(ref_loss)
+    assert _rel(gE, ref["E"]) <= 8e-3
