@@ -86,3 +86,22 @@ def test_kmeans_and_hubs_against_oracle():
     ann.ann_assign_hubs(dx, len(x), 128, ann.F32, cent, 64, hubs)
     h_o, _ = oracle.hubs(x, c.astype(np.float64))
     assert (hubs.cpu().numpy() == h_o).mean() >= 0.99
+
+
+@pytest.mark.parametrize("n,dim,k,empty", [(1, 4, 1, 0), (5, 8, 5, 0), (257, 36, 3, 1), (4_099, 128, 65, 3)])
+def test_kmeans_edges(n, dim, k, empty):
+    # one row, as many clusters as rows, clusters that get no row at first
+    # (their initial row is another's) and counts that are no multiple of a
+    # block.  Equal initial rows apart (the first wins), no row is within 1 of a
+    # tie at any step, by the oracle's centroids; a mean of m FP32 values is off
+    # by at most m 2^-24 times the largest
+    rng = np.random.default_rng(n)
+    at = np.arange(n) % (k - empty)
+    x = (rng.uniform(-20, 20, (k, dim))[at] + rng.uniform(-1, 1, (n, dim))).astype(np.float32)
+    init = np.concatenate([np.arange(k - empty), np.zeros(empty)]).astype(np.int32)
+    cent = torch.empty((k, dim), dtype=torch.float32, device=DEV)
+    obj = ann.ann_kmeans(torch.from_numpy(x).to(DEV), n, dim, ann.F32, np.arange(n), k, init, 3, cent)
+    cent_o, _, obj_o = oracle.kmeans(x, k, init, 3)
+    m = np.bincount(at).max()
+    assert np.abs(cent.cpu().numpy() - cent_o).max() <= m * 2.0**-24 * np.abs(x).max()
+    np.testing.assert_allclose(obj, obj_o, rtol=1e-4, atol=1e-6)
