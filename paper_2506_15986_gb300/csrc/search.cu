@@ -208,20 +208,25 @@ __global__ void __launch_bounds__(32 * kRerankWarps)
 size_t align_up(size_t v, size_t a) { return (v + a - 1) / a * a; }
 
 // The distance form of a launch: `chunks` 16-byte chunks of a row, a team of G
-// lanes.  Against one lane a team lane: 4 G chunks of G = 8 as two members in
-// turn: 1,835 -> 1,700 us (10,000 queries, d = 128 fp32); other rows of G = 8 as two
-// together: 31.6 -> 31.0 ms (100,000, d = 96 fp32); G = 16 or, in fp32, 32 as four
-// together: 4.41 -> 3.98 ms (10,000, d = 200 fp32).  16-bit rows of G = 32 lose by it
-// (960 coordinates: 4 %).
+// lanes.  One lane a team lane and a row at a time, against here (us, queries):
+// 4 G chunks of G = 8 as two lanes in turn: 1,835 -> 1,700 (10,000, d = 128 fp32);
+// the other rows of eight lanes or more several at once, so that their chains of
+// shared-memory loads and sums overlap: fp32 by twos up to G = 8 (10,000, d = 96:
+// 824 -> 784; by fours 100,000 of them lose 7 %), by fours above (10,000, d = 384:
+// 2,030 -> 1,389, by twos 1,529; 1,000, d = 960: 1,051 by twos, 978); 16-bit and int8
+// rows by twos (3,000, d = 960 fp16: 1,738 -> 1,383; by fours registers spill:
+// 1,397, and 1,209 -> 1,412 at d = 200).  Teams of four gain nothing (d = 128
+// fp16: 1,040, 1,034; uint8: 792, 795).
 int search_form(int dtype, int chunks, int G, bool gather4)
 {
-    if (dtype == ANN_U8 || dtype == ANN_I8S)
+    if (dtype == ANN_U8)
         return kOne;
-    if (!gather4 && G == 8 && chunks == 4 * G)
-        return kPair4;
-    if (!gather4 && dtype == ANN_F32 && G >= 8)
-        return G == 8 ? kPair : kQuad;
-    return chunks == 8 * G ? kOne8 : kOne;
+    if (!gather4 && G >= 8) {
+        if (G == 8 && chunks == 4 * G && dtype != ANN_I8S)
+            return kPair4;
+        return dtype == ANN_F32 && G > 8 ? kRows4 : kRows2;
+    }
+    return dtype != ANN_I8S && chunks == 8 * G ? kOne8 : kOne;
 }
 
 // Bytes of L2 the first-level visited tables may keep resident on the
@@ -329,13 +334,13 @@ ann_status launch_search(ann_index *idx, const SearchLaunch &L, cudaStream_t s)
     a.gather4 = (p->gather == 4 && idx->has_row_map) ? 1 : 0;
     if (a.gather4)
         a.row_map = idx->row_map;
-    // Lanes per distance: where it pays, four or eight lanes stand for the
-    // team, so that a round's rows take fewer passes and shuffles; the
-    // distances are bit for bit those of G lanes.  Tensor gathers write rows
-    // back to back, where few lanes a row would meet bank conflicts: they keep G
-    // lanes.
+    // Lanes per distance: where it pays, four lanes stand for a team of eight, or a
+    // team takes several rows at once, so that a round's rows take fewer passes
+    // and shuffles; the distances are bit for bit those of G lanes a row.  Tensor
+    // gathers write rows back to back, where few lanes a row or neighbouring
+    // rows at once would meet bank conflicts: they keep G lanes a row.
     const int form = search_form(idx->dtype, chunks, G, a.gather4);
-    const int P = idx->dtype == ANN_U8 && !a.gather4 ? std::min(G, 4) : G / form_members(form);
+    const int P = idx->dtype == ANN_U8 && !a.gather4 ? std::min(G, 4) : form == kPair4 ? G / 2 : G;
     a.team_lg = 0;
     while ((1 << a.team_lg) < P)
         ++a.team_lg;

@@ -206,24 +206,45 @@ __device__ __forceinline__ void migrate_keys(const uint32_t *src, int sbits, boo
     __syncwarp();
 }
 
-// One lane's part of the distance of a staged row to the query, for V members
-// of a team of G lanes: member v (team lane `first` + v P) sums the row's
-// 16-byte chunks first + v P, + G, + 2 G, ... into accumulators of its own, and
-// the V sums are added in the order of the team's xor-shuffles (G/2 first).
-// CPL > 0 (V = 1): exactly CPL chunks, unrolled so that their shared-memory
-// loads issue back to back; CPL = 0: any count.  int8 rows: the sum before the
-// scale (inner product), codes from byte 16.
-template <int DT, int MT, int V, int CPL>
-__device__ __forceinline__ auto lane_sum(const uint8_t *row, const uint8_t *q, int chunks, int first, int P, int G)
-{
-    static_assert(V == 1 || V == 2 || V == 4, "members summed together");
-    if constexpr (DT == ANN_U8) {
-        const uint4 *x4 = reinterpret_cast<const uint4 *>(row);
-        const uint4 *q4 = reinterpret_cast<const uint4 *>(q);
-        uint32_t acc = 0;
-        auto chunk = [&](int c) {
-            const uint4 x = x4[c], y = q4[c];
-            uint32_t d;
+// A running sum over 16-byte chunks of a row against the query's coordinates of
+// the same chunk, as every distance form adds them.  int8 rows: chunks of codes
+// (from byte 16 on), x_j = scale * code_j.  L2: the sum of (q_j - scale *
+// code_j)^2, each difference from one fused multiply-add; IP: the sum of q_j
+// code_j, to be scaled.  (The query buffer is zero beyond dim, where the codes
+// are zero too.)
+template <int DT, int MT>
+struct RowSum {
+    // four FP32 accumulators (coordinates 4c+0..3) held as two packed pairs:
+    // each f32x2 operation rounds both halves exactly as the scalar operations
+    // would, at half the instruction count, and the two pairs are independent
+    // dependency chains
+    uint64_t a = 0, b = 0;  // (0.f, 0.f)
+    float scale, c0 = 0.f, c1 = 0.f;  // int8 rows: their scale, and two accumulators
+
+    __device__ __forceinline__ void add4(float x0, float x1, float x2, float x3, float4 y)
+    {
+        if constexpr (MT == ANN_L2)
+            asm("{\n\t.reg .b64 x, y, d;\n\t"
+                "mov.b64 x, {%2, %3};\n\tmov.b64 y, {%6, %7};\n\t"
+                "sub.rn.f32x2 d, x, y;\n\tfma.rn.f32x2 %0, d, d, %0;\n\t"
+                "mov.b64 x, {%4, %5};\n\tmov.b64 y, {%8, %9};\n\t"
+                "sub.rn.f32x2 d, x, y;\n\tfma.rn.f32x2 %1, d, d, %1;\n\t}"
+                : "+l"(a), "+l"(b)
+                : "f"(x0), "f"(x1), "f"(x2), "f"(x3), "f"(y.x), "f"(y.y), "f"(y.z), "f"(y.w));
+        else
+            asm("{\n\t.reg .b64 x, y;\n\t"
+                "mov.b64 x, {%2, %3};\n\tmov.b64 y, {%6, %7};\n\t"
+                "fma.rn.f32x2 %0, x, y, %0;\n\t"
+                "mov.b64 x, {%4, %5};\n\tmov.b64 y, {%8, %9};\n\t"
+                "fma.rn.f32x2 %1, x, y, %1;\n\t}"
+                : "+l"(a), "+l"(b)
+                : "f"(x0), "f"(x1), "f"(x2), "f"(x3), "f"(y.x), "f"(y.y), "f"(y.z), "f"(y.w));
+    }
+    __device__ __forceinline__ void add(uint4 x, const uint8_t *q, int c)
+    {
+        if constexpr (DT == ANN_U8) {
+            const uint4 y = reinterpret_cast<const uint4 *>(q)[c];
+            uint32_t acc = static_cast<uint32_t>(a), d;  // exact integers in one word
             d = __vabsdiffu4(x.x, y.x);
             acc = __dp4a(d, d, acc);
             d = __vabsdiffu4(x.y, y.y);
@@ -231,132 +252,87 @@ __device__ __forceinline__ auto lane_sum(const uint8_t *row, const uint8_t *q, i
             d = __vabsdiffu4(x.z, y.z);
             acc = __dp4a(d, d, acc);
             d = __vabsdiffu4(x.w, y.w);
-            acc = __dp4a(d, d, acc);
-        };
-        if constexpr (CPL > 0) {
-#pragma unroll
-            for (int i = 0; i < CPL; ++i)
-                chunk(first + i * G);
-        } else {
-            for (int c = first; c < chunks; c += G)
-                chunk(c);
-        }
-        return acc;
-    } else {
-        float sum[V];
-        if constexpr (DT == ANN_I8S) {
-            // x_j = scale * code_j.  L2: sum of (q_j - scale * code_j)^2, each
-            // difference from one fused multiply-add; IP: scale * sum q_j code_j.
-            // The query buffer is zero beyond dim, where the codes are zero too.
-            const float scale = *reinterpret_cast<const float *>(row);
-            const uint4 *c4 = reinterpret_cast<const uint4 *>(row + 16);
+            a = __dp4a(d, d, acc);
+        } else if constexpr (DT == ANN_I8S) {
             const float4 *q4 = reinterpret_cast<const float4 *>(q);
-            float a0 = 0.f, a1 = 0.f;
-            for (int c = first; c < chunks - 1; c += G) {
-                const uint4 x = c4[c];
-                const uint32_t w[4] = {x.x, x.y, x.z, x.w};
+            const uint32_t w[4] = {x.x, x.y, x.z, x.w};
 #pragma unroll
-                for (int k = 0; k < 4; ++k) {
-                    const float4 y = q4[4 * c + k];
-                    const float c0 = static_cast<float>(static_cast<int8_t>(w[k] & 0xffu));
-                    const float c1 = static_cast<float>(static_cast<int8_t>((w[k] >> 8) & 0xffu));
-                    const float c2 = static_cast<float>(static_cast<int8_t>((w[k] >> 16) & 0xffu));
-                    const float c3 = static_cast<float>(static_cast<int8_t>(w[k] >> 24));
-                    if constexpr (MT == ANN_L2) {
-                        const float d0 = fmaf(-scale, c0, y.x), d1 = fmaf(-scale, c1, y.y);
-                        const float d2 = fmaf(-scale, c2, y.z), d3 = fmaf(-scale, c3, y.w);
-                        a0 = fmaf(d0, d0, a0);
-                        a1 = fmaf(d1, d1, a1);
-                        a0 = fmaf(d2, d2, a0);
-                        a1 = fmaf(d3, d3, a1);
-                    } else {
-                        a0 = fmaf(c0, y.x, a0);
-                        a1 = fmaf(c1, y.y, a1);
-                        a0 = fmaf(c2, y.z, a0);
-                        a1 = fmaf(c3, y.w, a1);
-                    }
-                }
-            }
-            sum[0] = a0 + a1;
-        } else {
-            const float4 *q4 = reinterpret_cast<const float4 *>(q);
-            // four FP32 accumulators (coordinates 4c+0..3) held as two packed
-            // pairs: each f32x2 operation rounds both halves exactly as the scalar
-            // operations would, at half the instruction count, and the two pairs
-            // are independent dependency chains
-            uint64_t acc[V], acc2[V];  // (0.f, 0.f)
-#pragma unroll
-            for (int v = 0; v < V; ++v)
-                acc[v] = acc2[v] = 0;
-            auto acc4 = [&](int v, float x0, float x1, float x2, float x3, float4 y) {
-                if constexpr (MT == ANN_L2)
-                    asm("{\n\t.reg .b64 x, y, d;\n\t"
-                        "mov.b64 x, {%2, %3};\n\tmov.b64 y, {%6, %7};\n\t"
-                        "sub.rn.f32x2 d, x, y;\n\tfma.rn.f32x2 %0, d, d, %0;\n\t"
-                        "mov.b64 x, {%4, %5};\n\tmov.b64 y, {%8, %9};\n\t"
-                        "sub.rn.f32x2 d, x, y;\n\tfma.rn.f32x2 %1, d, d, %1;\n\t}"
-                        : "+l"(acc[v]), "+l"(acc2[v])
-                        : "f"(x0), "f"(x1), "f"(x2), "f"(x3), "f"(y.x), "f"(y.y), "f"(y.z), "f"(y.w));
-                else
-                    asm("{\n\t.reg .b64 x, y;\n\t"
-                        "mov.b64 x, {%2, %3};\n\tmov.b64 y, {%6, %7};\n\t"
-                        "fma.rn.f32x2 %0, x, y, %0;\n\t"
-                        "mov.b64 x, {%4, %5};\n\tmov.b64 y, {%8, %9};\n\t"
-                        "fma.rn.f32x2 %1, x, y, %1;\n\t}"
-                        : "+l"(acc[v]), "+l"(acc2[v])
-                        : "f"(x0), "f"(x1), "f"(x2), "f"(x3), "f"(y.x), "f"(y.y), "f"(y.z), "f"(y.w));
-            };
-            auto chunk = [&](int v, int c) {
-                if constexpr (DT == ANN_F32) {
-                    const float4 x = reinterpret_cast<const float4 *>(row)[c];
-                    acc4(v, x.x, x.y, x.z, x.w, q4[c]);
+            for (int k = 0; k < 4; ++k) {
+                const float4 y = q4[4 * c + k];
+                const float e0 = static_cast<float>(static_cast<int8_t>(w[k] & 0xffu));
+                const float e1 = static_cast<float>(static_cast<int8_t>((w[k] >> 8) & 0xffu));
+                const float e2 = static_cast<float>(static_cast<int8_t>((w[k] >> 16) & 0xffu));
+                const float e3 = static_cast<float>(static_cast<int8_t>(w[k] >> 24));
+                if constexpr (MT == ANN_L2) {
+                    const float d0 = fmaf(-scale, e0, y.x), d1 = fmaf(-scale, e1, y.y);
+                    const float d2 = fmaf(-scale, e2, y.z), d3 = fmaf(-scale, e3, y.w);
+                    c0 = fmaf(d0, d0, c0);
+                    c1 = fmaf(d1, d1, c1);
+                    c0 = fmaf(d2, d2, c0);
+                    c1 = fmaf(d3, d3, c1);
                 } else {
-                    const uint4 x = reinterpret_cast<const uint4 *>(row)[c];
-                    float2 f0, f1, f2, f3;
-                    if constexpr (DT == ANN_F16) {
-                        f0 = __half22float2(*reinterpret_cast<const __half2 *>(&x.x));
-                        f1 = __half22float2(*reinterpret_cast<const __half2 *>(&x.y));
-                        f2 = __half22float2(*reinterpret_cast<const __half2 *>(&x.z));
-                        f3 = __half22float2(*reinterpret_cast<const __half2 *>(&x.w));
-                    } else {
-                        f0 = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162 *>(&x.x));
-                        f1 = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162 *>(&x.y));
-                        f2 = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162 *>(&x.z));
-                        f3 = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162 *>(&x.w));
-                    }
-                    acc4(v, f0.x, f0.y, f1.x, f1.y, q4[2 * c]);
-                    acc4(v, f2.x, f2.y, f3.x, f3.y, q4[2 * c + 1]);
-                }
-            };
-            if constexpr (CPL > 0) {
-#pragma unroll
-                for (int i = 0; i < CPL; ++i)
-                    chunk(0, first + i * G);
-            } else if constexpr (V == 1) {
-                for (int c = first; c < chunks; c += G)
-                    chunk(0, c);
-            } else {
-                for (int c = first; c < chunks; c += G) {
-#pragma unroll
-                    for (int v = 0; v < V; ++v)
-                        if (c + v * P < chunks)
-                            chunk(v, c + v * P);
+                    c0 = fmaf(e0, y.x, c0);
+                    c1 = fmaf(e1, y.y, c1);
+                    c0 = fmaf(e2, y.z, c0);
+                    c1 = fmaf(e3, y.w, c1);
                 }
             }
+        } else if constexpr (DT == ANN_F32) {
+            add4(__uint_as_float(x.x), __uint_as_float(x.y), __uint_as_float(x.z), __uint_as_float(x.w),
+                 reinterpret_cast<const float4 *>(q)[c]);
+        } else {
+            float2 f[4];
+            const uint32_t w[4] = {x.x, x.y, x.z, x.w};
 #pragma unroll
-            for (int v = 0; v < V; ++v)
-                sum[v] = (__uint_as_float(static_cast<uint32_t>(acc[v])) +
-                          __uint_as_float(static_cast<uint32_t>(acc[v] >> 32))) +
-                         (__uint_as_float(static_cast<uint32_t>(acc2[v])) +
-                          __uint_as_float(static_cast<uint32_t>(acc2[v] >> 32)));
+            for (int i = 0; i < 4; ++i) {
+                if constexpr (DT == ANN_F16)
+                    f[i] = __half22float2(*reinterpret_cast<const __half2 *>(&w[i]));
+                else
+                    f[i] = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162 *>(&w[i]));
+            }
+            const float4 *q4 = reinterpret_cast<const float4 *>(q);
+            add4(f[0].x, f[0].y, f[1].x, f[1].y, q4[2 * c]);
+            add4(f[2].x, f[2].y, f[3].x, f[3].y, q4[2 * c + 1]);
         }
-        if constexpr (V == 1)
-            return sum[0];
-        else if constexpr (V == 2)
-            return sum[0] + sum[1];
-        else
-            return (sum[0] + sum[2]) + (sum[1] + sum[3]);
     }
+    __device__ __forceinline__ auto sum() const
+    {
+        if constexpr (DT == ANN_U8)
+            return static_cast<uint32_t>(a);
+        else if constexpr (DT == ANN_I8S)
+            return c0 + c1;
+        else
+            return (__uint_as_float(static_cast<uint32_t>(a)) + __uint_as_float(static_cast<uint32_t>(a >> 32))) +
+                   (__uint_as_float(static_cast<uint32_t>(b)) + __uint_as_float(static_cast<uint32_t>(b >> 32)));
+    }
+};
+
+// A staged row's chunks: where they start and how many there are.
+template <int DT>
+__device__ __forceinline__ const uint4 *row_chunks(const uint8_t *row)
+{
+    return reinterpret_cast<const uint4 *>(row) + (DT == ANN_I8S ? 1 : 0);
+}
+
+// One team lane's part of the distance of a staged row to the query: chunks
+// first, first + G, ...  CPL > 0: exactly CPL chunks, unrolled so that their
+// shared-memory loads issue back to back; CPL = 0: any count.
+template <int DT, int MT, int CPL>
+__device__ __forceinline__ auto lane_sum(const uint8_t *row, const uint8_t *q, int chunks, int first, int G)
+{
+    const uint4 *x4 = row_chunks<DT>(row);
+    RowSum<DT, MT> acc;
+    if constexpr (DT == ANN_I8S)
+        acc.scale = *reinterpret_cast<const float *>(row);
+    if constexpr (CPL > 0) {
+#pragma unroll
+        for (int i = 0; i < CPL; ++i)
+            acc.add(x4[first + i * G], q, first + i * G);
+    } else {
+        for (int c = first; c < chunks; c += G)
+            acc.add(x4[c], q, c);
+    }
+    return acc.sum();
 }
 
 // How the lanes of a row's distance share the work of its team; each is a
@@ -367,42 +343,88 @@ enum Form {
     kOne,    // a lane is a team lane
     kOne8,   // the same, exactly 8 chunks each
     kPair4,  // two team lanes, one after the other, exactly 4 chunks each
-    kPair,   // two team lanes together
-    kQuad,   // four team lanes together
+    kRows2,  // a team lane of two rows at once
+    kRows4,  // of four rows at once
 };
-__host__ __device__ constexpr int form_members(int form)
+
+// Distances of the ch staged rows of the candidates in cbuf[0, ch) by teams of
+// G = 2^team_lg >= V lanes that take V rows at once: the query's chunks are read
+// once for V rows, the sums are V independent chains, and the lanes halve the
+// rows among themselves as the xor-shuffles go (G/2 apart first), so that V rows
+// take V + log2(G / V) - 1 of them.  Bit for bit one row at a time.
+template <int DT, int MT, int V>
+__device__ __forceinline__ void rows_distances(const uint8_t *stage, int stride, const uint8_t *q, int chunks,
+                                               uint64_t *cbuf, int ch, int team_lg, int lane)
 {
-    return form == kPair4 || form == kPair ? 2 : form == kQuad ? 4 : 1;
+    static_assert((V == 2 || V == 4) && DT != ANN_U8, "float rows, two or four at once");
+    const int G = 1 << team_lg, sub = lane & (G - 1), teams = 32 >> team_lg;
+    for (int r0 = 0; r0 < ch; r0 += V * teams) {
+        int row = r0 + (lane >> team_lg);  // and every teams-th: neighbouring teams read neighbouring rows
+        const uint4 *x[V];
+#pragma unroll
+        for (int v = 0; v < V; ++v)
+            x[v] = row_chunks<DT>(stage + min(row + v * teams, ch - 1) * stride);
+        RowSum<DT, MT> acc[V];
+        if constexpr (DT == ANN_I8S) {
+#pragma unroll
+            for (int v = 0; v < V; ++v)
+                acc[v].scale = *reinterpret_cast<const float *>(x[v] - 1);
+        }
+        for (int c = sub; c < chunks; c += G) {
+#pragma unroll
+            for (int v = 0; v < V; ++v)
+                acc[v].add(x[v][c], q, c);
+        }
+        int o = G >> 1;
+        const bool odd = lane & o;
+        auto half = [&](auto even_sum, auto odd_sum, bool mine) {
+            const auto give = mine ? even_sum : odd_sum;
+            return (mine ? odd_sum : even_sum) + __shfl_xor_sync(kFull, give, o);
+        };
+        auto s = half(acc[0].sum(), acc[1].sum(), odd);
+        row += odd ? teams : 0;
+        if constexpr (V == 4) {
+            const auto s2 = half(acc[2].sum(), acc[3].sum(), odd);
+            o >>= 1;
+            const bool high = lane & o;
+            s = half(s, s2, high);
+            row += high ? 2 * teams : 0;
+        }
+        while (o >>= 1)
+            s += __shfl_xor_sync(kFull, s, o);
+        if constexpr (DT == ANN_I8S && MT == ANN_IP)
+            s *= *reinterpret_cast<const float *>(stage + min(row, ch - 1) * stride);
+        const uint32_t bits = f32_to_ord(MT == ANN_IP ? -s : s);
+        if (row < ch && (sub & (G / V - 1)) == 0)
+            cbuf[row] = make_key(bits, key_id(cbuf[row]));
+    }
 }
 
 // Distance of one staged row to the query by P lanes (a power of two; sub =
-// lane % P) that stand for a team of P * members lanes: bit for bit the distance
-// the whole team computes, with fewer shuffles and more rows at once.  Every
-// lane returns the order-preserving key bits; the whole warp must call it.
+// lane % P) that stand for a team of P lanes, or of 2 P (kPair4): bit for bit the
+// distance the whole team computes, with fewer shuffles and more rows at once.
+// Every lane returns the order-preserving key bits; the whole warp must call it.
 template <int DT, int MT, int FORM>
 __device__ __forceinline__ uint32_t row_distance(const uint8_t *row, const uint8_t *q, int chunks, int sub, int P)
 {
-    if constexpr (DT == ANN_U8) {
-        uint32_t acc = lane_sum<DT, MT, 1, 0>(row, q, chunks, sub, P, P);  // exact integers: any order
+    auto team = [&](auto s) {
         for (int o = P >> 1; o > 0; o >>= 1)
-            acc += __shfl_xor_sync(kFull, acc, o);
-        return acc;  // exact non-negative int32, ordered as unsigned
+            s += __shfl_xor_sync(kFull, s, o);
+        return s;
+    };
+    if constexpr (DT == ANN_U8) {
+        // exact non-negative int32 in any order, ordered as unsigned
+        return team(lane_sum<DT, MT, 0>(row, q, chunks, sub, P));
     } else {
         float s;
         if constexpr (FORM == kPair4)
-            s = lane_sum<DT, MT, 1, 4>(row, q, chunks, sub, P, 2 * P) +
-                lane_sum<DT, MT, 1, 4>(row, q, chunks, sub + P, P, 2 * P);
-        else if constexpr (FORM == kOne8)
-            s = lane_sum<DT, MT, 1, 8>(row, q, chunks, sub, P, P);
+            s = lane_sum<DT, MT, 4>(row, q, chunks, sub, 2 * P) + lane_sum<DT, MT, 4>(row, q, chunks, sub + P, 2 * P);
         else
-            s = lane_sum<DT, MT, form_members(FORM), 0>(row, q, chunks, sub, P, form_members(FORM) * P);
-        for (int o = P >> 1; o > 0; o >>= 1)
-            s += __shfl_xor_sync(kFull, s, o);
+            s = lane_sum<DT, MT, FORM == kOne8 ? 8 : 0>(row, q, chunks, sub, P);
+        s = team(s);
         if constexpr (DT == ANN_I8S && MT == ANN_IP)
-            s = -(*reinterpret_cast<const float *>(row) * s);
-        else if constexpr (MT == ANN_IP)
-            s = -s;
-        return f32_to_ord(s);
+            s *= *reinterpret_cast<const float *>(row);
+        return f32_to_ord(MT == ANN_IP ? -s : s);
     }
 }
 
@@ -570,11 +592,15 @@ __global__ void __launch_bounds__(32 * kMaxSearchWarps, 16) beam_search_kernel(c
                     }
                     phase ^= 1u;
                     // a team of G lanes per staged row, 32 / G rows per pass
-                    for (int r0 = 0; r0 < ch; r0 += 32 >> a.team_lg) {
+                    const int chunks = a.rowbytes / 16 - (DT == ANN_I8S ? 1 : 0);
+                    if constexpr (FORM == kRows2 || FORM == kRows4)
+                        rows_distances<DT, MT, FORM == kRows2 ? 2 : 4>(stage, a.stage_stride, qbuf, chunks, cbuf + c0,
+                                                                       ch, a.team_lg, lane);
+                    else for (int r0 = 0; r0 < ch; r0 += 32 >> a.team_lg) {
                         const int r = r0 + (lane >> a.team_lg);
                         const int sub = lane & ((1 << a.team_lg) - 1);
                         const uint32_t bits = row_distance<DT, MT, FORM>(stage + min(r, ch - 1) * a.stage_stride,
-                                                                         qbuf, a.rowbytes / 16, sub, 1 << a.team_lg);
+                                                                         qbuf, chunks, sub, 1 << a.team_lg);
                         if (r < ch && sub == 0)
                             cbuf[c0 + r] = make_key(bits, key_id(cbuf[c0 + r]));
                     }
@@ -897,11 +923,13 @@ auto kernel_of_form(int maxc)
 template <int DT, int MT>
 auto kernel_for(int maxc, int form)
 {
+    if constexpr (DT != ANN_U8) {
+        if (form == kRows2)
+            return kernel_of_form<DT, MT, kRows2>(maxc);
+    }
     if constexpr (DT == ANN_F32) {
-        if (form == kPair)
-            return kernel_of_form<DT, MT, kPair>(maxc);
-        if (form == kQuad)
-            return kernel_of_form<DT, MT, kQuad>(maxc);
+        if (form == kRows4)
+            return kernel_of_form<DT, MT, kRows4>(maxc);
     }
     if constexpr (DT != ANN_U8 && DT != ANN_I8S) {
         if (form == kPair4)

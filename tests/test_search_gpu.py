@@ -392,10 +392,10 @@ def test_tables_sized_by_each_querys_own_L(hash_bits):
 @pytest.mark.parametrize("metric", [ann.L2, ann.IP])
 @pytest.mark.parametrize("dim,team", [(72, 0), (104, 0), (128, 0), (136, 0), (200, 0), (256, 0), (256, 8), (128, 4), (256, 32), (8, 0)])
 def test_distance_forms_are_bit_identical(dtype, metric, dim, team):
-    # rows read one by one are summed by fewer lanes than the team has (two or
-    # four members in turn or together, by the row's chunks and the type);
-    # tensor gathers always take one lane a member: the same bits either way,
-    # for every step width and the last, ragged round
+    # rows read one by one are summed by fewer lanes than the team has, or
+    # several rows at once, by the row's chunks and the type; tensor gathers
+    # always take a row at a time by the whole team: the same bits either way, for
+    # every step width and the last, ragged round
     rng = np.random.default_rng(dim + team)
     n = 3_000
     if dtype == np.float16:
@@ -411,5 +411,29 @@ def test_distance_forms_are_bit_identical(dtype, metric, dim, team):
             assert a[4] == b[4] == ann.OK
             for x, y in zip(a[:4], b[:4]):
                 assert np.array_equal(x.view(np.int32), y.view(np.int32))
+    finally:
+        ann.ann_free_index(h)
+
+
+@pytest.mark.parametrize("metric", [ann.L2, ann.IP])
+@pytest.mark.parametrize("dim", [496, 1_000, 1_008])
+def test_int8_distance_forms_are_bit_identical(metric, dim):
+    # as above for int8 rows with their scale (teams of 8 and 16); rows of 1,000
+    # codes end in zero codes
+    rng = np.random.default_rng(dim)
+    n = 2_000
+    x = torch.from_numpy(rng.standard_normal((n, dim)).astype(np.float32)).cuda()
+    packed = torch.empty((n, ann.ann_i8s_row_bytes(dim)), dtype=torch.uint8, device="cuda:0")
+    q = rng.standard_normal((150, dim)).astype(np.float32)
+    g = rng.integers(0, n, size=(n, 29)).astype(np.int32)
+    ann.ann_quantize_i8s(x, n, dim, packed)
+    h = ann.ann_index_create(packed, g, 5, ann.I8S, metric, n=n, dim=dim, degree=29)
+    try:
+        for W in (1, 4):
+            a = search(h, q, 20, 40, W=W, gather=1)
+            b = search(h, q, 20, 40, W=W, gather=4)
+            assert a[4] == b[4] == ann.OK
+            for u, v in zip(a[:4], b[:4]):
+                assert np.array_equal(u.view(np.int32), v.view(np.int32))
     finally:
         ann.ann_free_index(h)
