@@ -160,9 +160,9 @@ typedef struct {
  *             reports ANN_ERR_TIMEOUT through ann_sync_status.  The copies in
  *             flight still land, so the device and the index stay usable.
  *   gather    how a round of neighbour rows is fetched, 0 = chosen from the
- *             row size; 1: one bulk copy per row; 4: one TMA tensor gather per
- *             four rows (rows of 32-byte multiples up to 1 KiB; other sizes
- *             use 1).  Speed only, never results (see ann_autotune)
+ *             row size (4 up to 256 bytes, else 1); 1: one bulk copy per row;
+ *             4: one TMA tensor gather per four rows (rows of 32-byte
+ *             multiples up to 1 KiB; other sizes use 1).  Speed only, never results (see ann_autotune)
  *   d_k, d_L  optional per-query k and L (device int32[nq]); NULL = k, L
  *   d_target  optional per-query target node (device int32[nq]); when given
  *             the search runs in label mode: it stops after the step in which
@@ -772,9 +772,9 @@ ann_status ann_merge_shards(const int32_t *d_ids, const void *d_dists, int32_t P
 /*
  * Exact k nearest neighbours (Sec. 2.1, Problem 1; the ground truth R of
  * recall@k): for each of nq query rows, the k base rows with the smallest
- * (distance, id).  Candidate scores come from an fp32 GEMM; the best k + margin
- * candidates per query are re-scored exactly (int32 for uint8, fp32 direct
- * differences otherwise) and sorted.
+ * (distance, id).  Candidate scores come from the tensor cores; every candidate
+ * that their error leaves in question is re-scored exactly (int32 for uint8,
+ * fp32 direct differences otherwise) and sorted.
  *   d_base       n*dim base rows (dtype ANN_U8 or ANN_F32), 16-byte aligned
  *   d_queries    nq*dim rows of the same dtype; equal to d_base when
  *                exclude_self != 0 (then row i never returns id i)
@@ -782,8 +782,8 @@ ann_status ann_merge_shards(const int32_t *d_ids, const void *d_dists, int32_t P
  *   d_ids,d_dists out: nq*k int32 ids and distances (int32 for ANN_U8, fp32
  *                otherwise)
  * Blocking: returns after the results are written.  Temporary device memory
- * (about 4 GiB of scores plus fp32 copies of uint8 rows) is allocated on
- * `stream` and released before returning.
+ * (packed rows and candidate lists) comes from a pool of the device on `stream`;
+ * the pool keeps at most 1 GB.
  */
 ann_status ann_knn(const void *d_base, int64_t n, int32_t dim, int32_t dtype, int32_t metric,
                    const void *d_queries, int64_t nq, int32_t k, int32_t exclude_self,

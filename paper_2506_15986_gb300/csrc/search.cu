@@ -328,10 +328,13 @@ ann_status launch_search(ann_index *idx, const SearchLaunch &L, cudaStream_t s)
     // 16-byte chunks of a row to each lane, unless the caller fixed it
     const int chunks = idx->rowbytes / 16;
     const int G = p->team > 0 ? p->team : default_team(idx->rowbytes);
-    // gather mode: one TMA tensor gather per four rows when the index has a
-    // row map and the caller asks for it (or leaves it to the default, one
-    // bulk copy per row)
-    a.gather4 = (p->gather == 4 && idx->has_row_map) ? 1 : 0;
+    // gather mode, when the index has a row map: one TMA tensor gather per four
+    // rows when the caller asks for it or, left open, for rows of up to 256
+    // bytes, where issuing a copy per row costs more than the row; else a bulk
+    // copy per row (us, copies against gathers: 100 queries of 128-byte rows 283,
+    // 268, 10,000 914, 823; 100 of 256-byte rows 376, 347; 10,000 of 512-byte rows
+    // 1,179, 1,225; 1,000 of 1,024-byte rows 814, 918)
+    a.gather4 = idx->has_row_map && (p->gather == 4 || (p->gather == 0 && idx->rowbytes <= 256)) ? 1 : 0;
     if (a.gather4)
         a.row_map = idx->row_map;
     // Lanes per distance: where it pays, four lanes stand for a team of eight, or a
