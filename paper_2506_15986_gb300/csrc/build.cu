@@ -13,57 +13,80 @@
 namespace ann {
 namespace {
 
-// exact distance between a base row and a query row (uint8: int32 squared L2)
-template <int DT, int MT>
+// squared distance between two FP32 rows, as order-preserving key bits
 __device__ __forceinline__ uint32_t exact_dist_bits(const uint8_t *x, const uint8_t *q, int dim)
 {
+    const float4 *x4 = reinterpret_cast<const float4 *>(x);
+    const float4 *q4 = reinterpret_cast<const float4 *>(q);
+    float a0 = 0.f, a1 = 0.f, a2 = 0.f, a3 = 0.f;
+    for (int c = 0; c < dim / 4; ++c) {
+        const float4 u = x4[c], v = q4[c];
+        const float d0 = u.x - v.x, d1 = u.y - v.y, d2 = u.z - v.z, d3 = u.w - v.w;
+        a0 = fmaf(d0, d0, a0);
+        a1 = fmaf(d1, d1, a1);
+        a2 = fmaf(d2, d2, a2);
+        a3 = fmaf(d3, d3, a3);
+    }
+    return f32_to_ord((a0 + a1) + (a2 + a3));
+}
+
+// Squared distances of row x to the rows q0 and q1 at once, each as
+// exact_dist_bits adds it, as floats.
+template <int DT>
+__device__ __forceinline__ void two_dists(const uint8_t *x, const uint8_t *q0, const uint8_t *q1, int dim, float *d)
+{
     if constexpr (DT == ANN_U8) {
-        uint32_t acc = 0;
+        uint32_t a0 = 0, a1 = 0;
         for (int c = 0; c < dim / 4; ++c) {
-            const uint32_t a = reinterpret_cast<const uint32_t *>(x)[c];
-            const uint32_t b = reinterpret_cast<const uint32_t *>(q)[c];
-            const uint32_t d = __vabsdiffu4(a, b);
-            acc = __dp4a(d, d, acc);
+            const uint32_t u = reinterpret_cast<const uint32_t *>(x)[c];
+            const uint32_t e0 = __vabsdiffu4(u, reinterpret_cast<const uint32_t *>(q0)[c]);
+            const uint32_t e1 = __vabsdiffu4(u, reinterpret_cast<const uint32_t *>(q1)[c]);
+            a0 = __dp4a(e0, e0, a0);
+            a1 = __dp4a(e1, e1, a1);
         }
-        return acc;
+        d[0] = static_cast<float>(a0);
+        d[1] = static_cast<float>(a1);
     } else {
-        const float4 *x4 = reinterpret_cast<const float4 *>(x);
-        const float4 *q4 = reinterpret_cast<const float4 *>(q);
-        float a0 = 0.f, a1 = 0.f, a2 = 0.f, a3 = 0.f;
+        // four FP32 accumulators a row in two packed pairs: each f32x2 operation
+        // rounds both halves as two scalar ones would
+        uint64_t acc[2][2] = {};
+        auto add = [](uint64_t (&a)[2], float4 u, float4 v) {
+            asm("{\n\t.reg .b64 x, y, d;\n\t"
+                "mov.b64 x, {%2, %3};\n\tmov.b64 y, {%6, %7};\n\t"
+                "sub.rn.f32x2 d, x, y;\n\tfma.rn.f32x2 %0, d, d, %0;\n\t"
+                "mov.b64 x, {%4, %5};\n\tmov.b64 y, {%8, %9};\n\t"
+                "sub.rn.f32x2 d, x, y;\n\tfma.rn.f32x2 %1, d, d, %1;\n\t}"
+                : "+l"(a[0]), "+l"(a[1])
+                : "f"(u.x), "f"(u.y), "f"(u.z), "f"(u.w), "f"(v.x), "f"(v.y), "f"(v.z), "f"(v.w));
+        };
+#pragma unroll 4
         for (int c = 0; c < dim / 4; ++c) {
-            const float4 u = x4[c], v = q4[c];
-            if constexpr (MT == ANN_L2) {
-                const float d0 = u.x - v.x, d1 = u.y - v.y, d2 = u.z - v.z, d3 = u.w - v.w;
-                a0 = fmaf(d0, d0, a0);
-                a1 = fmaf(d1, d1, a1);
-                a2 = fmaf(d2, d2, a2);
-                a3 = fmaf(d3, d3, a3);
-            } else {
-                a0 = fmaf(u.x, v.x, a0);
-                a1 = fmaf(u.y, v.y, a1);
-                a2 = fmaf(u.z, v.z, a2);
-                a3 = fmaf(u.w, v.w, a3);
-            }
+            const float4 u = reinterpret_cast<const float4 *>(x)[c];
+            add(acc[0], u, reinterpret_cast<const float4 *>(q0)[c]);
+            add(acc[1], u, reinterpret_cast<const float4 *>(q1)[c]);
         }
-        float s = (a0 + a1) + (a2 + a3);
-        if constexpr (MT == ANN_IP)
-            s = -s;
-        return f32_to_ord(s);
+#pragma unroll
+        for (int i = 0; i < 2; ++i)
+            d[i] = (__uint_as_float(static_cast<uint32_t>(acc[i][0])) +
+                    __uint_as_float(static_cast<uint32_t>(acc[i][0] >> 32))) +
+                   (__uint_as_float(static_cast<uint32_t>(acc[i][1])) +
+                    __uint_as_float(static_cast<uint32_t>(acc[i][1] >> 32)));
     }
 }
 
 // Relative-neighbourhood pruning of node p's K candidates (sorted by exact
 // (dist, id)): c is kept unless a node s kept before it has
 // alpha * delta(s, c) <= delta(p, c); at most R are kept; -1 pads the row.
-// One CTA per node takes four candidates at a time, a warp each: its lanes
-// measure the candidate against the nodes kept so far and against the earlier
-// of the four, and the four are then decided in order.  So the chain of
-// decisions is a quarter as long as one candidate at a time and the staged
-// rows are shared by four warps (one warp a node left 6 warps on an SM: 4.26 ms
-// at 50,000 x 128, K = 64, R = 32; 2.34 ms here).
+// One CTA per node takes eight candidates at a time, two to a warp: its lanes
+// measure both against the nodes kept so far and against the earlier ones of the
+// eight, and the eight are then decided in order.  So the chain of decisions is
+// an eighth as long as one candidate at a time, the staged rows are shared by
+// four warps, and a kept row read from shared memory, whose bandwidth bounds the
+// kernel, serves two candidates (50,000 x 128, K = 64, R = 32: one warp a node
+// 4.26 ms, four with a candidate each 2.34 ms, 1.73 ms here).
 // STAGED: the K candidate rows are copied into shared memory first (when they
 // fit); otherwise they are read from global memory (L1/L2-cached) in place.
-constexpr int kPruneWarps = 4;
+constexpr int kPruneWarps = 4, kPruneGroup = 2 * kPruneWarps;
 
 template <int DT, bool STAGED>
 __global__ void __launch_bounds__(32 * kPruneWarps)
@@ -71,9 +94,9 @@ __global__ void __launch_bounds__(32 * kPruneWarps)
               int R, float alpha, int stride, int32_t *graph)
 {
     extern __shared__ __align__(16) uint8_t smem[];
-    __shared__ unsigned pruned[kPruneWarps];  // bit v < w: by the v-th of the four if kept; bit 31: by a kept node
+    __shared__ unsigned pruned[kPruneGroup];  // bit v < w: by the v-th of the eight if kept; bit 31: by a kept node
     __shared__ int32_t ids[128];
-    __shared__ int32_t kept[64 + kPruneWarps];
+    __shared__ int32_t kept[64 + kPruneGroup];
     const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
     const int64_t p = blockIdx.x;
     if (p >= n)
@@ -98,35 +121,41 @@ __global__ void __launch_bounds__(32 * kPruneWarps)
             return base + static_cast<int64_t>(ids[c]) * rowbytes;
     };
     int nk = 0;
-    for (int c0 = 0; c0 < K && nk < R; c0 += kPruneWarps) {
-        const int c = c0 + w;
-        const bool live = c < K && ids[c] >= 0;
-        unsigned by = 0;
-        if (live) {
-            float dpc;
+    for (int c0 = 0; c0 < K && nk < R; c0 += kPruneGroup) {
+        const int ca = c0 + w, cb = ca + kPruneWarps;
+        const bool live_a = ca < K && ids[ca] >= 0, live_b = cb < K && ids[cb] >= 0;
+        auto limit = [&](int c) {
             if constexpr (DT == ANN_U8)
-                dpc = static_cast<float>(reinterpret_cast<const int32_t *>(cand_d)[p * K + c]);
+                return static_cast<float>(reinterpret_cast<const int32_t *>(cand_d)[p * K + c]);
             else
-                dpc = reinterpret_cast<const float *>(cand_d)[p * K + c];
-            for (int j = lane; j < nk + w; j += 32) {
+                return reinterpret_cast<const float *>(cand_d)[p * K + c];
+        };
+        unsigned by_a = 0, by_b = 0;
+        if (live_a) {  // pads come last: cb is live only if ca is
+            const float la = limit(ca), lb = live_b ? limit(cb) : 0.f;
+            const uint8_t *xa = row(ca), *xb = live_b ? row(cb) : xa;
+            for (int j = lane; j < nk + w + (live_b ? kPruneWarps : 0); j += 32) {
                 const int s = j < nk ? kept[j] : c0 + (j - nk);
-                float dsc;
-                if constexpr (DT == ANN_U8)
-                    dsc = static_cast<float>(exact_dist_bits<ANN_U8, ANN_L2>(row(s), row(c), dim));
-                else
-                    dsc = ord_to_f32(exact_dist_bits<ANN_F32, ANN_L2>(row(s), row(c), dim));
-                if (alpha * dsc <= dpc)
-                    by |= j < nk ? 0x80000000u : 1u << (j - nk);
+                const unsigned bit = j < nk ? 0x80000000u : 1u << (j - nk);
+                float d[2];
+                two_dists<DT>(row(s), xa, xb, dim, d);
+                if (j < nk + w && alpha * d[0] <= la)
+                    by_a |= bit;
+                if (alpha * d[1] <= lb)
+                    by_b |= bit;
             }
         }
-        by = __reduce_or_sync(kFull, by);
-        if (lane == 0)
-            pruned[w] = by;
+        by_a = __reduce_or_sync(kFull, by_a);
+        by_b = __reduce_or_sync(kFull, by_b);
+        if (lane == 0) {
+            pruned[w] = by_a;
+            pruned[w + kPruneWarps] = by_b;
+        }
         __syncthreads();
-        // the four in order, by every thread alike
+        // the eight in order, by every thread alike
         unsigned in = 0;
         bool end = false;
-        for (int v = 0; v < kPruneWarps && !end; ++v) {
+        for (int v = 0; v < kPruneGroup && !end; ++v) {
             if (c0 + v >= K || ids[c0 + v] < 0 || nk >= R) {
                 end = true;
             } else if (!((pruned[v] & 0x80000000u) || (pruned[v] & in))) {
@@ -629,10 +658,10 @@ __global__ void reverse_prune(const float *x, int dim, const int32_t *touched, c
                 graph[static_cast<int64_t>(q) * R + deg + lane] = c1;
         } else {
             const uint8_t *xq = xb + static_cast<int64_t>(q) * rowbytes;
-            uint64_t k0 = c0 >= 0 ? make_key(exact_dist_bits<ANN_F32, ANN_L2>(xb + static_cast<int64_t>(c0) * rowbytes,
+            uint64_t k0 = c0 >= 0 ? make_key(exact_dist_bits(xb + static_cast<int64_t>(c0) * rowbytes,
                                                                                xq, dim), c0)
                                   : kKeyMax;
-            uint64_t k1 = c1 >= 0 ? make_key(exact_dist_bits<ANN_F32, ANN_L2>(xb + static_cast<int64_t>(c1) * rowbytes,
+            uint64_t k1 = c1 >= 0 ? make_key(exact_dist_bits(xb + static_cast<int64_t>(c1) * rowbytes,
                                                                                xq, dim), c1)
                                   : kKeyMax;
             warp_sort64(k0, k1, lane);
@@ -648,7 +677,7 @@ __global__ void reverse_prune(const float *x, int dim, const int32_t *touched, c
                 const float dqc = ord_to_f32(static_cast<uint32_t>(kc >> 32));
                 bool pruned = false;
                 for (int j = lane; j < nk; j += 32)
-                    pruned |= alpha * ord_to_f32(exact_dist_bits<ANN_F32, ANN_L2>(
+                    pruned |= alpha * ord_to_f32(exact_dist_bits(
                                           xb + static_cast<int64_t>(kept[j]) * rowbytes,
                                           xb + static_cast<int64_t>(id) * rowbytes, dim)) <= dqc;
                 if (!__any_sync(kFull, pruned)) {
