@@ -137,6 +137,36 @@ __device__ __forceinline__ int32_t key_id(uint64_t k)
     return static_cast<int32_t>((static_cast<uint32_t>(k)) >> 1);
 }
 
+// ---- chained launches --------------------------------------------------------
+
+// At the start of a kernel that launch_next may launch: lets the next one of
+// its stream start its blocks, and waits until all that the stream had before is
+// done and visible.
+__device__ __forceinline__ void begin_chained()
+{
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+
+// Launches a kernel that calls begin_chained: with `chained` its blocks are
+// placed while the kernel before it still runs, which takes the launch itself off
+// the chain.
+template <typename... P, typename... A>
+inline void launch_next(bool chained, void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, A... args)
+{
+    cudaLaunchAttribute at{};
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t c{};
+    c.gridDim = grid;
+    c.blockDim = block;
+    c.dynamicSmemBytes = smem;
+    c.stream = s;
+    c.attrs = &at;
+    c.numAttrs = chained ? 1 : 0;
+    cudaLaunchKernelEx(&c, kernel, static_cast<P>(args)...);
+}
+
 // ---- warp bitonic sorts (ascending) ------------------------------------------
 
 __device__ __forceinline__ uint64_t kmin(uint64_t a, uint64_t b) { return a < b ? a : b; }

@@ -66,6 +66,7 @@ __device__ __forceinline__ uint4 pack8_bf16(const float *a)
 
 __global__ void __launch_bounds__(128) tower_forward_kernel(const TowerArgs t)
 {
+    begin_chained();
     extern __shared__ __align__(1024) uint8_t smem[];
     uint8_t *sA = smem;            // 128 x 64 canonical (16 KB)
     uint8_t *sB = smem + 16384;    // 256 x 64 or 64 x 256 canonical (32 KB)
@@ -601,6 +602,7 @@ __global__ void __launch_bounds__(256)
                          __nv_bfloat16 *W2t, float *En, __nv_bfloat16 *Eb, float *Enrm, __nv_bfloat16 *W2b,
                          __nv_bfloat16 *EnT, int64_t ldE)
 {
+    begin_chained();
     __shared__ float t[64][65];
     __shared__ float scale[64];
     const int tid = threadIdx.x;
@@ -1028,7 +1030,7 @@ ann_status prepare_model(ann_entry_model *m, cudaStream_t s)
 }
 
 ann_status launch_tower(const ann_entry_model *m, const Operand &X, int64_t nq, float *qhat,
-                        __nv_bfloat16 *qhat_bf, const TowerTrain *train, int *status, cudaStream_t s)
+                        __nv_bfloat16 *qhat_bf, const TowerTrain *train, int *status, cudaStream_t s, bool chained)
 {
     if (nq == 0)
         return ANN_OK;
@@ -1049,7 +1051,7 @@ ann_status launch_tower(const ann_entry_model *m, const Operand &X, int64_t nq, 
                                          kTowerSmem);
     if (e != cudaSuccess)
         return cuda_status(e);
-    tower_forward_kernel<<<static_cast<unsigned>((nq + 127) / 128), 128, kTowerSmem, s>>>(t);
+    launch_next(chained, tower_forward_kernel, static_cast<unsigned>((nq + 127) / 128), 128, kTowerSmem, s, t);
     return cuda_status(cudaGetLastError());
 }
 

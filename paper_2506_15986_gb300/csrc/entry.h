@@ -60,7 +60,8 @@ struct TowerTrain {
     int64_t ld;
 };
 ann_status launch_tower(const ann_entry_model *m, const Operand &X, int64_t nq, float *qhat,
-                        __nv_bfloat16 *qhat_bf, const TowerTrain *train, int *status, cudaStream_t s);
+                        __nv_bfloat16 *qhat_bf, const TowerTrain *train, int *status, cudaStream_t s,
+                        bool chained = false);
 // Exhaustive entry selection in one kernel: the query tower, every hub's
 // score and the topm (1..8) best hubs' nodes per query (nq x topm, best
 // first); qhat (optional) receives the fp32 query embeddings.
