@@ -12,11 +12,11 @@
 // shared memory holds:
 //   - the query row;
 //   - a staging area the neighbour rows are gathered into by bulk copies
-//     (cp.async.bulk, one 16-byte-aligned row per copy, completion counted on
-//     an mbarrier);
+//     (cp.async.bulk, one 16-byte-aligned row per copy) or tensor gathers (four
+//     rows each), completion counted on an mbarrier;
 //   - the candidate pool: L 64-bit (distance, id, expanded) keys kept sorted;
-//     new candidates are sorted by a warp-shuffle bitonic network and merged
-//     in by rank (merge path);
+//     new candidates are sorted (by counting, or a warp-shuffle bitonic
+//     network) and merged in by rank;
 //   - optionally, the first level of the visited set (hash_bits > 0).
 // The visited set is an exact open-addressing hash (linear probing, key id+1,
 // 0 = empty) with up to three levels: the optional shared-memory table, a

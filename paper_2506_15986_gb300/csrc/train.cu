@@ -6,7 +6,7 @@
 //   forward   q_hat = tower(q) (tower_forward_kernel, saving Z1, A1, |Z2|);
 //             e_hat = E / |E|; S = q_hat e_hat^T / tau        (tcgen05 GEMM)
 //   loss      per query: -(1/|P|) sum_{v in P} log softmax_{P u N}(S)_v,
-//             averaged over queries with |P| > 0               (infonce_kernel)
+//             averaged over queries with |P| > 0          (infonce_rows_kernel)
 //   backward  dS = (softmax - 1[P]/|P|) / n_valid; dP = dS / tau
 //             dq_hat = dP e_hat, de_hat = dP^T q_hat            (tcgen05 GEMMs)
 //             through the normalisations, dZ2 -> dW2 = A1^T dZ2, db2,
