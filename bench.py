@@ -125,16 +125,11 @@ MEASURED_TRAFFIC = {
     # DRAM bytes read + written per headline launch, valid for these kernel
     # sources, entry mode, L, batch and tuned sizes: the mean of the three
     # searches of a capture sequence (bench.py --capture) on the fully
-    # trained headline, 2.921 GB read and 0.005-0.010 GB written each.
+    # trained headline, 3.020 GB read and 0.009-0.018 GB written each.
     "shift": [
-        dict(digest="25b45d1fbcd4631a", entry="exhaustive", L=93, nq=10_000, hash_bits=-1, stage_rows=8,
-             team=4, spill_bits=12, gather=0, visited_l2=True, group_entries=True,
-             bytes=((2.9226e9 + 0.0048e9) + (2.9206e9 + 0.0075e9) + (2.9194e9 + 0.0104e9)) / 3),
-        # the same with the plain work order (the autotuner picks either; grouping
-        # lets queries with one entry hub share their first rows in L2)
-        dict(digest="25b45d1fbcd4631a", entry="exhaustive", L=93, nq=10_000, hash_bits=-1, stage_rows=8,
-             team=4, spill_bits=12, gather=0, visited_l2=True, group_entries=False,
-             bytes=((3.3604e9 + 0.0056e9) + (3.3585e9 + 0.0086e9) + (3.3574e9 + 0.0119e9)) / 3),
+        dict(digest="de415cc66a3b5aa1", entry="exhaustive", L=93, nq=10_000, hash_bits=-1, stage_rows=8,
+             team=4, spill_bits=12, gather=4, visited_l2=True, group_entries=True,
+             bytes=((3.0236e9 + 0.0091e9) + (3.0172e9 + 0.0130e9) + (3.0184e9 + 0.0176e9)) / 3),
     ],
 }
 
