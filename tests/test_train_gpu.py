@@ -183,3 +183,36 @@ def test_row_losses_on_both_sides_of_the_hub_limits(H):
                                       E.astype(np.float64), mask[rows], 0.1)
     assert abs(loss - ref_loss) <= 1e-4 * abs(ref_loss)
     assert _rel(gE, ref["E"]) <= 8e-3
+
+
+def test_a_captured_step_gives_the_direct_steps_gradients():
+    # launches chain on a plain stream and are recorded as ordinary ones under
+    # capture; the batch's split sums add in any order (1e-5, as above)
+    X, W1, b1, W2, b2, E, mask, rows = _problem(B=700, D=128, H=200, seed=9)
+    cand, lab, M = dense_as_listed(mask)
+    x, r = torch.from_numpy(X).to(DEV), torch.from_numpy(rows).to(DEV)
+    out = []
+    for captured in (False, True):
+        t = ann.ann_trainer_create(128, W1, b1, W2, b2, E, 700, tau=0.1, lr=1e-3)
+        try:
+            step = lambda: ann.load_library().ann_trainer_step(  # noqa: E731
+                t, x.data_ptr(), r.data_ptr(), len(rows), cand.data_ptr(), lab.data_ptr(), M, 0, None,
+                torch.cuda.current_stream().cuda_stream)
+            if captured:
+                assert step() == ann.OK
+                torch.cuda.synchronize()
+                g = torch.cuda.CUDAGraph()
+                with torch.cuda.graph(g):
+                    assert step() == ann.OK
+                g.replay()
+                g.replay()
+            else:
+                assert step() == ann.OK
+            torch.cuda.synchronize()
+            gr = {k: np.zeros_like(v) for k, v in dict(W1=W1, b1=b1, W2=W2, b2=b2, E=E).items()}
+            ann.ann_trainer_get(t, gr["W1"], gr["b1"], gr["W2"], gr["b2"], gr["E"], gradients=True)
+        finally:
+            ann.ann_trainer_free(t)
+        out.append(gr)
+    for k in out[0]:
+        assert _rel(out[1][k], out[0][k]) <= 1e-5, k
