@@ -64,10 +64,9 @@ struct KnnArgs {
     int64_t unit;          // CTAs take ranges of this many (query tile, base tile) pairs: 1 or tiles_n
     int ip, self;          // inner product; skip the query's own index
     int dim, k;
-    uint64_t *lists;       // [rows rounded up to kTile][slots][cap] candidate keys
+    uint64_t *lists;       // [rows rounded up to kTile][slots][list_keys(KR)] candidate keys
     uint2 *ends;           // [rows rounded up to kTile][slots] a list's length and last threshold
     int slots, slot0;      // lists per query; the block's first
-    int cap;               // keys a list holds
     int *status;
 };
 
@@ -121,33 +120,72 @@ __device__ __forceinline__ void merge_sorted(uint64_t (&T)[KPL], uint64_t v, int
     }
 }
 
-// A list that is full keeps its 32 KPL smallest keys (at most half of it).
-// The lists of the lanes in `rows`, cnt keys each; returns the lane's new count.
-template <int KPL>
-__device__ __noinline__ int compact_rows(unsigned rows, int cnt, uint64_t *mine)
+// A list that is full keeps its KP smallest keys, in the order they came in (at
+// most half of it).  The lists of the lanes in `rows`, cnt keys each, at most
+// 32 J; returns the lane's new count and threshold.  A list's keys come in the
+// order of their ids, so from then on only a score below its largest one can
+// enter: that bounds what a list takes in when the slack hides every
+// difference between the scores (rows far from the origin, or one row farther
+// than the rest): 10,000 queries among 300,000 rows of 128 coordinates, k = 10,
+// one row of 1e20: 148 ms without the cut, 8.9 ms with it; 4.7 ms without that
+// row.  The KP-th smallest score is found bit by bit over the keys in
+// registers, keys of equal score stay by their order; sorting the list 32 keys
+// at a time instead took 12.8 ms, its warp's chain of shuffles holding up the
+// others at the next tile.
+struct ListEnd {
+    int cnt;
+    float thr;
+};
+
+template <int J, int KP>
+__device__ __noinline__ ListEnd compact_rows(unsigned rows, int cnt, uint64_t *mine, float thr)
 {
+    static_assert(32 * J >= 2 * KP, "room for what comes between two compactions");
     const int lane = threadIdx.x & 31;
     __syncwarp();
     while (rows) {
         const int r = __ffs(rows) - 1;
         rows &= rows - 1;
-        const int nb = __shfl_sync(kFull, cnt, r);
+        const int nb = __shfl_sync(kFull, cnt, r);  // more than 32 J - 32 >= KP
         uint64_t *L = reinterpret_cast<uint64_t *>(__shfl_sync(kFull, reinterpret_cast<unsigned long long>(mine), r));
-        uint64_t T[KPL];
+        uint64_t key[J];
 #pragma unroll
-        for (int i = 0; i < KPL; ++i)
-            T[i] = kKeyMax;
-        for (int i = 0; i < nb; i += 32)
-            merge_sorted<KPL>(T, warp_sort32(i + lane < nb ? L[i + lane] : kKeyMax, lane), lane);
-        __syncwarp();
+        for (int j = 0; j < J; ++j)
+            key[j] = 32 * j + lane < nb ? L[32 * j + lane] : kKeyMax;
+        uint32_t v = 0;   // the leading bits of the KP-th smallest score
+        int left = KP;    // its rank among the keys with those bits
+#pragma unroll 1
+        for (uint32_t bit = 0x80000000u; bit; bit >>= 1) {
+            int below = 0;  // keys with the bits found so far and a zero here
 #pragma unroll
-        for (int i = 0; i < KPL; ++i)
-            L[32 * i + lane] = T[i];
-        if (lane == r)
-            cnt = min(nb, 32 * KPL);
+            for (int j = 0; j < J; ++j) {
+                const uint32_t o = static_cast<uint32_t>(key[j] >> 32);
+                below += __popc(__ballot_sync(kFull, (o ^ v) < bit));
+            }
+            if (below < left) {
+                left -= below;
+                v |= bit;
+            }
+        }
+        int at = 0;
+#pragma unroll
+        for (int j = 0; j < J; ++j) {
+            const uint32_t o = static_cast<uint32_t>(key[j] >> 32);
+            const unsigned same = __ballot_sync(kFull, o == v);
+            const bool in = o < v || (o == v && __popc(same & lanemask_lt()) < left);
+            left = max(0, left - __popc(same));
+            const unsigned m = __ballot_sync(kFull, in);
+            if (in)
+                L[at + __popc(m & lanemask_lt())] = key[j];
+            at += __popc(m);
+        }
+        if (lane == r) {
+            cnt = KP;
+            thr = fminf(thr, ord_to_f32(v));  // a NaN gives way
+        }
         __syncwarp();
     }
-    return cnt;
+    return {cnt, thr};
 }
 
 // 32 columns of several accumulators with one wait
@@ -181,6 +219,10 @@ __device__ __forceinline__ void tmem_landed(uint32_t (&r)[32])
                    "+r"(r[30]), "+r"(r[31])::"memory");
 }
 
+// Keys that a list holds: about what a search of a million rows in random order
+// appends, and well above what a compaction leaves.
+constexpr int list_keys(int KR) { return KR == 1 ? 160 : KR <= 32 ? 256 : 512; }
+
 // P planes (1: BF16 values, 3: fp32 split), 32 KPL candidates kept of a list that
 // fills, KR >= k scores in registers, EW epilogue warps, MULTI: more than one
 // phase (128 coordinates) a tile.
@@ -211,7 +253,7 @@ __device__ __forceinline__ void tmem_landed(uint32_t (&r)[32])
 // The A images of a query tile stay in shared memory when they fit (K x P <=
 // six images: 128 fp32 or 384 uint8 coordinates), else they stream with the
 // base's.  The threshold is the k-th best score plus what the scores' errors
-// could hide.
+// could hide, and no more than the last key that a compaction kept.
 // 10,000 queries among 300,000 rows of 128 coordinates, k = 10: an SGEMM, its 12 GB
 // of scores and a pass that selects from them 23.3 ms; 4.5 ms here, six products
 // at 1,030 TFLOP/s, 55 % of the measured BF16 rate (bounded by shared-memory
@@ -402,7 +444,7 @@ __global__ void __launch_bounds__(64 + 32 * EW, 1) knn_tile_kernel(const KnnArgs
         }
     } else {
         // ---- epilogue: thread = query row of the tile and its columns, or half of them
-        constexpr int kHalves = EW / 4;
+        constexpr int kHalves = EW / 4, kCap = list_keys(KR);
         constexpr int kCols = kTile / kHalves;
         const int quad = warp & 3;         // a warp reads its own quarter of the TMEM lanes
         const int half = (warp - 2) >> 2;  // warps 2..5 the first half of the columns, 6..9 the second
@@ -435,7 +477,7 @@ __global__ void __launch_bounds__(64 + 32 * EW, 1) knn_tile_kernel(const KnnArgs
                     ++seg;
                 const int64_t row = tm * kTile + m;
                 list = row * a.slots + a.slot0 + kHalves * (blockIdx.x - cta_of_tile(tm * a.tiles_n / a.unit, T, G)) + half;
-                mine = a.lists + list * a.cap;
+                mine = a.lists + list * kCap;
                 cnt = 0;
 #pragma unroll
                 for (int i = 0; i < KR; ++i)
@@ -547,9 +589,12 @@ __global__ void __launch_bounds__(64 + 32 * EW, 1) knn_tile_kernel(const KnnArgs
                     todo &= width > cc ? (1u << (width - cc)) - 1u : 0u;
                 if (self >= id0 && self < id0 + 32)
                     todo &= ~(1u << static_cast<int>(self - id0));
-                const unsigned full = __ballot_sync(kFull, cnt > a.cap - 32);
-                if (full)
-                    cnt = compact_rows<KPL>(full, cnt, mine);
+                const unsigned full = __ballot_sync(kFull, cnt + __popc(todo) > kCap);
+                if (full) {
+                    const ListEnd end = compact_rows<kCap / 32, 32 * KPL>(full, cnt, mine, thr);
+                    cnt = end.cnt;
+                    thr = end.thr;
+                }
                 while (__any_sync(kFull, todo != 0)) {
                     const int j = __ffs(todo) - 1;
                     float h[16];
@@ -938,8 +983,7 @@ template <typename S, int P, int KPL, int KR, int EW>
 ann_status knn_typed(const S *base, int64_t n, int dim, int metric, const S *queries, int64_t nq, int k,
                      bool exclude_self, int32_t *d_ids, void *d_dists, cudaStream_t s)
 {
-    // keys of a list: about what a search of a million rows in random order appends
-    constexpr int kCap = KR == 1 ? 96 : KR <= 32 ? 256 : 512;
+    constexpr int kCap = list_keys(KR);
     const int chunks = (dim + 63) / 64;
     const size_t tile_bytes = static_cast<size_t>(chunks) * P * kImage;
     int dev = 0, sms = 0;
@@ -1035,7 +1079,6 @@ ann_status knn_typed(const S *base, int64_t n, int dim, int metric, const S *que
             a.k = k;
             a.lists = lists.as<uint64_t>();
             a.ends = ends.as<uint2>();
-            a.cap = kCap;
             a.slots = static_cast<int>(slots);
             a.slot0 = static_cast<int>(at[b]);
             a.status = status;

@@ -187,3 +187,56 @@ def test_graph_edges_match_oracle(n, dim, K, R, dtype):
     og, orep = oracle.build_graph(base, K=K, R=R, alpha=1.0)
     assert np.array_equal(g, og) and rep == orep
     assert med == oracle.medoid(base)
+
+
+def _best_ms(fn, n=5):
+    """Least time of n calls (ms, events around each) after two more."""
+    out = []
+    for i in range(n + 2):
+        a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+        a.record()
+        fn()
+        b.record()
+        b.synchronize()
+        out.append(a.elapsed_time(b))
+    return min(out[2:])
+
+
+@pytest.mark.parametrize("k,metric", [(1, "l2"), (10, "l2"), (10, "ip"), (64, "l2")])
+def test_knn_one_far_row(k, metric):
+    # one row of 1e20, whose norm hides every difference between the scores:
+    # the others' whole numbers keep theirs exact, every row is there three times
+    # so that ties go by id, and a query still takes in few of the rows
+    rng = np.random.default_rng(k)
+    base = rng.integers(-9, 10, size=(100_002, 64)).astype(np.float32)
+    base[1::3] = base[::3]
+    base[2::3] = base[::3]
+    q = rng.integers(-9, 10, size=(500, 64)).astype(np.float32)
+    far = base.copy()
+    far[77_777] = 1e20 if metric == "l2" else 0.0
+    if metric == "ip":
+        far[77_777, 0] = 1e20
+        q[:, 0] = 0.0  # x.y of the far row is zero, its error is not
+    m = ann.IP if metric == "ip" else ann.L2
+    ids, d = _knn_gpu(far, q, k, m)
+    oi, od = oracle.knn(far, q.astype(np.float64), k, metric=oracle.IP if metric == "ip" else oracle.L2)
+    assert np.array_equal(ids, oi) and np.array_equal(d.astype(np.float64), od)
+
+    def call(x):
+        x, y = torch.from_numpy(x).to(DEV), torch.from_numpy(q).to(DEV)
+        out = torch.empty((500, k), dtype=torch.int32, device=DEV), torch.empty((500, k), device=DEV)
+        return lambda: ann.ann_knn(x, len(x), 64, ann.F32, m, y, 500, k, *out)
+    assert _best_ms(call(far)) <= 7 * _best_ms(call(base))
+
+
+def test_knn_far_from_the_origin_takes_no_longer():
+    # all rows about (1000, ..., 1000): every score is within the others' slack
+    rng = np.random.default_rng(3)
+    base = torch.from_numpy(rng.standard_normal((100_000, 64)).astype(np.float32)).to(DEV)
+    q = base[:2000].clone()
+    out = torch.empty((2000, 10), dtype=torch.int32, device=DEV), torch.empty((2000, 10), device=DEV)
+    ms = []
+    for off in (0.0, 1000.0):
+        x, y = base + off, q + off
+        ms.append(_best_ms(lambda: ann.ann_knn(x, len(x), 64, ann.F32, ann.L2, y, len(y), 10, *out)))
+    assert ms[1] <= 7 * ms[0], ms
