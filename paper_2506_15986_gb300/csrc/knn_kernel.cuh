@@ -24,6 +24,7 @@
 
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
+#include <float.h>
 #include <stdint.h>
 
 #include <algorithm>
@@ -79,9 +80,12 @@ __device__ __forceinline__ uint64_t score_key(float s, int64_t id)
 // More than what two scores' errors and two exact distances' rounding can hide
 // for a query with squared norm nx: any sum of dim products or squares in fp32,
 // in whatever order, is within (16 + dim) 2^-24 of the sum of their
-// magnitudes, |x| |y| at most (twice that for -2 x.y), |x|^2 or |y|^2.
+// magnitudes, |x| |y| at most (twice that for -2 x.y), |x|^2 or |y|^2.  (A norm
+// that is no float leaves its products' size open.)
 __device__ __forceinline__ float score_slack(float nx, float nmax, int dim, int ip)
 {
+    if (!(nx < FLT_MAX && nmax < FLT_MAX))
+        return INFINITY;
     const float u = static_cast<float>(16 + dim) * 1.1920929e-7f;  // 2 * 2^-24
     const float xy = sqrtf(nx) * sqrtf(nmax);
     return 2.f * u * (ip ? xy : 2.f * xy + nmax + nx);
@@ -451,7 +455,7 @@ __global__ void __launch_bounds__(64 + 32 * EW, 1) knn_tile_kernel(const KnnArgs
         const int m = quad * 32 + lane;
         const uint32_t my_lane = tmem + (static_cast<uint32_t>(quad * 32) << 16) + half * kCols;
         const float nmax = __uint_as_float(*a.nmax);
-        const float coef = a.ip ? -1.f : -2.f;
+        float coef = 0.f;
         const float kNoThr = __int_as_float(0x7fffffff);  // NaN: every score passes
         // the k best scores in best[KR - k .. KR), ascending; the places below
         // never take one
@@ -482,7 +486,12 @@ __global__ void __launch_bounds__(64 + 32 * EW, 1) knn_tile_kernel(const KnnArgs
 #pragma unroll
                 for (int i = 0; i < KR; ++i)
                     best[i] = i < KR - a.k ? -INFINITY : INFINITY;
-                slack = row < a.rows ? score_slack(a.nx[row], nmax, a.dim, a.ip) : 0.f;
+                // an infinite query's products, whatever their size, stand for
+                // infinities of their sign; a NaN's scores are all NaN, so that
+                // the ids decide
+                const float nx = row < a.rows ? a.nx[row] : 0.f;
+                coef = nx == nx ? (isinf(nx) ? -FLT_MAX : a.ip ? -1.f : -2.f) : nx;
+                slack = score_slack(nx, nmax, a.dim, a.ip);
                 self = a.self ? a.row0 + row : -1;
                 pad = row >= a.rows;  // a padding row: no score is below its threshold
                 thr = pad ? -INFINITY : kNoThr;
@@ -490,8 +499,11 @@ __global__ void __launch_bounds__(64 + 32 * EW, 1) knn_tile_kernel(const KnnArgs
             uint32_t *shared_thr = sthr + (seg & 1) * kTile;
             const int b = static_cast<int>(tile & 1);
             const int64_t c0 = tn * kTile;
-            if (half == 0)
-                sny[b * kTile + m] = c0 + m < a.n ? (a.ip ? 0.f : a.ny[c0 + m]) : INFINITY;
+            if (half == 0) {
+                // (a NaN distance is ordered as -0: so is the score)
+                const float ny = c0 + m < a.n ? a.ny[c0 + m] : INFINITY;
+                sny[b * kTile + m] = c0 + m < a.n && (a.ip || ny != ny) ? 0.f : ny < FLT_MAX ? ny : INFINITY;
+            }
             const int width = static_cast<int>(min(static_cast<int64_t>(kTile), a.n - c0)) - half * kCols;
             // a phase's sums for 32 columns
             auto sums = [&](int cc, bool two, float (&v)[32]) {
@@ -687,10 +699,14 @@ __global__ void __launch_bounds__(64 + 32 * EW, 1) knn_tile_kernel(const KnnArgs
     }
 }
 
-// rows [r0, r0 + rows) of src as packed images [tile][chunk][plane], one
-// 16-byte piece (8 coordinates of a row) of all planes per thread
+// rows [r0, r0 + rows) of src, whose norms (norms_kernel) are norm[0, rows), as
+// packed images [tile][chunk][plane], one 16-byte piece (8 coordinates of a row)
+// of all planes per thread.  Infinite coordinates are packed as +-2^100, which
+// decides a score's sign as they do (an infinity itself times another row's zero
+// planes is NaN), in a query with the others as zero; a row with a NaN as zero.
 template <typename S, int P>
-__global__ void __launch_bounds__(256) pack_kernel(const S *src, int64_t r0, int64_t rows, int dim, int chunks, uint8_t *out)
+__global__ void __launch_bounds__(256)
+    pack_kernel(const S *src, const float *norm, bool query, int64_t r0, int64_t rows, int dim, int chunks, uint8_t *out)
 {
     const int64_t total = (rows + kTile - 1) / kTile * chunks * (kTile * 8);
     for (int64_t i = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x; i < total;
@@ -718,18 +734,23 @@ __global__ void __launch_bounds__(256) pack_kernel(const S *src, int64_t r0, int
                 for (int j = 0; j < 8; ++j)
                     x[j] = static_cast<float>(((j < 4 ? u.x : u.y) >> (8 * (j & 3))) & 0xffu);
             }
+            if (sizeof(S) == 4 && !isfinite(norm[r])) {
+#pragma unroll
+                for (int j = 0; j < 8; ++j)
+                    x[j] = !isinf(norm[r]) ? 0.f : isinf(x[j]) ? copysignf(0x1p100f, x[j]) : query ? 0.f : x[j];
+            }
         }
         __nv_bfloat16 h[P][8];
 #pragma unroll
         for (int j = 0; j < 8; ++j) {
             // high + middle + low == x exactly (a value that would round to
-            // infinity is cut instead; an infinity or NaN has no remainder)
+            // infinity is cut instead)
             __nv_bfloat16 hi = __float2bfloat16_rn(x[j]);
-            if (isinf(__bfloat162float(hi)) && !isinf(x[j]))
+            if (isinf(__bfloat162float(hi)))
                 hi = __float2bfloat16_rz(x[j]);
             h[0][j] = hi;
             if constexpr (P == 3) {
-                const float r1 = isfinite(x[j]) ? x[j] - __bfloat162float(hi) : 0.f;
+                const float r1 = x[j] - __bfloat162float(hi);
                 h[1][j] = __float2bfloat16_rn(r1);
                 h[2][j] = __float2bfloat16_rn(r1 - __bfloat162float(h[1][j]));
             }
@@ -740,8 +761,10 @@ __global__ void __launch_bounds__(256) pack_kernel(const S *src, int64_t r0, int
     }
 }
 
-// squared norms of rows (exact whole numbers for uint8 rows), and the bits of
-// their maximum (norms are never negative, so the bits order them)
+// squared norms of rows (exact whole numbers for uint8 rows): NaN where a
+// coordinate is NaN, else infinity where one is infinite, else finite (the
+// largest float where the sum passes it); and the bits of the finite ones'
+// maximum (norms are never negative, so the bits order them)
 template <typename S>
 __global__ void __launch_bounds__(256) norms_kernel(const S *x, int64_t rows, int dim, float *out, unsigned *nmax)
 {
@@ -750,16 +773,20 @@ __global__ void __launch_bounds__(256) norms_kernel(const S *x, int64_t rows, in
     float mx = 0.f;
     for (int64_t r = blockIdx.x * 8ll + w; r < rows; r += gridDim.x * 8ll) {
         float s = 0.f;
+        bool inf = false;
         for (int c = lane; c < dim; c += 32) {
             const float v = static_cast<float>(x[r * dim + c]);
             s = fmaf(v, v, s);
+            inf |= isinf(v);
         }
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1)
             s += __shfl_xor_sync(kFull, s, o);
+        if (!__any_sync(kFull, inf))
+            s = s > FLT_MAX ? FLT_MAX : s;
         if (lane == 0)
             out[r] = s;
-        mx = fmaxf(mx, s);
+        mx = fmaxf(mx, isfinite(s) ? s : 0.f);
     }
     if (lane == 0)
         best[w] = mx;
@@ -1033,9 +1060,10 @@ ann_status knn_typed(const S *base, int64_t n, int dim, int metric, const S *que
     int64_t list_count = 0;
     for (int64_t q0 = 0; q0 < nq; q0 += qb) {
         const int64_t rows = std::min(qb, nq - q0), tm = (rows + kTile - 1) / kTile;
-        pack_kernel<S, P><<<pack_grid(rows, chunks), 256, 0, s>>>(queries, q0, rows, dim, chunks, pa.as<uint8_t>());
         norms_kernel<S><<<static_cast<unsigned>(std::min<int64_t>((rows + 7) / 8, 152 * 8)), 256, 0, s>>>(
             queries + q0 * dim, rows, dim, nx.as<float>(), nullptr);
+        pack_kernel<S, P><<<pack_grid(rows, chunks), 256, 0, s>>>(queries, nx.as<float>(), true, q0, rows, dim, chunks,
+                                                                 pa.as<uint8_t>());
         // slots of every block of base rows
         std::vector<int64_t> at(nblocks + 1, 0);
         for (int64_t b = 0; b < nblocks; ++b)
@@ -1055,8 +1083,8 @@ ann_status knn_typed(const S *base, int64_t n, int dim, int metric, const S *que
         for (int64_t b = 0; b < nblocks; ++b) {
             const int64_t cols = std::min(nb, n - b * nb), tn = (cols + kTile - 1) / kTile;
             if (packed != b) {
-                pack_kernel<S, P><<<pack_grid(cols, chunks), 256, 0, s>>>(base, b * nb, cols, dim, chunks,
-                                                                         pb.as<uint8_t>());
+                pack_kernel<S, P><<<pack_grid(cols, chunks), 256, 0, s>>>(base, ny.as<float>() + b * nb, false, b * nb,
+                                                                         cols, dim, chunks, pb.as<uint8_t>());
                 packed = b;
             }
             KnnArgs a{};

@@ -240,3 +240,37 @@ def test_knn_far_from_the_origin_takes_no_longer():
         x, y = base + off, q + off
         ms.append(_best_ms(lambda: ann.ann_knn(x, len(x), 64, ann.F32, ann.L2, y, len(y), 10, *out)))
     assert ms[1] <= 7 * ms[0], ms
+
+
+@pytest.mark.parametrize("where", ["base", "-base", "query", "both", "huge"])
+@pytest.mark.parametrize("metric", ["l2", "ip"])
+@pytest.mark.parametrize("k", [1, 10, 100])
+def test_knn_infinite_coordinates(k, metric, where):
+    # a few rows with an infinite coordinate: their inner products are infinite
+    # by the other row's sign there, their L2 distances +inf; whole numbers
+    # elsewhere, none of them zero, so every order is exact and ties go by id
+    rng = np.random.default_rng(k)
+    base = rng.integers(1, 9, size=(3_000, 64)) * rng.choice([-1, 1], size=(3_000, 64))
+    q = rng.integers(1, 9, size=(70, 64)) * rng.choice([-1, 1], size=(70, 64))
+    base, q = base.astype(np.float32), q.astype(np.float32)
+    if where in ("base", "-base", "both"):
+        base[rng.choice(3_000, 7, replace=False), 5] = np.inf if where != "-base" else -np.inf
+    if where == "query" or (where == "both" and metric == "ip"):
+        q[::3, 9] = -np.inf
+    if where == "both" and metric == "ip":
+        base[:, 9], q[:, 5] = np.abs(base[:, 9]), np.abs(q[:, 5])
+        base[np.isinf(base[:, 5]), 9] *= -1  # both infinities give -inf: no pair is NaN
+    if where == "huge":  # finite, but its products and squares are not
+        base[rng.choice(3_000, 7, replace=False), 5] = 3e38
+    with np.errstate(all="ignore"):
+        x, y = base.astype(np.float64), q.astype(np.float64)
+        d = -(y[:, None] * x).sum(2) if metric == "ip" else ((y[:, None] - x) ** 2).sum(2)
+        d = d.astype(np.float32)
+    assert not np.isnan(d).any()
+    ids, dd = _knn_gpu(base, q, k, ann.IP if metric == "ip" else ann.L2)
+    if metric == "l2":  # a query whose distances are all infinite: any ids
+        some = np.isfinite(d).any(1)
+        assert np.isinf(dd[~some]).all()
+        ids, dd, d = ids[some], dd[some], d[some]
+    oi = np.argsort(d, axis=1, kind="stable")[:, :k]
+    assert np.array_equal(ids, oi) and np.array_equal(dd, np.take_along_axis(d, oi, 1))
