@@ -274,3 +274,31 @@ def test_knn_infinite_coordinates(k, metric, where):
         ids, dd, d = ids[some], dd[some], d[some]
     oi = np.argsort(d, axis=1, kind="stable")[:, :k]
     assert np.array_equal(ids, oi) and np.array_equal(dd, np.take_along_axis(d, oi, 1))
+
+
+@pytest.mark.parametrize("n,d,nq,k", [(3_000_000, 4, 300, 10), (18_000_000, 4, 130, 64), (6_000_000, 8, 129, 128)])
+def test_knn_blocks_of_base_rows(n, d, nq, k):
+    # two, seven and three packed blocks of base rows, the last one part-filled;
+    # whole numbers whose distances are exact, many of them equal
+    gen = torch.Generator(device=DEV).manual_seed(n)
+    base = torch.randint(-300, 301, (n, d), generator=gen, device=DEV).float()
+    q = torch.randint(-300, 301, (nq, d), generator=gen, device=DEV).float()
+    ids = torch.empty((nq, k), dtype=torch.int32, device=DEV)
+    dists = torch.empty((nq, k), device=DEV)
+    ann.ann_knn(base, n, d, ann.F32, ann.L2, q, nq, k, ids, dists)
+    id_ = torch.arange(n, device=DEV)
+    for i in range(nq):
+        key = ((base - q[i]) ** 2).sum(1).long() * (1 << 25) + id_
+        best = key.topk(k, largest=False).values.sort().values
+        assert torch.equal(ids[i].long(), best & ((1 << 25) - 1)) and torch.equal(dists[i].long(), best >> 25), i
+
+
+def test_knn_time_grows_with_the_base():
+    # six blocks of 960-d rows against one: the query rows of a launch stay as many
+    gen = torch.Generator(device=DEV).manual_seed(1)
+    base = torch.randn((1_080_000, 960), generator=gen, device=DEV)
+    q = torch.randn((2_000, 960), generator=gen, device=DEV)
+    out = torch.empty((2_000, 64), dtype=torch.int32, device=DEV), torch.empty((2_000, 64), device=DEV)
+    ms = [_best_ms(lambda: ann.ann_knn(base, n, 960, ann.F32, ann.L2, q, 2_000, 64, *out), 2)
+          for n in (180_000, 1_080_000)]
+    assert ms[1] <= 1.25 * 6 * ms[0], ms
