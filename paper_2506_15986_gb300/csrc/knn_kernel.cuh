@@ -869,17 +869,21 @@ __device__ __forceinline__ uint32_t eight_dists(const float *base, int dim, cons
 // over, the rest sorted and merged 32 at a time), of which those that the
 // scores' errors leave in question (the first ones: all below the k-th best
 // score plus the slack) are re-scored exactly and sorted by (distance, id).
-template <int DT, int MT, int KPL>
-__global__ void __launch_bounds__(128)
+// Few queries have many lists, one or two of every CTA of the chip: then WARPS of
+// a CTA share a query's lists, and the first merges what the others kept (one
+// query, k = 64, 200,000 x 960: whole call 3,610 us by one warp, 1,650 us by sixteen).
+template <int DT, int MT, int KPL, int WARPS>
+__global__ void __launch_bounds__(WARPS == 1 ? 128 : 32 * WARPS)
     rescore_kernel(const uint8_t *base, int rowbytes, const uint8_t *queries, int qbytes, int dim, int64_t rows,
                    const uint64_t *lists, const uint2 *ends, int slots, int cap, const float *nx, const unsigned *nmax,
                    int k, int32_t *out_ids, void *out_dists)
 {
     constexpr int KP = 32 * KPL;
-    __shared__ uint64_t sh[4][KP];  // first the candidates not yet merged, fewer than 64
-    __shared__ __align__(16) float tile[DT == ANN_U8 ? 1 : 4][9][132];
+    constexpr int kQueries = WARPS == 1 ? 4 : 1;
+    __shared__ uint64_t sh[kQueries * WARPS][KP];  // first the candidates not yet merged, fewer than 64
+    __shared__ __align__(16) float tile[DT == ANN_U8 ? 1 : kQueries][9][132];
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    const int64_t r = blockIdx.x * 4ll + w;
+    const int64_t r = WARPS == 1 ? blockIdx.x * 4ll + w : blockIdx.x;
     if (r >= rows)
         return;
     float low = __int_as_float(0x7fffffff);
@@ -903,7 +907,7 @@ __global__ void __launch_bounds__(128)
         merge_sorted<KPL>(T, v, lane);
         __syncwarp();
     };
-    for (int s = 0; s < slots; ++s) {
+    for (int s = WARPS == 1 ? 0 : w; s < slots; s += WARPS) {
         const uint2 end = ends[r * slots + s];
         const int len = static_cast<int>(end.x) < 0 ? 0 : static_cast<int>(end.x);  // -1: no list
         const uint64_t *L = lists + (r * slots + s) * cap;
@@ -921,6 +925,19 @@ __global__ void __launch_bounds__(128)
     if (nq > 0)
         merge();
     __syncwarp();
+    if constexpr (WARPS > 1) {
+#pragma unroll
+        for (int i = 0; i < KPL; ++i)
+            sh[w][32 * i + lane] = T[i];
+        __syncthreads();
+        if (w > 0)
+            return;
+        for (int v = 1; v < WARPS; ++v) {
+#pragma unroll 1
+            for (int i = 0; i < KP && sh[v][i] != kKeyMax; i += 32)
+                merge_sorted<KPL>(T, sh[v][i + lane], lane);
+        }
+    }
     uint64_t kth = kKeyMax;
 #pragma unroll
     for (int i = 0; i < KPL; ++i) {
@@ -1012,7 +1029,7 @@ template <typename S, int P, int KPL, int KR, int EW>
 ann_status knn_typed(const S *base, int64_t n, int dim, int metric, const S *queries, int64_t nq, int k,
                      bool exclude_self, int32_t *d_ids, void *d_dists, cudaStream_t s)
 {
-    constexpr int kCap = list_keys(KR);
+    constexpr int kCap = list_keys(KR), kShare = 16;
     const int chunks = (dim + 63) / 64;
     const size_t tile_bytes = static_cast<size_t>(chunks) * P * kImage;
     int dev = 0, sms = 0;
@@ -1117,21 +1134,24 @@ ann_status knn_typed(const S *base, int64_t n, int dim, int metric, const S *que
             KNN_CK(cudaGetLastError());
         }
         const int rowbytes = dim * static_cast<int>(sizeof(S));
-        const unsigned grid = static_cast<unsigned>((rows + 3) / 4);
         const uint8_t *bb = reinterpret_cast<const uint8_t *>(base);
         const uint8_t *qq = reinterpret_cast<const uint8_t *>(queries + q0 * dim);
         int32_t *oi = d_ids + q0 * k;
         void *od = static_cast<uint8_t *>(d_dists) + q0 * k * 4;
-        auto rescore = [&](auto kernel) {
-            kernel<<<grid, 128, 0, s>>>(bb, rowbytes, qq, rowbytes, dim, rows, lists.as<uint64_t>(), ends.as<uint2>(),
-                                        static_cast<int>(slots), kCap, nx.as<float>(), nmax, k, oi, od);
+        // up to four queries an SM, sixteen warps each: below, one warp a query
+        // leaves most of the chip idle
+        const bool few = rows <= 4 * int64_t{sms};
+        auto rescore = [&](auto one, auto shared) {
+            (few ? shared : one)<<<static_cast<unsigned>(few ? rows : (rows + 3) / 4), few ? 32 * kShare : 128, 0, s>>>(
+                bb, rowbytes, qq, rowbytes, dim, rows, lists.as<uint64_t>(), ends.as<uint2>(), static_cast<int>(slots),
+                kCap, nx.as<float>(), nmax, k, oi, od);
         };
         if constexpr (sizeof(S) == 1)
-            rescore(rescore_kernel<ANN_U8, ANN_L2, KPL>);
+            rescore(rescore_kernel<ANN_U8, ANN_L2, KPL, 1>, rescore_kernel<ANN_U8, ANN_L2, KPL, kShare>);
         else if (metric == ANN_L2)
-            rescore(rescore_kernel<ANN_F32, ANN_L2, KPL>);
+            rescore(rescore_kernel<ANN_F32, ANN_L2, KPL, 1>, rescore_kernel<ANN_F32, ANN_L2, KPL, kShare>);
         else
-            rescore(rescore_kernel<ANN_F32, ANN_IP, KPL>);
+            rescore(rescore_kernel<ANN_F32, ANN_IP, KPL, 1>, rescore_kernel<ANN_F32, ANN_IP, KPL, kShare>);
         KNN_CK(cudaGetLastError());
     }
     int failed = 0;

@@ -302,3 +302,25 @@ def test_knn_time_grows_with_the_base():
     ms = [_best_ms(lambda: ann.ann_knn(base, n, 960, ann.F32, ann.L2, q, 2_000, 64, *out), 2)
           for n in (180_000, 1_080_000)]
     assert ms[1] <= 1.25 * 6 * ms[0], ms
+
+
+@pytest.mark.parametrize("nq,k", [(1, 64), (5, 128), (609, 33), (608, 10)])
+def test_knn_few_queries(nq, k):
+    # their lists, one or two of every CTA, are shared by the warps of a CTA (up
+    # to 608 queries, four an SM), whole numbers as in test_knn_edges_exact
+    rng = np.random.default_rng(nq)
+    base = rng.integers(-3, 4, size=(30_000, 96)).astype(np.float32)
+    q = rng.integers(-3, 4, size=(nq, 96)).astype(np.float32)
+    ids, dd = _knn_gpu(base, q, k)
+    oi, od = oracle.knn(base, q.astype(np.float64), k)
+    assert np.array_equal(ids, oi) and np.array_equal(dd.astype(np.float64), od)
+
+
+def test_knn_of_one_query_is_no_slower_for_more_neighbours():
+    # one query among 200,000 x 960 (by selection from stored scores k = 64 took 1.66
+    # times what k = 1 takes here)
+    gen = torch.Generator(device=DEV).manual_seed(1)
+    base = torch.randn((200_000, 960), generator=gen, device=DEV)
+    out = torch.empty((1, 64), dtype=torch.int32, device=DEV), torch.empty((1, 64), device=DEV)
+    ms = [_best_ms(lambda: ann.ann_knn(base, len(base), 960, ann.F32, ann.L2, base, 1, k, *out)) for k in (1, 64)]
+    assert ms[1] <= 1.66 * ms[0], ms
