@@ -307,13 +307,21 @@ __device__ __forceinline__ float hb_penalty(float lam, float m, int cj)
 //     are decided over all children at their exact sizes (lane = child);
 //   - until no assumption changes.  Then every member has the child that the
 //     visit one by one gives it: by induction each assumption is the choice at
-//     the sizes that the earlier choices lead to.  After i passes the first i
-//     members are final, so at most 32 W + 1 passes run; two or three do.
+//     the sizes that the earlier choices lead to.  Two or three passes do, unless
+//     the penalties outweigh the distances or rows lie in the order of their
+//     clusters, so that most choices hang on the ones before: after kVisitPasses
+//     passes, or one that changes an eighth of the members, the rest of the
+//     round goes one by one, from the first warp with a member that changed (all
+//     before it are final).
 // For large clusters, whose sizes move slowly against their members'
 // preferences (about one member in thirty is uncertain); small ones go to
 // hb_visit_warp.  60,000 rows, k = 32: 11 ms a visit at level 1 one by one with a
 // 64-bit shuffle argmin per member, 5.2 ms one by one as hb_visit_warp, 790 us
-// here (990 us with W = 8, 910 us with 32).
+// here (990 us with W = 8, 910 us with 32).  Two levels of ten visits each, random
+// rows 12.5 ms; lambda = 1e9, rows along a line, and tight clusters stored one
+// after another 2,937, 2,728 and 1,240 ms with passes alone (one member at a time
+// with a 64-bit argmin: 175), 51, 52 and 45 ms here.
+constexpr int kVisitPasses = 4;
 constexpr int kVisitSmem = kVisitWarps * kMaxBranch * 33 * 4;
 
 template <int W>
@@ -328,6 +336,9 @@ __global__ void __launch_bounds__(32 * W)
     __shared__ float pen[kMaxBranch];
     __shared__ int size[kMaxBranch];
     __shared__ unsigned mask[W][kMaxBranch];   // the warp's lanes that assume a child
+    __shared__ unsigned moved[2];              // warps with a member that changed in this pass, and in the last
+    __shared__ int moves[2];                   // such members
+    __shared__ int2 won[32 * W];               // members decided one by one: child and rank
     const int64_t c = blockIdx.x;
     const int64_t b = seg[c], e = seg[c + 1];
     const float lam = lamv[c], m = mv[c];
@@ -350,6 +361,8 @@ __global__ void __launch_bounds__(32 * W)
     __syncthreads();
     for (int64_t i0 = b; i0 < e; i0 += 32 * W) {
         const bool live = i0 + tid < e;
+        if (tid < 2)
+            moved[tid] = moves[tid] = 0;
         uint32_t o1 = 0xffffffffu, o2 = 0xffffffffu;
         int j1 = 0, j2 = 0;
         float d1 = 0.f;
@@ -372,12 +385,15 @@ __global__ void __launch_bounds__(32 * W)
         }
         load(i0 + 32 * W + tid);  // in flight during the passes
         int my = j1, at = 0;
-        for (;;) {
+        bool alone = false;  // the round ends one by one
+        for (int pass = 0;; ++pass) {
             mask[w][lane] = 0u;
             __syncwarp();
             if (live)
                 atomicOr(&mask[w][my], 1u << lane);
             __syncthreads();
+            if (tid == 0)  // the next pass's, read before this pass's first meeting
+                moved[(pass + 1) & 1] = moves[(pass + 1) & 1] = 0;
             int fl = size[lane];  // lane = child: its size when the warp's members come
 #pragma unroll
             for (int v = 0; v < W - 1; ++v)
@@ -401,14 +417,55 @@ __global__ void __launch_bounds__(32 * W)
                     my = win;
                 }
             }
-            if (!__syncthreads_or(changed))
+            const int here = __popc(__ballot_sync(kAll, changed));
+            if (lane == 0 && here > 0) {
+                atomicOr(&moved[pass & 1], 1u << w);
+                atomicAdd(&moves[pass & 1], here);
+            }
+            __syncthreads();
+            const unsigned open_warps = moved[pass & 1];
+            if (!open_warps)
                 break;
+            if (pass + 1 < kVisitPasses && moves[pass & 1] < 4 * W)
+                continue;
+            alone = true;
+            const int w0 = __ffs(open_warps) - 1;
+            if (w == 0) {  // lane = child, as hb_visit_warp
+                int cj = size[lane];
+                for (int v = 0; v < w0; ++v)
+                    cj += __popc(mask[v][lane]);
+                float now = hb_penalty(lam, m, cj), next = hb_penalty(lam, m, cj + 1);
+                const int count = static_cast<int>(min(static_cast<int64_t>(32 * W), e - i0));
+                for (int v = w0; 32 * v < count; ++v) {
+                    const int left = min(32, count - 32 * v);
+#pragma unroll 4
+                    for (int u = 0; u < left; ++u) {
+                        const uint32_t key = lane < kk ? ord_bits(__fadd_rn(tile[v][lane][u], now)) : 0xffffffffu;
+                        const uint32_t mn = __reduce_min_sync(kAll, key);
+                        const unsigned eq = __ballot_sync(kAll, key == mn);
+                        const bool win = key == mn && (eq & ((1u << lane) - 1u)) == 0;
+                        if (win)
+                            won[32 * v + u] = make_int2(lane, cj);
+                        cj += win ? 1 : 0;
+                        now = win ? next : now;
+                        next = hb_penalty(lam, m, cj + 1);
+                    }
+                }
+                size[lane] = cj;
+                pen[lane] = now;
+            }
+            __syncthreads();
+            if (live && w >= w0) {
+                my = won[tid].x;
+                at = won[tid].y;
+            }
+            break;
         }
         if (live) {
             lab[i0 + tid] = my;
             rank[i0 + tid] = at;
         }
-        if (w == 0) {
+        if (w == 0 && !alone) {
             int sz = size[lane];
             for (int v = 0; v < W; ++v)
                 sz += __popc(mask[v][lane]);
@@ -729,7 +786,7 @@ ann_status ann_hbkm(const float *d_x, int64_t n, int32_t dim, int32_t k, int32_t
         hb_init_children<<<static_cast<unsigned>(P * k), 128, 0, s>>>(d_x, dim, k, init.as<int32_t>(),
                                                                        cent.as<float>(), cent2.as<float>());
         // large clusters: position tiles (a tile spans one or two clusters)
-        // and the visit by rounds of 256 members; below, pairs and warps.
+        // and the visit by rounds of 512 members; below, pairs and warps.
         // A visit by rounds assumes sizes up to 512 members old: its
         // uncertain members grow as the round's share of a cluster.  At 1 % of a
         // cluster it is 6.6 times as fast as one by one, at 27 % (1,875 members)

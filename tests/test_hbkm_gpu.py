@@ -113,3 +113,43 @@ def test_visits_by_rounds(n, dim, k, levels, lam):
     rng = np.random.default_rng(n)
     x = rng.integers(0, 3, size=(n, dim)).astype(np.float32)
     _same(x, k, levels, lam, 3, synth.hbkm_keys(n, seed=5))
+
+
+def _hard_rows(n, kind):
+    """Rows whose visits hang on one another: (rows, lambda)."""
+    rng = np.random.default_rng(n)
+    if kind == "line":  # equal steps, in order
+        return np.repeat(np.arange(n, dtype=np.float32)[:, None] / n, 128, 1), 1.0
+    x = rng.standard_normal((n, 128)).astype(np.float32)
+    if kind == "penalty":
+        return x, 1e9
+    centres = rng.standard_normal((60, 128)).astype(np.float32)
+    return (centres[np.arange(n) * 60 // n] + np.float32(0.01) * x).astype(np.float32), 1.0  # tight, one after another
+
+
+@pytest.mark.parametrize("kind", ["line", "penalty", "clusters"])
+def test_visits_whose_choices_hang_together(kind):
+    # most members of a round depend on the ones before: part of the rounds go
+    # one by one, from the first 32 members that are not settled
+    x, lam = _hard_rows(20_011, kind)
+    _same(x, 32, 2, lam, 3, synth.hbkm_keys(len(x), seed=6))
+
+
+def test_visits_one_by_one_bound_the_time():
+    # never slower than every member one by one, which took 14 times what random
+    # rows take here (175 and 12.4 ms)
+    def ms(x, lam):
+        dx, keys = torch.from_numpy(x).to(DEV), torch.from_numpy(synth.hbkm_keys(len(x), seed=6).view(np.int32)).to(DEV)
+        hubs = torch.empty(1024, dtype=torch.int32, device=DEV)
+        out = []
+        for _ in range(3):
+            a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+            a.record()
+            ann.ann_hbkm(dx, len(x), 128, 32, 2, lam, 10, keys, hubs)
+            b.record()
+            b.synchronize()
+            out.append(a.elapsed_time(b))
+        return min(out)
+    plain = ms(np.random.default_rng(1).standard_normal((60_000, 128)).astype(np.float32), 1.0)
+    for kind in ("line", "penalty", "clusters"):
+        assert ms(*_hard_rows(60_000, kind)) <= 14 * plain, kind
