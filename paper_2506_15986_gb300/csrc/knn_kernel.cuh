@@ -28,6 +28,7 @@
 #include <stdint.h>
 
 #include <algorithm>
+#include <numeric>
 
 #include "device_util.cuh"
 #include "internal.h"
@@ -61,6 +62,7 @@ struct KnnArgs {
     int64_t rows;          // queries of the block
     int64_t row0;          // index of its first query (self exclusion)
     int64_t tiles_m, tiles_n;
+    int64_t stride;        // the j-th base tile a query tile meets is j * stride mod tiles_n
     int64_t unit;          // CTAs take ranges of this many (query tile, base tile) pairs: 1 or tiles_n
     int ip, self;          // inner product; skip the query's own index
     int dim, k;
@@ -68,6 +70,24 @@ struct KnnArgs {
     uint2 *ends;           // [rows rounded up to kTile][slots] a list's length and last threshold
     int slots;             // lists per query
     int *status;
+};
+
+// A (query tile, base tile) pair in the order that CTAs take them: query tile tm's
+// j-th pair has base tile j * stride mod tiles_n.
+struct TileWalk {
+    int64_t tm, j, tn;
+    __device__ TileWalk(const KnnArgs &a, int64_t t) : tm(t / a.tiles_n), j(t - tm * a.tiles_n), tn(j * a.stride % a.tiles_n)
+    {
+    }
+    __device__ void next(const KnnArgs &a)
+    {
+        tn += a.stride;
+        tn -= tn >= a.tiles_n ? a.tiles_n : 0;
+        if (++j == a.tiles_n) {
+            j = tn = 0;
+            ++tm;
+        }
+    }
 };
 
 // The score of a certain candidate: keys are (order-preserving score, id).
@@ -123,25 +143,25 @@ __device__ __forceinline__ void merge_sorted(uint64_t (&T)[KPL], uint64_t v, int
     }
 }
 
-// A list that is full keeps its KP smallest keys, in the order they came in (at
-// most half of it).  The lists of the lanes in `rows`, cnt keys each, at most
-// 32 J; returns the lane's new count and threshold.  A list's keys come in the
-// order of their ids, so from then on only a score below its largest one can
-// enter: that bounds what a list takes in when the slack hides every
+// A list that is full keeps its KP smallest keys (at most half of it).  The lists
+// of the lanes in `rows`, cnt keys each, at most 32 J; returns the lane's new
+// count and its list's last key.  From then on only a key below that can enter,
+// which bounds what a list takes in when the slack hides every
 // difference between the scores (rows far from the origin, or one row farther
 // than the rest): 10,000 queries among 300,000 rows of 128 coordinates, k = 10,
 // one row of 1e20: 148 ms without the cut, 8.9 ms with it; 4.7 ms without that
 // row.  The KP-th smallest score is found bit by bit over the keys in
-// registers, keys of equal score stay by their order; sorting the list 32 keys
+// registers, and where it cuts equal scores their ids'; sorting the list 32 keys
 // at a time instead took 12.8 ms, its warp's chain of shuffles holding up the
 // others at the next tile.
 struct ListEnd {
     int cnt;
-    float thr;
+    float score;
+    uint32_t id;
 };
 
 template <int J, int KP>
-__device__ __noinline__ ListEnd compact_rows(unsigned rows, int cnt, uint64_t *mine, float thr)
+__device__ __noinline__ ListEnd compact_rows(unsigned rows, int cnt, uint64_t *mine, float score, uint32_t id)
 {
     static_assert(32 * J >= 2 * KP, "room for what comes between two compactions");
     const int lane = threadIdx.x & 31;
@@ -170,13 +190,31 @@ __device__ __noinline__ ListEnd compact_rows(unsigned rows, int cnt, uint64_t *m
                 v |= bit;
             }
         }
+        int same = 0;
+#pragma unroll
+        for (int j = 0; j < J; ++j)
+            same += __popc(__ballot_sync(kFull, static_cast<uint32_t>(key[j] >> 32) == v));
+        uint32_t cut = 0xffffffffu;  // the last id kept of that score
+        if (same > left) {
+            cut = 0;
+#pragma unroll 1
+            for (uint32_t bit = 0x80000000u; bit; bit >>= 1) {
+                int below = 0;
+#pragma unroll
+                for (int j = 0; j < J; ++j)
+                    below += __popc(__ballot_sync(kFull, static_cast<uint32_t>(key[j] >> 32) == v &&
+                                                             (static_cast<uint32_t>(key[j]) ^ cut) < bit));
+                if (below < left) {
+                    left -= below;
+                    cut |= bit;
+                }
+            }
+        }
+        const uint64_t most = static_cast<uint64_t>(v) << 32 | cut;
         int at = 0;
 #pragma unroll
         for (int j = 0; j < J; ++j) {
-            const uint32_t o = static_cast<uint32_t>(key[j] >> 32);
-            const unsigned same = __ballot_sync(kFull, o == v);
-            const bool in = o < v || (o == v && __popc(same & lanemask_lt()) < left);
-            left = max(0, left - __popc(same));
+            const bool in = key[j] <= most;
             const unsigned m = __ballot_sync(kFull, in);
             if (in)
                 L[at + __popc(m & lanemask_lt())] = key[j];
@@ -184,11 +222,12 @@ __device__ __noinline__ ListEnd compact_rows(unsigned rows, int cnt, uint64_t *m
         }
         if (lane == r) {
             cnt = KP;
-            thr = fminf(thr, ord_to_f32(v));  // a NaN gives way
+            score = ord_to_f32(v);
+            id = cut;
         }
         __syncwarp();
     }
-    return {cnt, thr};
+    return {cnt, score, id};
 }
 
 // 32 columns of several accumulators with one wait
@@ -326,9 +365,10 @@ __global__ void __launch_bounds__(64 + 32 * EW, 1) knn_tile_kernel(const KnnArgs
                 }
             };
             int64_t uses = 0;
-            for (int64_t t = t0; t < t1 && ok; ++t) {
-                const int64_t tm = t / a.tiles_n, tn = t - tm * a.tiles_n;
-                if (resident && (t == t0 || tn == 0))
+            TileWalk at(a, t0);
+            for (int64_t t = t0; t < t1 && ok; ++t, at.next(a)) {
+                const int64_t tm = at.tm, tn = at.tn;
+                if (resident && (t == t0 || at.j == 0))
                     copy_resident(tm, uses++);
                 for (int c = 0; c < chunks && ok; ++c) {
                     const uint8_t *sa = a.A + (tm * chunks + c) * P * kImage, *sb = a.B + (tn * chunks + c) * P * kImage;
@@ -374,9 +414,9 @@ __global__ void __launch_bounds__(64 + 32 * EW, 1) knn_tile_kernel(const KnnArgs
                            smem_desc(smem + kOffB + sb * kImage + kk * 256, 128, 1024), ID,
                            (first && kk == 0) ? 0u : 1u);
             };
-            for (int64_t t = t0; t < t1 && ok; ++t) {
-                const int64_t tn = t % a.tiles_n;
-                const bool fresh = t == t0 || tn == 0;
+            TileWalk at(a, t0);
+            for (int64_t t = t0; t < t1 && ok; ++t, at.next(a)) {
+                const bool fresh = t == t0 || at.j == 0;
                 if (fresh)
                     ++uses;
                 for (int c = 0; c < chunks && ok; ++c) {
@@ -438,7 +478,7 @@ __global__ void __launch_bounds__(64 + 32 * EW, 1) knn_tile_kernel(const KnnArgs
                         ++ph;
                     }
                 }
-                if (resident && (tn == a.tiles_n - 1 || t == t1 - 1))
+                if (resident && (at.j == a.tiles_n - 1 || t == t1 - 1))
                     for (int s = 0; s < chunks * P; ++s)
                         tc_commit(&bars->empty_a[s]);
             }
@@ -458,7 +498,10 @@ __global__ void __launch_bounds__(64 + 32 * EW, 1) knn_tile_kernel(const KnnArgs
         // the k best scores in best[KR - k .. KR), ascending; the places below
         // never take one
         float best[KR];
-        float thr = 0.f, slack = 0.f;  // a NaN threshold: every score passes
+        // scores up to thr pass (all, when it is NaN), but of those equal to cut, the
+        // list's last score at its last compaction, only ids below cut_id
+        float thr = 0.f, slack = 0.f, cut = 0.f;
+        uint32_t cut_id = 0;
         int cnt = 0;
         int64_t self = -1, list = -1, seg = 0;
         uint64_t *mine = nullptr;
@@ -470,9 +513,10 @@ __global__ void __launch_bounds__(64 + 32 * EW, 1) knn_tile_kernel(const KnnArgs
             if (list >= 0)
                 a.ends[list] = make_uint2(static_cast<uint32_t>(cnt), __float_as_uint(thr));
         };
-        for (int64_t t = t0, tile = 0; t < t1 && ok; ++t, ++tile) {
-            const int64_t tm = t / a.tiles_n, tn = t - tm * a.tiles_n;
-            const bool fresh = t == t0 || tn == 0;
+        TileWalk at(a, t0);
+        for (int64_t t = t0, tile = 0; t < t1 && ok; ++t, ++tile, at.next(a)) {
+            const int64_t tm = at.tm, tn = at.tn;
+            const bool fresh = t == t0 || at.j == 0;
             if (fresh) {
                 end_list();
                 if (t != t0)
@@ -497,6 +541,8 @@ __global__ void __launch_bounds__(64 + 32 * EW, 1) knn_tile_kernel(const KnnArgs
                 self = a.self ? a.row0 + row : -1;
                 pad = row >= a.rows;  // a padding row: no score is below its threshold
                 thr = pad ? -INFINITY : __uint_as_float(end.y);
+                cut = pad ? thr : __int_as_float(0x7fffffff);
+                cut_id = 0;
             }
             uint32_t *shared_thr = sthr + (seg & 1) * kTile;
             const int b = static_cast<int>(tile & 1);
@@ -589,7 +635,7 @@ __global__ void __launch_bounds__(64 + 32 * EW, 1) knn_tile_kernel(const KnnArgs
                     s[4 * g + 3] = fmaf(coef, s[4 * g + 3], y.w);
                     lo = fminf(lo, fminf(fminf(s[4 * g], s[4 * g + 1]), fminf(s[4 * g + 2], s[4 * g + 3])));
                 }
-                if (!__any_sync(kFull, !(lo >= thr)))
+                if (!__any_sync(kFull, !(lo > thr)))
                     return;
                 // the columns that pass, then every lane its own one after
                 // another: a few turns, not one for every column that passes
@@ -598,16 +644,27 @@ __global__ void __launch_bounds__(64 + 32 * EW, 1) knn_tile_kernel(const KnnArgs
                 unsigned todo = 0;
 #pragma unroll
                 for (int j = 0; j < 32; ++j)
-                    todo |= (s[j] >= thr ? 0u : 1u) << j;
+                    todo |= (s[j] > thr ? 0u : 1u) << j;
+                if (__any_sync(kFull, thr == cut)) {
+                    unsigned equal = 0;
+#pragma unroll
+                    for (int j = 0; j < 32; ++j)
+                        equal |= (s[j] == cut ? 1u : 0u) << j;
+                    const int64_t ids = max(static_cast<int64_t>(0), cut_id - id0);
+                    if (thr == cut && ids < 32)
+                        todo &= ~(equal & ~((1u << ids) - 1u));
+                }
                 if (width - cc < 32)
                     todo &= width > cc ? (1u << (width - cc)) - 1u : 0u;
                 if (self >= id0 && self < id0 + 32)
                     todo &= ~(1u << static_cast<int>(self - id0));
                 const unsigned full = __ballot_sync(kFull, cnt + __popc(todo) > kCap);
                 if (full) {
-                    const ListEnd end = compact_rows<kCap / 32, 32 * KPL>(full, cnt, mine, thr);
+                    const ListEnd end = compact_rows<kCap / 32, 32 * KPL>(full, cnt, mine, cut, cut_id);
                     cnt = end.cnt;
-                    thr = end.thr;
+                    cut = end.score;
+                    cut_id = end.id;
+                    thr = fminf(thr, cut);  // a NaN gives way
                 }
                 while (__any_sync(kFull, todo != 0)) {
                     const int j = __ffs(todo) - 1;
@@ -625,7 +682,7 @@ __global__ void __launch_bounds__(64 + 32 * EW, 1) knn_tile_kernel(const KnnArgs
                     for (int i = 0; i < 2; ++i)
                         h[i] = j & 2 ? h[2 + i] : h[i];
                     float x = j & 1 ? h[1] : h[0];
-                    if (todo != 0 && !(x >= thr)) {
+                    if (todo != 0 && !(x > thr)) {
                         mine[cnt++] = score_key(x, id0 + j);
                         x = x == x ? x : INFINITY;
 #pragma unroll
@@ -1057,6 +1114,17 @@ ann_status knn_typed(const S *base, int64_t n, int dim, int metric, const S *que
                 most = std::max(most, cta_of_tile((i + 1) * tn - 1, T, G) - cta_of_tile(i * tn, T, G) + 1);
         return most * (EW / 4);
     };
+    // Base tiles are met by the golden section of their number, all CTAs alike (they
+    // share them in L2).  In their own order, rows that lie along a path would
+    // come nearer and nearer to a query until its own place, each of them among
+    // the best so far (among themselves, 100,000 steps of a random walk, d = 96, k =
+    // 64: 273 ms so, 22 here; along a line, k = 100: 412, 19).
+    auto scattered = [](int64_t tn) {
+        int64_t stride = std::max<int64_t>(1, static_cast<int64_t>(0.6180339887 * static_cast<double>(tn)));
+        while (std::gcd(stride, tn) != 1)
+            ++stride;
+        return stride;
+    };
     const int64_t tn_max = nb / kTile;
     for (;;) {
         const int64_t tm = qb / kTile;
@@ -1083,8 +1151,7 @@ ann_status knn_typed(const S *base, int64_t n, int dim, int metric, const S *que
             queries + q0 * dim, rows, dim, nx.as<float>(), nullptr);
         pack_kernel<S, P><<<pack_grid(rows, chunks), 256, 0, s>>>(queries, nx.as<float>(), true, q0, rows, dim, chunks,
                                                                  pa.as<uint8_t>());
-        // a query's lists go on from block to block of the base rows, whose ids
-        // ascend (a list of each block's own took memory by their number, which
+        // a query's lists go on from block to block of the base rows (a list of each block's own took memory by their number, which
         // left query blocks of 128 rows that each packed the whole base again:
         // 10,000 queries among 1,000,000 x 960, k = 64, 1,140 ms; 172 ms)
         const int64_t last = n - (nblocks - 1) * nb;
@@ -1122,6 +1189,7 @@ ann_status knn_typed(const S *base, int64_t n, int dim, int metric, const S *que
             a.tiles_m = tm;
             a.tiles_n = tn;
             a.unit = unit_of(tm, tn);
+            a.stride = scattered(tn);
             a.ip = metric == ANN_IP;
             a.self = exclude_self;
             a.dim = dim;
