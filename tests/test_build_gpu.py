@@ -355,3 +355,31 @@ def test_knn_rows_along_a_path_take_no_longer_than_a_selection():
         ms = [_best_ms(lambda: ann.ann_knn(y, 20_000, y.shape[1], ann.F32, ann.L2, y, 20_000, k, *out, exclude_self=True), 3)
               for y in (x, x[p].contiguous())]
         assert ms[0] <= bar * ms[1], (k, ms)
+
+
+def _line(n, lines=1):
+    x = np.zeros((n, 16), np.float32)
+    x[:, 0] = np.arange(n)
+    x[n // 2:, 1] = 2048 * (lines - 1)
+    return x
+
+
+@pytest.mark.parametrize("lines", [1, 2])
+def test_graph_of_rows_along_a_line(lines):
+    # a path: as many levels as nodes to the farther end, and with two lines one
+    # of them attached by the repair and walked from there; exact distances
+    x = _line(3_000, lines)
+    g, med, rep = _graph_gpu(x, 64, 32)
+    og, orep = oracle.build_graph(x, K=64, R=32)
+    assert np.array_equal(g, og) and rep == orep and med == oracle.medoid(x)
+    assert rep >= lines - 1
+
+
+def test_graph_of_a_long_path_takes_no_longer_than_on_the_host():
+    # 10,000 levels: with the search on the host the line took 3.8 times what random
+    # rows take here
+    def ms(x):
+        dx, g = torch.from_numpy(x).to(DEV), torch.empty((len(x), 32), dtype=torch.int32, device=DEV)
+        return _best_ms(lambda: ann.ann_build_graph(dx, len(x), 16, ann.F32, 64, 32, 1.0, g), 3)
+    plain = ms(np.random.default_rng(1).standard_normal((20_000, 16)).astype(np.float32))
+    assert ms(_line(20_000)) <= 3.8 * plain
