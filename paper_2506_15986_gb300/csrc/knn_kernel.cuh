@@ -73,18 +73,24 @@ struct KnnArgs {
 };
 
 // A (query tile, base tile) pair in the order that CTAs take them: query tile tm's
-// j-th pair has base tile j * stride mod tiles_n.
+// j-th pair has base tile j * stride mod tiles_n.  (Tiles, and a CTA's pairs, are
+// counted in 32 bits: the epilogue's registers are few.)
 struct TileWalk {
-    int64_t tm, j, tn;
-    __device__ TileWalk(const KnnArgs &a, int64_t t) : tm(t / a.tiles_n), j(t - tm * a.tiles_n), tn(j * a.stride % a.tiles_n)
+    int tm, j;
+    unsigned tn;
+    __device__ TileWalk(const KnnArgs &a, int64_t t)
+        : tm(static_cast<int>(t / a.tiles_n)), j(static_cast<int>(t - static_cast<int64_t>(tm) * a.tiles_n)),
+          tn(static_cast<unsigned>(j * a.stride % a.tiles_n))
     {
     }
     __device__ void next(const KnnArgs &a)
     {
-        tn += a.stride;
-        tn -= tn >= a.tiles_n ? a.tiles_n : 0;
-        if (++j == a.tiles_n) {
-            j = tn = 0;
+        const unsigned n = static_cast<unsigned>(a.tiles_n);
+        tn += static_cast<unsigned>(a.stride);
+        tn -= tn >= n ? n : 0;
+        if (++j == static_cast<int>(n)) {
+            j = 0;
+            tn = 0;
             ++tm;
         }
     }
@@ -332,7 +338,8 @@ __global__ void __launch_bounds__(64 + 32 * EW, 1) knn_tile_kernel(const KnnArgs
     tc_fence_after();
     const uint32_t tmem = *slot;
     const int64_t T = a.tiles_m * a.tiles_n / a.unit, G = gridDim.x;
-    const int64_t t0 = blockIdx.x * T / G * a.unit, t1 = (blockIdx.x + 1) * T / G * a.unit;
+    const int64_t t0 = blockIdx.x * T / G * a.unit;
+    const int pairs = static_cast<int>((blockIdx.x + 1) * T / G * a.unit - t0);
     const int chunks = a.chunks;
     const bool resident = chunks * P <= kSlotsA;
 
@@ -366,9 +373,9 @@ __global__ void __launch_bounds__(64 + 32 * EW, 1) knn_tile_kernel(const KnnArgs
             };
             int64_t uses = 0;
             TileWalk at(a, t0);
-            for (int64_t t = t0; t < t1 && ok; ++t, at.next(a)) {
+            for (int t = 0; t < pairs && ok; ++t, at.next(a)) {
                 const int64_t tm = at.tm, tn = at.tn;
-                if (resident && (t == t0 || at.j == 0))
+                if (resident && (t == 0 || at.j == 0))
                     copy_resident(tm, uses++);
                 for (int c = 0; c < chunks && ok; ++c) {
                     const uint8_t *sa = a.A + (tm * chunks + c) * P * kImage, *sb = a.B + (tn * chunks + c) * P * kImage;
@@ -415,8 +422,8 @@ __global__ void __launch_bounds__(64 + 32 * EW, 1) knn_tile_kernel(const KnnArgs
                            (first && kk == 0) ? 0u : 1u);
             };
             TileWalk at(a, t0);
-            for (int64_t t = t0; t < t1 && ok; ++t, at.next(a)) {
-                const bool fresh = t == t0 || at.j == 0;
+            for (int t = 0; t < pairs && ok; ++t, at.next(a)) {
+                const bool fresh = t == 0 || at.j == 0;
                 if (fresh)
                     ++uses;
                 for (int c = 0; c < chunks && ok; ++c) {
@@ -478,7 +485,7 @@ __global__ void __launch_bounds__(64 + 32 * EW, 1) knn_tile_kernel(const KnnArgs
                         ++ph;
                     }
                 }
-                if (resident && (at.j == a.tiles_n - 1 || t == t1 - 1))
+                if (resident && (at.j == a.tiles_n - 1 || t == pairs - 1))
                     for (int s = 0; s < chunks * P; ++s)
                         tc_commit(&bars->empty_a[s]);
             }
@@ -503,9 +510,11 @@ __global__ void __launch_bounds__(64 + 32 * EW, 1) knn_tile_kernel(const KnnArgs
         float thr = 0.f, slack = 0.f, cut = 0.f;
         uint32_t cut_id = 0;
         int cnt = 0;
-        int64_t self = -1, list = -1, seg = 0;
+        uint32_t self = 0xffffffffu;
+        int64_t list = -1;
+        int seg = 0;
         uint64_t *mine = nullptr;
-        int64_t ph = 0;
+        unsigned ph = 0;
         bool ok = true, pad = false;
         if (half == 0)
             sthr[m] = sthr[kTile + m] = 0xffffffffu;
@@ -514,14 +523,13 @@ __global__ void __launch_bounds__(64 + 32 * EW, 1) knn_tile_kernel(const KnnArgs
                 a.ends[list] = make_uint2(static_cast<uint32_t>(cnt), __float_as_uint(thr));
         };
         TileWalk at(a, t0);
-        for (int64_t t = t0, tile = 0; t < t1 && ok; ++t, ++tile, at.next(a)) {
-            const int64_t tm = at.tm, tn = at.tn;
-            const bool fresh = t == t0 || at.j == 0;
+        for (int t = 0; t < pairs && ok; ++t, at.next(a)) {
+            const bool fresh = t == 0 || at.j == 0;
             if (fresh) {
                 end_list();
-                if (t != t0)
+                if (t != 0)
                     ++seg;
-                const int64_t row = tm * kTile + m;
+                const int64_t tm = at.tm, row = tm * kTile + m;
                 list = row * a.slots + kHalves * (blockIdx.x - cta_of_tile(tm * a.tiles_n / a.unit, T, G)) + half;
                 mine = a.lists + list * kCap;
                 // what the block of base rows before this one left (none: -1, NaN).
@@ -538,15 +546,15 @@ __global__ void __launch_bounds__(64 + 32 * EW, 1) knn_tile_kernel(const KnnArgs
                 const float nx = row < a.rows ? a.nx[row] : 0.f;
                 coef = nx == nx ? (isinf(nx) ? -FLT_MAX : a.ip ? -1.f : -2.f) : nx;
                 slack = score_slack(nx, nmax, a.dim, a.ip);
-                self = a.self ? a.row0 + row : -1;
+                self = a.self ? static_cast<uint32_t>(a.row0 + row) : 0xffffffffu;
                 pad = row >= a.rows;  // a padding row: no score is below its threshold
                 thr = pad ? -INFINITY : __uint_as_float(end.y);
                 cut = pad ? thr : __int_as_float(0x7fffffff);
                 cut_id = 0;
             }
             uint32_t *shared_thr = sthr + (seg & 1) * kTile;
-            const int b = static_cast<int>(tile & 1);
-            const int64_t c0 = tn * kTile;
+            const int b = t & 1;
+            const int64_t c0 = static_cast<int64_t>(at.tn) * kTile;
             if (half == 0) {
                 // (a NaN distance is ordered as -0: so is the score)
                 const float ny = c0 + m < a.n ? a.ny[c0 + m] : INFINITY;
@@ -640,7 +648,7 @@ __global__ void __launch_bounds__(64 + 32 * EW, 1) knn_tile_kernel(const KnnArgs
                 // the columns that pass, then every lane its own one after
                 // another: a few turns, not one for every column that passes
                 // in some lane
-                const int64_t id0 = a.col0 + c0 + half * kCols + cc;
+                const uint32_t id0 = static_cast<uint32_t>(a.col0 + c0) + half * kCols + cc;
                 unsigned todo = 0;
 #pragma unroll
                 for (int j = 0; j < 32; ++j)
@@ -650,14 +658,14 @@ __global__ void __launch_bounds__(64 + 32 * EW, 1) knn_tile_kernel(const KnnArgs
 #pragma unroll
                     for (int j = 0; j < 32; ++j)
                         equal |= (s[j] == cut ? 1u : 0u) << j;
-                    const int64_t ids = max(static_cast<int64_t>(0), cut_id - id0);
+                    const uint32_t ids = cut_id > id0 ? cut_id - id0 : 0;
                     if (thr == cut && ids < 32)
                         todo &= ~(equal & ~((1u << ids) - 1u));
                 }
                 if (width - cc < 32)
                     todo &= width > cc ? (1u << (width - cc)) - 1u : 0u;
-                if (self >= id0 && self < id0 + 32)
-                    todo &= ~(1u << static_cast<int>(self - id0));
+                if (self - id0 < 32)
+                    todo &= ~(1u << (self - id0));
                 const unsigned full = __ballot_sync(kFull, cnt + __popc(todo) > kCap);
                 if (full) {
                     const ListEnd end = compact_rows<kCap / 32, 32 * KPL>(full, cnt, mine, cut, cut_id);
