@@ -97,7 +97,10 @@ cudaMemPool_t builder_pool(bool make)
 cudaError_t builder_alloc(void **p, size_t bytes, cudaStream_t s)
 {
     bytes = std::max<size_t>(bytes, 16);
-    cudaMemPool_t pool = builder_pool(true);
+    // under capture the memory is the graph's, not a pool's
+    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+    const bool capturing = cudaStreamIsCapturing(s, &cs) != cudaSuccess || cs != cudaStreamCaptureStatusNone;
+    cudaMemPool_t pool = capturing ? nullptr : builder_pool(true);
     return pool ? cudaMallocFromPoolAsync(p, bytes, pool, s) : cudaMallocAsync(p, bytes, s);
 }
 

@@ -105,3 +105,42 @@ def test_kmeans_edges(n, dim, k, empty):
     m = np.bincount(at).max()
     assert np.abs(cent.cpu().numpy() - cent_o).max() <= m * 2.0**-24 * np.abs(x).max()
     np.testing.assert_allclose(obj, obj_o, rtol=1e-4, atol=1e-6)
+
+
+_FIRST = """
+import sys
+sys.path.insert(0, {root!r})
+import torch
+from paper_2506_15986_gb300 import ann
+dev = "cuda:0"
+gen = torch.Generator(device=dev).manual_seed(1)
+n, i32 = 5000, torch.int32
+x = torch.randn((n, 32), generator=gen, device=dev)
+ints = lambda hi, *s: torch.randint(hi, s, generator=gen, device=dev).to(i32)
+h = ann.ann_index_create(x, ints(n, n, 16), 0, ann.F32)
+q, target, cand, hubs = x[:64].clone(), ints(n, 64), ints(8, 64, 4), torch.arange(8, device=dev).to(i32)
+ev, ho = (torch.full((64, 4), -5, dtype=i32, device=dev) for _ in range(2))
+call = lambda: ann.ann_hub_costs(h, q, 64, target, cand, 4, hubs, 32, ev, ho)
+graph = torch.cuda.CUDAGraph()
+with torch.cuda.graph(graph):
+    call()
+graph.replay()
+torch.cuda.synchronize()
+got = ev.clone(), ho.clone()
+assert (got[0] > 0).all()
+call()
+torch.cuda.synchronize()
+assert torch.equal(got[0], ev) and torch.equal(got[1], ho)
+print("same")
+"""
+
+
+def test_a_label_search_captured_first_of_all():
+    # a process of its own, whose first builder scratch is the captured search's
+    import os
+    import subprocess
+    import sys
+    root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+    r = subprocess.run([sys.executable, "-c", _FIRST.format(root=root)], capture_output=True, text=True,
+                       timeout=300)
+    assert r.returncode == 0 and "same" in r.stdout, r.stderr[-2000:]
