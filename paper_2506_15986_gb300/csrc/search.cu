@@ -408,7 +408,10 @@ ann_status launch_search(ann_index *idx, const SearchLaunch &L, cudaStream_t s)
         };
         // a table for three times the typical evaluations, at most 32 KB
         const int table = std::min(13, default_spill_bits(p->L));
-        const int tables[2] = {p->hash_bits ? p->hash_bits : table, p->hash_bits ? p->hash_bits : -1};
+        // without it the visited set has the global tables only, which must hold as
+        // much (they do unless the caller asks for small ones)
+        const int none = sb + 2 >= table ? -1 : table;
+        const int tables[2] = {p->hash_bits ? p->hash_bits : table, p->hash_bits ? p->hash_bits : none};
         const int kRows[] = {32, 24, 16, 12, 8, 4};
         const int r0 = want < kFullTeams ? 0 : 1, r1 = a.stage_stride > 1024 ? 6 : 5;
         bool fits = false;

@@ -438,3 +438,20 @@ def test_int8_distance_forms_are_bit_identical(metric, dim):
                 assert np.array_equal(u.view(np.int32), v.view(np.int32))
     finally:
         ann.ann_free_index(h)
+
+
+def test_small_spill_tables_of_a_large_batch():
+    # about 4,800 evaluations a query: more than the global tables of spill_bits =
+    # 10 hold, so the shared table stays although it costs the batch occupancy
+    rng = np.random.default_rng(1)
+    x = rng.standard_normal((5_000, 16)).astype(np.float32)
+    g = rng.integers(0, 5_000, size=(5_000, 32)).astype(np.int32)
+    q = rng.standard_normal((5_000, 16)).astype(np.float32)
+    h = make_index(x, g, 0)
+    try:
+        a = search(h, q, 10, 512, W=4)
+        b = search(h, q, 10, 512, W=4, spill_bits=10)
+    finally:
+        ann.ann_free_index(h)
+    assert a[4] == ann.OK and b[4] == ann.OK
+    assert a[2].max() > 3072 and all(np.array_equal(u, v) for u, v in zip(a[:4], b[:4]))
