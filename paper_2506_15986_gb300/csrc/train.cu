@@ -218,6 +218,24 @@ __global__ void __launch_bounds__(128) gemm_kernel(const GemmArgs g, const int e
     }
 }
 
+// Shared memory of a GEMM with `stages` stages: at most 512 / BN CTAs fit an SM's
+// 228 KB, so that they never ask for more than its 512 TMEM columns.
+template <int BN>
+constexpr int gemm_smem(int stages)
+{
+    return std::max(stages * (16384 + BN * 128) + 64, 228 * 1024 / (512 / BN + 1) + 1);
+}
+
+// The kernel's limit, which belongs to the device and not to a launch: the most
+// that any GEMM takes, so that trainers of several threads never lower it
+// between another one's look at it and its launch.
+template <int BN>
+cudaError_t gemm_limit()
+{
+    return cudaFuncSetAttribute(gemm_kernel<BN>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                gemm_smem<BN>(kGemmStages));
+}
+
 // Queues one GEMM.  With EPI_STORE and few output tiles over a long reduction
 // K is split over CTAs, at least min_k columns each, that add into `out`, which
 // the caller has zeroed.
@@ -238,13 +256,7 @@ ann_status gemm(const GemmArgs &g, cudaStream_t s, bool chained, int epi = EPI_S
     }
     const int64_t chunks = ((h.ksplit ? h.ksplit : g.K) + 63) / 64;
     h.stages = static_cast<int>(std::min<int64_t>(kGemmStages, chunks));
-    // at most 512 / BN CTAs fit an SM's 228 KB, so that they never ask for
-    // more than its 512 TMEM columns
-    const int smem = std::max(h.stages * (16384 + BN * 128) + 64, 228 * 1024 / (512 / BN + 1) + 1);
-    cudaError_t e = cudaFuncSetAttribute(gemm_kernel<BN>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-    if (e != cudaSuccess)
-        return cuda_status(e);
-    launch_next(chained, gemm_kernel<BN>, grid, 128, smem, s, h, epi);
+    launch_next(chained, gemm_kernel<BN>, grid, 128, gemm_smem<BN>(h.stages), s, h, epi);
     return cuda_status(cudaGetLastError());
 }
 
@@ -889,7 +901,8 @@ ann_status ann_trainer_create(int device, int32_t in_dim, int32_t n_hubs, const 
     if (cudaFuncSetAttribute(infonce_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxTrainHubs) !=
             cudaSuccess ||
         cudaFuncSetAttribute(infonce_rows_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             kRowWarps * kRowHubs) != cudaSuccess)
+                             kRowWarps * kRowHubs) != cudaSuccess ||
+        gemm_limit<64>() != cudaSuccess || gemm_limit<128>() != cudaSuccess || gemm_limit<256>() != cudaSuccess)
         return ANN_ERR_CUDA;
     ann_trainer *t = new (std::nothrow) ann_trainer();
     if (!t)

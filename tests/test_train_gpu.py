@@ -216,3 +216,37 @@ def test_a_captured_step_gives_the_direct_steps_gradients():
         out.append(gr)
     for k in out[0]:
         assert _rel(out[1][k], out[0][k]) <= 1e-5, k
+
+
+def test_trainers_of_two_threads():
+    # two threads train on one GPU, their GEMMs with rings of four stages and of
+    # one: every step launches, and both end where they end alone
+    import threading
+    probs = [_problem(B=2000, D=128, H=1000, seed=1), _problem(B=64, D=32, H=40, seed=2)]
+    epochs = (60, 3000)
+
+    def fit(i, out):
+        X, W1, b1, W2, b2, E, mask, _ = probs[i]
+        t = ann.ann_trainer_create(X.shape[1], W1, b1, W2, b2, E, len(X), tau=0.1, lr=1e-5)
+        try:
+            dX, labels = torch.from_numpy(X).to(DEV), dense_as_listed(mask)
+            losses = torch.zeros(epochs[i], device=DEV)
+            torch.cuda.synchronize()
+            ann.ann_trainer_fit(t, dX, len(X), *labels, None, epochs[i], losses, stream=torch.cuda.Stream())
+            out[i] = losses.cpu().numpy()
+        except ann.AnnError as e:
+            out[i] = e
+        finally:
+            ann.ann_trainer_free(t)
+
+    alone, both = {}, {}
+    for i in (0, 1):
+        fit(i, alone)
+    threads = [threading.Thread(target=fit, args=(i, both)) for i in (0, 1)]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    for i in (0, 1):
+        assert not isinstance(both[i], ann.AnnError), both[i]
+        np.testing.assert_allclose(both[i], alone[i], rtol=1e-4)  # split sums add in any order
