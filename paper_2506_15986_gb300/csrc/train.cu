@@ -704,12 +704,18 @@ void trainer_free(ann_trainer *t)
 {
     if (!t)
         return;
+    // the trainer's device, whichever is current: its kernels are waited for and
+    // its builder scratch is given back
+    int prev = 0;
+    cudaGetDevice(&prev);
+    cudaSetDevice(t->device);
     cudaDeviceSynchronize();
     for (void *p : t->owned)
         cudaFree(p);
     fusion_free(t->fu);
     delete t;
     builder_trim();
+    cudaSetDevice(prev);
 }
 
 // one Adam step over every parameter block
