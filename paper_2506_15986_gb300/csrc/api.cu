@@ -65,7 +65,28 @@ namespace {
 constexpr int kMaxDevices = 64;
 constexpr uint64_t kBuilderKeep = uint64_t{1} << 30;  // bytes a builder pool keeps between calls
 std::mutex g_builder_mu;
-cudaMemPool_t g_builder_pool[kMaxDevices] = {};
+struct BuilderPool {
+    cudaMemPool_t pool;
+    unsigned long long context;  // that the pool belongs to
+} g_builder_pool[kMaxDevices] = {};
+
+// The number of the current device's context (0: none, or the driver has no such
+// call).  A device reset ends the context and its pools; the next one has
+// another number.
+unsigned long long context_number()
+{
+    using GetIdFn = CUresult (*)(CUcontext, unsigned long long *);
+    static const GetIdFn get_id = [] {
+        void *fn = nullptr;
+        cudaDriverEntryPointQueryResult q{};
+        if (cudaGetDriverEntryPointByVersion("cuCtxGetId", &fn, 12000, cudaEnableDefault, &q) != cudaSuccess ||
+            q != cudaDriverEntryPointSuccess)
+            fn = nullptr;
+        return reinterpret_cast<GetIdFn>(fn);
+    }();
+    unsigned long long id = 0;
+    return get_id && get_id(nullptr, &id) == CUDA_SUCCESS ? id : 0;
+}
 
 // the current device's pool, made on first use (null: none can be made)
 cudaMemPool_t builder_pool(bool make)
@@ -74,7 +95,10 @@ cudaMemPool_t builder_pool(bool make)
     if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices)
         return nullptr;
     std::lock_guard<std::mutex> lock(g_builder_mu);
-    if (!g_builder_pool[dev] && make) {
+    BuilderPool &own = g_builder_pool[dev];
+    if (own.pool && own.context != context_number())
+        own.pool = nullptr;  // gone with its context
+    if (!own.pool && make) {
         cudaMemPoolProps props = {};
         props.allocType = cudaMemAllocationTypePinned;
         props.location.type = cudaMemLocationTypeDevice;
@@ -83,13 +107,13 @@ cudaMemPool_t builder_pool(bool make)
         uint64_t keep = kBuilderKeep;
         if (cudaMemPoolCreate(&p, &props) == cudaSuccess) {
             if (cudaMemPoolSetAttribute(p, cudaMemPoolAttrReleaseThreshold, &keep) == cudaSuccess)
-                g_builder_pool[dev] = p;
+                own = {p, context_number()};
             else
                 cudaMemPoolDestroy(p);
         }
         cudaGetLastError();
     }
-    return g_builder_pool[dev];
+    return own.pool;
 }
 
 }  // namespace

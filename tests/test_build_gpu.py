@@ -383,3 +383,45 @@ def test_graph_of_a_long_path_takes_no_longer_than_on_the_host():
         return _best_ms(lambda: ann.ann_build_graph(dx, len(x), 16, ann.F32, 64, 32, 1.0, g), 3)
     plain = ms(np.random.default_rng(1).standard_normal((20_000, 16)).astype(np.float32))
     assert ms(_line(20_000)) <= 3.8 * plain
+
+
+_RESET = """
+import ctypes, sys
+sys.path.insert(0, {root!r})
+import numpy as np
+from paper_2506_15986_gb300 import ann
+ann.load_library()
+rt = ctypes.CDLL("libcudart.so.13")  # the one that the library loaded
+rng = np.random.default_rng(1)
+x = rng.integers(-3, 4, size=(3000, 32)).astype(np.float32)
+
+def device(nbytes):
+    p = ctypes.c_void_p()
+    assert rt.cudaMalloc(ctypes.byref(p), ctypes.c_size_t(nbytes)) == 0
+    return p.value
+
+def knn():
+    base, ids, dd = device(x.nbytes), device(100 * 40), device(100 * 40)
+    assert rt.cudaMemcpy(ctypes.c_void_p(base), ctypes.c_void_p(x.ctypes.data), ctypes.c_size_t(x.nbytes), 1) == 0
+    ann.ann_knn(base, 3000, 32, ann.F32, ann.L2, base, 100, 10, ids, dd, stream=0)
+    out = np.empty((100, 10), np.int32)
+    assert rt.cudaMemcpy(ctypes.c_void_p(out.ctypes.data), ctypes.c_void_p(ids), ctypes.c_size_t(out.nbytes), 2) == 0
+    return out
+
+a = knn()
+assert rt.cudaDeviceReset() == 0
+b = knn()
+assert np.array_equal(a, b) and (a[:, 0] >= 0).all()
+print("same")
+"""
+
+
+def test_builders_after_a_device_reset():
+    # a process of its own resets its context between two calls: the scratch kept
+    # for the first one went with it
+    import os
+    import subprocess
+    import sys
+    root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+    r = subprocess.run([sys.executable, "-c", _RESET.format(root=root)], capture_output=True, text=True, timeout=300)
+    assert r.returncode == 0 and "same" in r.stdout, r.stderr[-2000:]
