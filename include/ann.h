@@ -298,6 +298,14 @@ ann_status ann_sync_status(ann_index *idx, void *stream);
  */
 ann_status ann_release_l2(ann_index *idx);
 
+/*
+ * Gives back the device memory that the builders (k-NN, graphs, clustering, the
+ * label search) keep between calls on a device, at most 1 GB; the next such
+ * call allocates again.  Freeing an index or a trainer of the device does the
+ * same.  Waits for the device.  ANN_ERR_CUDA for a device that is not there.
+ */
+ann_status ann_release_scratch(int device);
+
 /* ---- batching line: CUDA-graph plans and the autotuner -------------------- */
 
 typedef struct ann_plan ann_plan;
@@ -783,7 +791,7 @@ ann_status ann_merge_shards(const int32_t *d_ids, const void *d_dists, int32_t P
  *                otherwise)
  * Blocking: returns after the results are written.  Temporary device memory
  * (packed rows and candidate lists) comes from a pool of the device on `stream`;
- * the pool keeps at most 1 GB.
+ * the pool keeps at most 1 GB (ann_release_scratch).
  */
 ann_status ann_knn(const void *d_base, int64_t n, int32_t dim, int32_t dtype, int32_t metric,
                    const void *d_queries, int64_t nq, int32_t k, int32_t exclude_self,

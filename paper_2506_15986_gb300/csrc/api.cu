@@ -534,6 +534,17 @@ ann_status ann_search_batch(ann_index *idx, const void *d_queries, int64_t nq, c
     return launch_search(idx, L, static_cast<cudaStream_t>(stream));
 }
 
+ann_status ann_release_scratch(int device)
+{
+    int ndev = 0;
+    if (cudaGetDeviceCount(&ndev) != cudaSuccess || device < 0 || device >= ndev)
+        return ANN_ERR_CUDA;
+    DeviceGuard guard(device);
+    const cudaError_t e = cudaDeviceSynchronize();  // what is queued gives its scratch back first
+    builder_trim();
+    return cuda_status(e);
+}
+
 ann_status ann_release_l2(ann_index *idx)
 {
     if (!idx)

@@ -54,7 +54,8 @@ void scratch_free(ann_index *idx, void *p, cudaStream_t s);
 // freed with cudaFreeAsync.  It comes from a pool of the current device that
 // keeps at most 1 GB between calls: fresh device memory costs 2.3 ms a GB to
 // map, and one call's scratch is mostly the next one's.  What it keeps is given
-// back when an index or a trainer is freed.  Any thread, any stream.
+// back when an index or a trainer is freed, or by ann_release_scratch.  Any
+// thread, any stream.
 cudaError_t builder_alloc(void **p, size_t bytes, cudaStream_t s);
 void builder_trim();
 

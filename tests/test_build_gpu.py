@@ -425,3 +425,27 @@ def test_builders_after_a_device_reset():
     root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
     r = subprocess.run([sys.executable, "-c", _RESET.format(root=root)], capture_output=True, text=True, timeout=300)
     assert r.returncode == 0 and "same" in r.stdout, r.stderr[-2000:]
+
+
+def test_builders_give_their_scratch_back():
+    # a program that only calls the builders: what they keep is at most 1 GB, and
+    # ann_release_scratch returns it to the device
+    x = torch.randn((300_000, 256), device=DEV)
+    out = torch.empty((2000, 10), dtype=torch.int32, device=DEV), torch.empty((2000, 10), device=DEV)
+
+    def call():
+        ann.ann_knn(x, len(x), 256, ann.F32, ann.L2, x, 2000, 10, *out)
+        torch.cuda.synchronize()
+        return torch.cuda.mem_get_info()[0]
+    call()  # the kernels are loaded
+    ann.ann_release_scratch()
+    before = torch.cuda.mem_get_info()[0]
+    kept = before - call()
+    assert 0 < kept <= (1 << 30) + (64 << 20)  # and what a pool rounds up
+    ann.ann_release_scratch()
+    assert torch.cuda.mem_get_info()[0] == before
+    first = out[0].clone()
+    call()
+    assert torch.equal(out[0], first)
+    with pytest.raises(ann.AnnError):
+        ann.ann_release_scratch(99)
