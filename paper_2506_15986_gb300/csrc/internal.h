@@ -86,6 +86,8 @@ int default_team(int rowbytes);
 // log2 slots of the first global visited table when ann_search_params.
 // spill_bits is 0: 40 evaluations per pool slot below 3/4 load, 12..15.
 int default_spill_bits(int L);
+// Whether a gather mode left open means tensor gathers of four rows.
+bool opens_to_gathers(const ann_index *idx);
 
 // Scratch bytes launch_search needs for `teams` teams at the given params
 // (order_items: work items of a grouped work order, 0 without one).

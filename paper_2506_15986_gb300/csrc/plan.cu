@@ -146,6 +146,9 @@ ann_status ann_autotune(ann_index *idx, const void *d_queries, int64_t nq, const
         if (hb >= 8 && hb <= 15)
             hbs.push_back(hb);
     const int srs[] = {4, 6, 8, 12, 16};
+    // the first stages time bulk copies (unless the caller fixed the mode), also
+    // where a mode left open means tensor gathers: the fourth times those
+    const int gather = p->gather == 0 && ann::opens_to_gathers(idx) ? 1 : p->gather;
     float bms = 1e30f;
     ann_search_params bp = *p;
     // times one candidate: reps batches, batch r on lane r mod lanes; false on
@@ -191,6 +194,7 @@ ann_status ann_autotune(ann_index *idx, const void *d_queries, int64_t nq, const
             ann_search_params c = *p;
             c.hash_bits = hbs[h];
             c.stage_rows = sr;
+            c.gather = gather;
             c.team = p->team > 0 ? p->team : ann::default_team(idx->rowbytes);
             if (!(ok = trial(c)))
                 break;

@@ -278,6 +278,8 @@ int default_team(int rowbytes)
 
 int default_spill_bits(int L) { return spill_bits_for(L); }
 
+bool opens_to_gathers(const ann_index *idx) { return idx->has_row_map && idx->rowbytes <= 256; }
+
 size_t search_scratch_bytes(int teams, int spill_bits, int64_t order_items)
 {
     return 256 + static_cast<size_t>(teams) * (static_cast<size_t>(20) << spill_bits) +
@@ -334,7 +336,7 @@ ann_status launch_search(ann_index *idx, const SearchLaunch &L, cudaStream_t s)
     // copy per row (us, copies against gathers: 100 queries of 128-byte rows 283,
     // 268, 10,000 914, 823; 100 of 256-byte rows 376, 347; 10,000 of 512-byte rows
     // 1,179, 1,225; 1,000 of 1,024-byte rows 814, 918)
-    a.gather4 = idx->has_row_map && (p->gather == 4 || (p->gather == 0 && idx->rowbytes <= 256)) ? 1 : 0;
+    a.gather4 = p->gather == 0 ? opens_to_gathers(idx) : p->gather == 4 && idx->has_row_map;
     if (a.gather4)
         a.row_map = idx->row_map;
     // Lanes per distance: where it pays, four lanes stand for a team of eight, or a

@@ -164,3 +164,23 @@ def test_concurrent_batches_on_lanes(case):
     for j, ids, dd in outs:
         assert np.array_equal(ids.cpu().numpy(), ref[j][0])
         assert np.array_equal(dd.cpu().numpy(), ref[j][1])
+
+
+@pytest.mark.parametrize("dim", [64, 60])
+def test_autotune_times_both_gather_modes_of_short_rows(dim):
+    # rows of 256 bytes, which an open mode fetches by tensor gathers: the chosen
+    # sizes name the mode that was timed, copies or gathers; rows of 240 bytes have
+    # copies only, whatever the mode says
+    rng = np.random.default_rng(dim)
+    x = rng.standard_normal((5_000, dim)).astype(np.float32)
+    g = rng.integers(0, 5_000, size=(5_000, 16)).astype(np.int32)
+    h = ann.ann_index_create(x, g, 0, ann.F32, ann.L2)
+    try:
+        q, ids = _t(x[:300]), torch.empty((300, 10), dtype=torch.int32, device=DEV)
+        dd = torch.empty((300, 10), device=DEV)
+        best, _ = ann.ann_autotune(h, q, 300, None, ann.search_params(10, 64), ids, dd, reps=2)
+        assert best.gather in ((1, 4) if dim == 64 else (0, 4))
+        best, _ = ann.ann_autotune(h, q, 300, None, ann.search_params(10, 64, gather=4), ids, dd, reps=2)
+        assert best.gather == 4
+    finally:
+        ann.ann_free_index(h)
