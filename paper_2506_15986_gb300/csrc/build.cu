@@ -590,16 +590,16 @@ ann_status prune_rows(const void *d_base, int64_t n, int dim, int dtype, int K, 
         s16 += 1;
     const int stride = s16 * 16;
     // staged up to two CTAs an SM
-    const bool staged = static_cast<size_t>(K) * stride <= 108 * 1024;
+    constexpr int kStaged = 108 * 1024;  // also the kernel's limit whatever K is: a builder of another thread never lowers it
+    const bool staged = static_cast<size_t>(K) * stride <= kStaged;
     const size_t smem = staged ? static_cast<size_t>(K) * stride : 0;
     const uint8_t *bb = static_cast<const uint8_t *>(d_base);
     const unsigned grid = static_cast<unsigned>(n);
 #define PRUNE(DT, ST)                                                                                          \
     do {                                                                                                       \
-        CK(cudaFuncSetAttribute(rng_prune<DT, ST>, cudaFuncAttributeMaxDynamicSharedMemorySize,               \
-                                static_cast<int>(smem)));                                                      \
-        rng_prune<DT, ST><<<grid, 32 * kPruneWarps, smem, s>>>(bb, rowbytes, dim, n, cand, cand_d, K, R, alpha, stride,      \
-                                                 d_graph);                                                     \
+        CK(cudaFuncSetAttribute(rng_prune<DT, ST>, cudaFuncAttributeMaxDynamicSharedMemorySize, kStaged));     \
+        rng_prune<DT, ST><<<grid, 32 * kPruneWarps, smem, s>>>(bb, rowbytes, dim, n, cand, cand_d, K, R,       \
+                                                               alpha, stride, d_graph);                        \
     } while (0)
     if (dtype == ANN_U8 && staged)
         PRUNE(ANN_U8, true);

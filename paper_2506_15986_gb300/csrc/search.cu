@@ -507,15 +507,11 @@ ann_status launch_search(ann_index *idx, const SearchLaunch &L, cudaStream_t s)
         const size_t rs = static_cast<size_t>(P) * 8;
         const unsigned grid = static_cast<unsigned>(std::min<int64_t>(L.nq, static_cast<int64_t>(idx->num_sms) * 16));
         auto rk = idx->metric == ANN_IP ? rerank_kernel<ANN_IP> : rerank_kernel<ANN_L2>;
-        e = cudaFuncSetAttribute(rk, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(rs));
-        if (e == cudaSuccess) {
-            rk<<<grid, 32 * kRerankWarps, rs, s>>>(idx->d_base_f32, idx->dim,
-                                                    static_cast<const float *>(L.queries), L.nq, a.qdiv,
-                                                    a.pool_out, p->L, P, p->k, p->d_k, L.ids,
-                                                    static_cast<float *>(L.dists));
-            e = cudaGetLastError();
-        }
-        st = cuda_status(e);
+        static_assert(ANN_MAX_L * 8 <= 48 * 1024, "within every kernel's limit");
+        rk<<<grid, 32 * kRerankWarps, rs, s>>>(idx->d_base_f32, idx->dim, static_cast<const float *>(L.queries), L.nq,
+                                                a.qdiv, a.pool_out, p->L, P, p->k, p->d_k, L.ids,
+                                                static_cast<float *>(L.dists));
+        st = cuda_status(cudaGetLastError());
     }
     if (pool_buf)
         scratch_free(idx, pool_buf, s);

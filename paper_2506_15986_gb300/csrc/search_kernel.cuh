@@ -949,18 +949,24 @@ template <int DT, int MT>
 ann_status teams_for(ann_index *idx, size_t per_warp, int maxc, int form, int64_t nq, int *teams, int *wpc)
 {
     auto kern = kernel_for<DT, MT>(maxc, form);
+    // The kernel's limit belongs to the device and not to a launch: always the
+    // most a CTA may have, so that a search of another thread never lowers it
+    // between this one's look at it and its launch.
+    int cta_smem = 0;
+    cudaError_t e = cudaDeviceGetAttribute(&cta_smem, cudaDevAttrMaxSharedMemoryPerBlockOptin, idx->device);
+    if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, cta_smem);
+    if (e != cudaSuccess)
+        return cuda_status(e);
     int best = 0, best_w = 1;
     for (int w = 1; w <= kMaxSearchWarps; ++w) {
         if (static_cast<int64_t>(best) * idx->num_sms >= nq)
             break;
         const size_t smem = per_warp * w;
-        if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem)) !=
-            cudaSuccess) {
-            cudaGetLastError();  // too large for one CTA: not a candidate
-            continue;
-        }
+        if (smem > static_cast<size_t>(cta_smem))
+            break;  // too large for one CTA: not a candidate
         int per_sm = 0;
-        const cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, 32 * w, smem);
+        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, 32 * w, smem);
         if (e != cudaSuccess)
             return cuda_status(e);
         if (per_sm * w > best) {
@@ -970,10 +976,6 @@ ann_status teams_for(ann_index *idx, size_t per_warp, int maxc, int form, int64_
     }
     if (best < 1)
         return ANN_ERR_UNSUPPORTED;  // the per-query state does not fit in shared memory
-    const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                               static_cast<int>(per_warp * best_w));
-    if (e != cudaSuccess)
-        return cuda_status(e);
     *teams = best * idx->num_sms;
     *wpc = best_w;
     return ANN_OK;

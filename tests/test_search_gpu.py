@@ -455,3 +455,33 @@ def test_small_spill_tables_of_a_large_batch():
         ann.ann_free_index(h)
     assert a[4] == ann.OK and b[4] == ann.OK
     assert a[2].max() > 3072 and all(np.array_equal(u, v) for u, v in zip(a[:4], b[:4]))
+
+
+def test_searches_of_two_threads(f32_case):
+    # one index, searched by two threads with small and with large pools (whose
+    # shared memory differs): every search launches, with its usual results
+    import threading
+    q = f32_case["queries"][:100]
+    out = {}
+
+    def run(L):
+        h, dq, s = f32_case["h"], torch.from_numpy(q).to("cuda:0"), torch.cuda.Stream()
+        ids = torch.empty((100, 10), dtype=torch.int32, device="cuda:0")
+        dd = torch.empty((100, 10), device="cuda:0")
+        p = ann.search_params(10, L, W=4)
+        torch.cuda.synchronize()
+        try:
+            for _ in range(3000):
+                ann.ann_search_batch(h, dq, 100, None, p, ids, dd, stream=s)
+                s.synchronize()
+            out[L] = ids.cpu().numpy()
+        except ann.AnnError as e:
+            out[L] = e
+    threads = [threading.Thread(target=run, args=(L,)) for L in (16, 1024)]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    for L in (16, 1024):
+        assert not isinstance(out[L], ann.AnnError), out[L]
+        assert np.array_equal(out[L], search(f32_case["h"], q, 10, L, W=4)[0])
