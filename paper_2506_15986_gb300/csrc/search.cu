@@ -392,7 +392,10 @@ ann_status launch_search(ann_index *idx, const SearchLaunch &L, cudaStream_t s)
     // the longest round that still let every SM hold its share of the queries
     // (up to kFullTeams, where registers end; rounds past 24 rows gain only on
     // part-full SMs), else no table, and rounds of eight rows, or of four when
-    // rows pass 1 KB (d = 384 fp32: 2,770 us with four, 3,240 with eight).
+    // rows pass 1 KB (d = 384 fp32: 2,770 us with four, 3,240 with eight), but
+    // never fewer than the warp takes at once, which are many when the caller
+    // fixed a small team (6,000 queries at d = 960 fp16, teams of two: 2,285 us
+    // with four rows, 1,300 with the sixteen that it takes).
     // Measured (us, shared table sized for 12 evaluations per
     // pool slot and rounds of 16 before, this rule after): 100,000 queries of
     // mixed L <= 512 at d = 96: 78,600 -> 28,300; 10,000 at d = 200, L = 256:
@@ -415,7 +418,10 @@ ann_status launch_search(ann_index *idx, const SearchLaunch &L, cudaStream_t s)
         const int none = sb + 2 >= table ? -1 : table;
         const int tables[2] = {p->hash_bits ? p->hash_bits : table, p->hash_bits ? p->hash_bits : none};
         const int kRows[] = {32, 24, 16, 12, 8, 4};
-        const int r0 = want < kFullTeams ? 0 : 1, r1 = a.stage_stride > 1024 ? 6 : 5;
+        int r0 = want < kFullTeams ? 0 : 1, r1 = a.stage_stride > 1024 ? 6 : 5;
+        while (r1 > 1 && kRows[r1 - 1] < 32 >> a.team_lg)
+            --r1;
+        r0 = std::min(r0, r1 - 1);
         bool fits = false;
         for (int t = 0; t < 2 && !fits; ++t) {
             if (p->stage_rows > 0) {

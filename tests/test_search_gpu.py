@@ -485,3 +485,45 @@ def test_searches_of_two_threads(f32_case):
     for L in (16, 1024):
         assert not isinstance(out[L], ann.AnnError), out[L]
         assert np.array_equal(out[L], search(f32_case["h"], q, 10, L, W=4)[0])
+
+
+def _long_rows(dtype, dim, nq):
+    """An index of 960-d rows and a function that times a search of it (ms)."""
+    rng = np.random.default_rng(dim)
+    x = rng.standard_normal((5_000, dim)).astype(np.float32)
+    g = rng.integers(0, 5_000, size=(5_000, 32)).astype(np.int32)
+    dx = torch.from_numpy(x).to("cuda:0")
+    rows = dx.half()
+    if dtype == ann.I8S:
+        rows = torch.empty((5_000, ann.ann_i8s_row_bytes(dim)), dtype=torch.uint8, device="cuda:0")
+        ann.ann_quantize_i8s(dx, 5_000, dim, rows)
+    h = ann.ann_index_create(rows, torch.from_numpy(g).to("cuda:0"), 0, dtype, n=5_000, dim=dim, degree=32)
+    q = dx.repeat(2, 1)[:nq].contiguous()
+    ids = torch.empty((nq, 10), dtype=torch.int32, device="cuda:0")
+    dd = torch.empty((nq, 10), device="cuda:0")
+
+    def ms(**knobs):
+        p = ann.search_params(10, 16, W=4, **knobs)
+        out = []
+        for _ in range(7):
+            a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+            a.record()
+            ann.ann_search_batch(h, q, nq, None, p, ids, dd)
+            b.record()
+            b.synchronize()
+            out.append(a.elapsed_time(b))
+        return min(out[2:]), ids.clone()
+    return h, ms
+
+
+@pytest.mark.parametrize("dtype,team", [(ann.F16, 2), (ann.I8S, 4)])
+def test_open_rounds_fill_the_warp(dtype, team):
+    # a small team fixed, the round left open: as many rows as the warp takes at
+    # once, so no slower than asking for rounds of sixteen
+    h, ms = _long_rows(dtype, 960, 6_000)
+    try:
+        (a, ia), (b, ib) = ms(team=team, hash_bits=-1), ms(team=team, hash_bits=-1, stage_rows=16)
+        assert torch.equal(ia, ib) and a <= 1.1 * b, (a, b)
+        ms(team=1)  # 32 rows at once: the longest round, or what fits
+    finally:
+        ann.ann_free_index(h)
