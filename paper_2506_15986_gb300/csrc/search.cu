@@ -216,15 +216,18 @@ size_t align_up(size_t v, size_t a) { return (v + a - 1) / a * a; }
 // 2,030 -> 1,389, by twos 1,529; 1,000, d = 960: 1,051 by twos, 978); 16-bit and int8
 // rows by twos (3,000, d = 960 fp16: 1,738 -> 1,383; by fours registers spill:
 // 1,397, and 1,209 -> 1,412 at d = 200).  Teams of four gain nothing (d = 128
-// fp16: 1,040, 1,034; uint8: 792, 795).
-int search_form(int dtype, int chunks, int G, bool gather4)
+// fp16: 1,040, 1,034; uint8: 792, 795).  A round (`rows`, 0: left open) that the
+// teams take at once, one row each, leaves half of them idle by twos (one query, d
+// = 960 int8, teams of eight, rounds of four: 447 us by twos, 311 by one).
+int search_form(int dtype, int chunks, int G, bool gather4, int rows)
 {
     if (dtype == ANN_U8)
         return kOne;
     if (!gather4 && G >= 8) {
         if (G == 8 && chunks == 4 * G && dtype != ANN_I8S)
             return kPair4;
-        return dtype == ANN_F32 && G > 8 ? kRows4 : kRows2;
+        if (rows == 0 || rows * G > 32)
+            return dtype == ANN_F32 && G > 8 ? kRows4 : kRows2;
     }
     return dtype != ANN_I8S && chunks == 8 * G ? kOne8 : kOne;
 }
@@ -344,7 +347,7 @@ ann_status launch_search(ann_index *idx, const SearchLaunch &L, cudaStream_t s)
     // and shuffles; the distances are bit for bit those of G lanes a row.  Tensor
     // gathers write rows back to back, where few lanes a row or neighbouring
     // rows at once would meet bank conflicts: they keep G lanes a row.
-    const int form = search_form(idx->dtype, chunks, G, a.gather4);
+    const int form = search_form(idx->dtype, chunks, G, a.gather4, p->stage_rows);
     const int P = idx->dtype == ANN_U8 && !a.gather4 ? std::min(G, 4) : form == kPair4 ? G / 2 : G;
     a.team_lg = 0;
     while ((1 << a.team_lg) < P)

@@ -527,3 +527,14 @@ def test_open_rounds_fill_the_warp(dtype, team):
         ms(team=1)  # 32 rows at once: the longest round, or what fits
     finally:
         ann.ann_free_index(h)
+
+
+def test_short_rounds_keep_every_team_busy():
+    # rounds of as many rows as the warp has teams: a row each, not two for half of
+    # them (rounds of four took 1.27 times what rounds of eight take here)
+    h, ms = _long_rows(ann.I8S, 960, 1)
+    try:
+        (a, ia), (b, ib) = ms(team=8, stage_rows=4), ms(team=8, stage_rows=8)
+        assert torch.equal(ia, ib) and a <= 1.27 * b, (a, b)
+    finally:
+        ann.ann_free_index(h)
