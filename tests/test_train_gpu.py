@@ -250,3 +250,37 @@ def test_trainers_of_two_threads():
     for i in (0, 1):
         assert not isinstance(both[i], ann.AnnError), both[i]
         np.testing.assert_allclose(both[i], alone[i], rtol=1e-4)  # split sums add in any order
+
+
+def test_a_captured_step_reads_its_inputs_when_it_is_replayed():
+    # the queries, the batch and the labels change between the capture and its
+    # replay: the gradients that come out are the new batch's, as a direct step
+    # gives them, and not what an earlier step left
+    X, W1, b1, W2, b2, E, mask, rows = _problem(B=700)
+    X2, *_, mask2, rows2 = _problem(B=700, seed=9)
+    grads = {}
+    for captured in (False, True):
+        t = ann.ann_trainer_create(128, W1, b1, W2, b2, E, 700, tau=0.1, lr=1e-3)
+        try:
+            cand, lab, M = dense_as_listed(mask if captured else mask2)
+            x, r = torch.from_numpy(X if captured else X2).to(DEV), torch.from_numpy(rows if captured else rows2).to(DEV)
+            step = lambda: ann.load_library().ann_trainer_step(  # noqa: E731
+                t, x.data_ptr(), r.data_ptr(), len(rows), cand.data_ptr(), lab.data_ptr(), M, 0, None,
+                torch.cuda.current_stream().cuda_stream)
+            assert step() == ann.OK
+            if captured:
+                torch.cuda.synchronize()
+                g = torch.cuda.CUDAGraph()
+                with torch.cuda.graph(g):
+                    assert step() == ann.OK
+                for old, new in ((x, X2), (r, rows2), (lab, mask2)):
+                    old.copy_(torch.from_numpy(np.ascontiguousarray(new)))
+                g.replay()
+            torch.cuda.synchronize()
+            gr = {k: np.zeros_like(v) for k, v in dict(W1=W1, b1=b1, W2=W2, b2=b2, E=E).items()}
+            ann.ann_trainer_get(t, gr["W1"], gr["b1"], gr["W2"], gr["b2"], gr["E"], gradients=True)
+        finally:
+            ann.ann_trainer_free(t)
+        grads[captured] = gr
+    for k in grads[False]:
+        assert _rel(grads[True][k], grads[False][k]) <= 1e-5, k
