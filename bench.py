@@ -138,14 +138,15 @@ def kernel_digest():
     """Digest of the sources that define the search kernel, comments and
     blank space left out (a comment edit does not change the kernel), and the
     public header's function prototypes too (a new entry point does not)."""
+    import glob
     import hashlib
     import re
     h = hashlib.sha1()
-    for rel in ("paper_2506_15986_gb300/csrc/search.cu", "paper_2506_15986_gb300/csrc/search_kernel.cuh",
-                "paper_2506_15986_gb300/csrc/device_util.cuh", "paper_2506_15986_gb300/csrc/internal.h",
-                "include/ann.h"):
-        if not os.path.exists(os.path.join(ROOT, rel)):
-            continue
+    csrc = "paper_2506_15986_gb300/csrc"
+    kernel = [f"{csrc}/{os.path.basename(f)}" for f in sorted(glob.glob(os.path.join(ROOT, csrc, "search*.cu*")))]
+    if not kernel:
+        raise FileNotFoundError(f"no search kernel source in {csrc}")
+    for rel in (*kernel, f"{csrc}/device_util.cuh", f"{csrc}/internal.h", "include/ann.h"):
         with open(os.path.join(ROOT, rel), encoding="utf-8") as f:
             src = f.read()
         src = re.sub(r"/\*.*?\*/", " ", src, flags=re.S)

@@ -84,3 +84,24 @@ def test_hub_graph_options(monkeypatch):
     args = bench.parse()
     assert args.hub_graph == "16:0" and args.l_hub == 16 and args.hub_seeds == 32
     assert [item.split(":") for item in args.nav_sweep.split(",")] == [["16", "0", "16", "32"], ["32", "32"]]
+
+
+def test_kernel_digest_follows_every_search_source(tmp_path, monkeypatch):
+    # whatever the search kernel's files are called, an edit of one is an edit of
+    # the kernel, and without any there is nothing to tie a measurement to
+    root = tmp_path / "r"
+    shutil.copytree(os.path.join(bench.ROOT, "include"), root / "include")
+    csrc = root / "paper_2506_15986_gb300/csrc"
+    csrc.mkdir(parents=True)
+    for f in os.listdir(os.path.join(bench.ROOT, "paper_2506_15986_gb300/csrc")):
+        shutil.copy(os.path.join(bench.ROOT, "paper_2506_15986_gb300/csrc", f), csrc / f)
+    monkeypatch.setattr(bench, "ROOT", str(root))
+    (csrc / "search_kernel.cuh").rename(csrc / "search_steps.cuh")
+    d = bench.kernel_digest()
+    with open(csrc / "search_steps.cuh", "a") as f:
+        f.write("int another;\n")
+    assert bench.kernel_digest() != d
+    for f in csrc.glob("search*"):
+        f.unlink()
+    with pytest.raises(FileNotFoundError):
+        bench.kernel_digest()
