@@ -422,7 +422,7 @@ __global__ void __launch_bounds__(32 * kRowWarps)
                         const int32_t *rowmap, __nv_bfloat16 *dS, int64_t ldS, float *row_loss, int *valid)
 {
     begin_chained();
-    extern __shared__ int8_t lrow_all[];
+    extern __shared__ __align__(16) int8_t lrow_all[];
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     const int64_t r = blockIdx.x * static_cast<int64_t>(kRowWarps) + wid;
     if (r >= B)
