@@ -95,8 +95,8 @@ __device__ __forceinline__ void load_tile(uint8_t *tile, const Mat &m, int64_t r
 // Staging each K chunk, waiting for its MMAs and storing a row per lane took
 // 339 us for the six GEMMs of a step (8,192 rows, 1,024 hubs); 108 us here,
 // bounded by load latency and, for the logits, by the 34 MB they write.
-template <int BN>
-__global__ void __launch_bounds__(128) gemm_kernel(const GemmArgs g, const int epi)
+template <int BN, int EPI>
+__global__ void __launch_bounds__(128) gemm_kernel(const GemmArgs g)
 {
     begin_chained();
     extern __shared__ __align__(1024) uint8_t smem[];
@@ -173,7 +173,7 @@ __global__ void __launch_bounds__(128) gemm_kernel(const GemmArgs g, const int e
         for (int cc = 0; cc < BN && c0 + cc < g.N; cc += 32) {
             float v[32];
             tmem_ld32(my_lane + cc, v);
-            if (epi == EPI_HIDDEN) {
+            if constexpr (EPI == EPI_HIDDEN) {
                 const uint32_t mask = row < g.M ? g.mask[((c0 + cc) >> 5) * g.ldt + row] : 0u;
 #pragma unroll
                 for (int j = 0; j < 32; ++j) {
@@ -227,27 +227,29 @@ constexpr int gemm_smem(int stages)
 }
 
 // The kernel's limit, which belongs to the device and not to a launch: the most
-// that any GEMM takes, so that trainers of several threads never lower it
-// between another one's look at it and its launch.
-template <int BN>
-cudaError_t gemm_limit()
+// that any of its GEMMs takes, so that trainers of several threads never lower
+// it between another one's look at it and its launch.  (No more than that: with
+// the limit of the 256-wide split GEMM on the one with the hidden layer's
+// epilogue too, a step took 1 % longer.)
+template <int BN, int EPI>
+cudaError_t gemm_limit(int stages)
 {
-    return cudaFuncSetAttribute(gemm_kernel<BN>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                gemm_smem<BN>(kGemmStages));
+    return cudaFuncSetAttribute(gemm_kernel<BN, EPI>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                gemm_smem<BN>(stages));
 }
 
 // Queues one GEMM.  With EPI_STORE and few output tiles over a long reduction
 // K is split over CTAs, at least min_k columns each, that add into `out`, which
 // the caller has zeroed.
-template <int BN>
-ann_status gemm(const GemmArgs &g, cudaStream_t s, bool chained, int epi = EPI_STORE, int64_t min_k = 512)
+template <int BN, int EPI = EPI_STORE>
+ann_status gemm(const GemmArgs &g, cudaStream_t s, bool chained, int64_t min_k = 512)
 {
     dim3 grid(static_cast<unsigned>((g.M + 127) / 128), static_cast<unsigned>((g.N + BN - 1) / BN));
     // up to about two CTAs per SM
     GemmArgs h = g;
     h.ksplit = 0;
     const int64_t tiles = static_cast<int64_t>(grid.x) * grid.y;
-    if (epi == EPI_STORE && tiles < 128 && g.K >= 1024) {
+    if (EPI == EPI_STORE && tiles < 128 && g.K >= 1024) {
         const int64_t want = std::min<int64_t>(g.K / min_k, std::max<int64_t>(1, 256 / tiles));
         if (want > 1) {
             h.ksplit = ((g.K + want - 1) / want + 63) / 64 * 64;
@@ -256,7 +258,7 @@ ann_status gemm(const GemmArgs &g, cudaStream_t s, bool chained, int epi = EPI_S
     }
     const int64_t chunks = ((h.ksplit ? h.ksplit : g.K) + 63) / 64;
     h.stages = static_cast<int>(std::min<int64_t>(kGemmStages, chunks));
-    launch_next(chained, gemm_kernel<BN>, grid, 128, gemm_smem<BN>(h.stages), s, h, epi);
+    launch_next(chained, gemm_kernel<BN, EPI>, grid, 128, gemm_smem<BN>(h.stages), s, h);
     return cuda_status(cudaGetLastError());
 }
 
@@ -718,7 +720,6 @@ void trainer_free(ann_trainer *t)
     cudaSetDevice(prev);
 }
 
-// one Adam step over every parameter block
 // A step is a chain of some fifteen short kernels: each one's launch overlaps
 // the one before, except under capture, which records plain dependencies.  A
 // step at batch 8,192: 323 us without, 294 here.
@@ -728,6 +729,7 @@ bool may_chain(cudaStream_t s)
     return cudaStreamIsCapturing(s, &cs) == cudaSuccess && cs == cudaStreamCaptureStatusNone;
 }
 
+// one Adam step over every parameter block
 void adam_all(ann_trainer *t, cudaStream_t s)
 {
     const bool chained = may_chain(s);
@@ -831,7 +833,7 @@ ann_status trainer_grads(ann_trainer *t, const float *d_queries, const int32_t *
     g.K = B;
     g.out = t->dEh;
     // (sums that no later rounding to BF16 reads are split further)
-    if ((st = gemm<64>(g, s, chained, EPI_STORE, 256)) != ANN_OK)
+    if ((st = gemm<64>(g, s, chained, 256)) != ANN_OK)
         return st;
     // through the normalisations
     launch_next(chained, query_backward_kernel, blocks_for(B, 32), 256, 0, s, t->qhat, t->tower.nrm, t->dQ, B, t->dZ2,
@@ -852,7 +854,7 @@ ann_status trainer_grads(ann_trainer *t, const float *d_queries, const int32_t *
     g.alpha = 1.f;
     g.out = t->grads + o.W2;
     g.ldo = 64;
-    if ((st = gemm<64>(g, s, chained, EPI_STORE, 256)) != ANN_OK)
+    if ((st = gemm<64>(g, s, chained, 256)) != ANN_OK)
         return st;
     // dZ1 = (dZ2 W2^T) * [Z1 > 0]  (B x 256, K = 64), written transposed, with db1's partial sums
     g = GemmArgs{};
@@ -867,7 +869,7 @@ ann_status trainer_grads(ann_trainer *t, const float *d_queries, const int32_t *
     g.outT = t->dZ1T;
     g.ldt = t->ldB;
     g.part = t->part1;
-    if ((st = gemm<256>(g, s, chained, EPI_HIDDEN)) != ANN_OK)
+    if ((st = gemm<256, EPI_HIDDEN>(g, s, chained)) != ANN_OK)
         return st;
     launch_next(chained, bias_sum_kernel, 10, 1024, 0, s, t->part1, (B + 127) / 128 * 4, t->part2, (B + 31) / 32,
                 t->grads + o.b1, t->grads + o.b2);
@@ -882,7 +884,7 @@ ann_status trainer_grads(ann_trainer *t, const float *d_queries, const int32_t *
     g.alpha = 1.f;
     g.out = t->grads + o.W1;
     g.ldo = 256;
-    if ((st = gemm<256>(g, s, chained, EPI_STORE, 256)) != ANN_OK)
+    if ((st = gemm<256>(g, s, chained, 256)) != ANN_OK)
         return st;
     return cuda_status(cudaGetLastError());
 }
@@ -908,7 +910,10 @@ ann_status ann_trainer_create(int device, int32_t in_dim, int32_t n_hubs, const 
             cudaSuccess ||
         cudaFuncSetAttribute(infonce_rows_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              kRowWarps * kRowHubs) != cudaSuccess ||
-        gemm_limit<64>() != cudaSuccess || gemm_limit<128>() != cudaSuccess || gemm_limit<256>() != cudaSuccess)
+        gemm_limit<64, EPI_STORE>(kGemmStages) != cudaSuccess ||
+        gemm_limit<128, EPI_STORE>(1) != cudaSuccess ||   // the logits: K = 64
+        gemm_limit<256, EPI_HIDDEN>(1) != cudaSuccess ||  // dZ1: K = 64
+        gemm_limit<256, EPI_STORE>(kGemmStages) != cudaSuccess)
         return ANN_ERR_CUDA;
     ann_trainer *t = new (std::nothrow) ann_trainer();
     if (!t)
