@@ -336,8 +336,7 @@ __global__ void __launch_bounds__(32 * W)
     __shared__ float pen[kMaxBranch];
     __shared__ int size[kMaxBranch];
     __shared__ unsigned mask[W][kMaxBranch];   // the warp's lanes that assume a child
-    __shared__ unsigned moved[2];              // warps with a member that changed in this pass, and in the last
-    __shared__ int moves[2];                   // such members
+    __shared__ int first_open;                 // the first warp with a member that changed
     __shared__ int2 won[32 * W];               // members decided one by one: child and rank
     const int64_t c = blockIdx.x;
     const int64_t b = seg[c], e = seg[c + 1];
@@ -361,8 +360,6 @@ __global__ void __launch_bounds__(32 * W)
     __syncthreads();
     for (int64_t i0 = b; i0 < e; i0 += 32 * W) {
         const bool live = i0 + tid < e;
-        if (tid < 2)
-            moved[tid] = moves[tid] = 0;
         uint32_t o1 = 0xffffffffu, o2 = 0xffffffffu;
         int j1 = 0, j2 = 0;
         float d1 = 0.f;
@@ -392,8 +389,6 @@ __global__ void __launch_bounds__(32 * W)
             if (live)
                 atomicOr(&mask[w][my], 1u << lane);
             __syncthreads();
-            if (tid == 0)  // the next pass's, read before this pass's first meeting
-                moved[(pass + 1) & 1] = moves[(pass + 1) & 1] = 0;
             int fl = size[lane];  // lane = child: its size when the warp's members come
 #pragma unroll
             for (int v = 0; v < W - 1; ++v)
@@ -417,19 +412,19 @@ __global__ void __launch_bounds__(32 * W)
                     my = win;
                 }
             }
-            const int here = __popc(__ballot_sync(kAll, changed));
-            if (lane == 0 && here > 0) {
-                atomicOr(&moved[pass & 1], 1u << w);
-                atomicAdd(&moves[pass & 1], here);
-            }
-            __syncthreads();
-            const unsigned open_warps = moved[pass & 1];
-            if (!open_warps)
+            const int moves = __syncthreads_count(changed);
+            if (moves == 0)
                 break;
-            if (pass + 1 < kVisitPasses && moves[pass & 1] < 4 * W)
+            if (pass + 1 < kVisitPasses && moves < 4 * W)
                 continue;
             alone = true;
-            const int w0 = __ffs(open_warps) - 1;
+            if (tid == 0)
+                first_open = W;
+            __syncthreads();
+            if (changed)
+                atomicMin(&first_open, w);
+            __syncthreads();
+            const int w0 = first_open;
             if (w == 0) {  // lane = child, as hb_visit_warp
                 int cj = size[lane];
                 for (int v = 0; v < w0; ++v)
@@ -743,7 +738,7 @@ ann_status ann_hbkm(const float *d_x, int64_t n, int32_t dim, int32_t k, int32_t
         if (nc > kMaxClusters)
             return ANN_ERR_INVALID_ARG;
     }
-    if (static_cast<size_t>(k) * dim * 4 > 227 * 1024)
+    if (static_cast<size_t>(k) * dim * 4 > 227 * 1024)  // the interface's bound, no kernel's here
         return ANN_ERR_UNSUPPORTED;
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     HB_CK(cudaFuncSetAttribute(hb_visit<kVisitWarps>, cudaFuncAttributeMaxDynamicSharedMemorySize, kVisitSmem));
