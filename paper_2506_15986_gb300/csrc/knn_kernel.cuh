@@ -4,8 +4,9 @@
 // Scores |y|^2 - 2 x.y (or -x.y) of every (query, base) pair come from
 // tcgen05 tensor cores and never reach memory: a CTA keeps 128 queries as the
 // A operand, streams the base through in tiles of 128 rows, and its epilogue
-// warps keep each query's best KP candidates.  Those are then re-scored exactly
-// (direct differences: int32 for uint8, fp32 otherwise) and sorted by
+// warps keep each query's best KP candidates (64 up to k = 32, else 128).  Of
+// those, the ones that the scores' errors leave in question are then re-scored
+// exactly (direct differences: int32 for uint8, fp32 otherwise) and sorted by
 // (distance, id).
 //
 // Precision of the scores.  An fp32 value is the exact sum of three BF16 values
@@ -37,6 +38,7 @@
 namespace ann {
 namespace {
 
+constexpr int kEpiWarps = 8;          // epilogue warps of a CTA
 constexpr int kTile = 128;            // queries, and base rows, of one MMA tile
 constexpr int kImage = kTile * 128;   // bytes of a tile's 64-wide K chunk of one plane
 constexpr int kSlotsA = 6, kSlotsB = 8;  // images in the operands' rings
@@ -66,7 +68,7 @@ struct KnnArgs {
     int64_t unit;          // CTAs take ranges of this many (query tile, base tile) pairs: 1 or tiles_n
     int ip, self;          // inner product; skip the query's own index
     int dim, k;
-    uint64_t *lists;       // [rows rounded up to kTile][slots][list_keys(KR)] candidate keys
+    uint64_t *lists;       // [rows rounded up to kTile][slots][list_keys(KPL, KR)] candidate keys
     uint2 *ends;           // [rows rounded up to kTile][slots] a list's length and last threshold
     int slots;             // lists per query
     int *status;
@@ -177,54 +179,71 @@ __device__ __noinline__ ListEnd compact_rows(unsigned rows, int cnt, uint64_t *m
         rows &= rows - 1;
         const int nb = __shfl_sync(kFull, cnt, r);  // more than 32 J - 32 >= KP
         uint64_t *L = reinterpret_cast<uint64_t *>(__shfl_sync(kFull, reinterpret_cast<unsigned long long>(mine), r));
-        uint64_t key[J];
+        // (the scores only: with whole keys in registers the call would cost the
+        // epilogue more spills)
+        uint32_t o[J];
 #pragma unroll
         for (int j = 0; j < J; ++j)
-            key[j] = 32 * j + lane < nb ? L[32 * j + lane] : kKeyMax;
+            o[j] = 32 * j + lane < nb ? static_cast<uint32_t>(L[32 * j + lane] >> 32) : 0xffffffffu;
         uint32_t v = 0;   // the leading bits of the KP-th smallest score
         int left = KP;    // its rank among the keys with those bits
 #pragma unroll 1
         for (uint32_t bit = 0x80000000u; bit; bit >>= 1) {
             int below = 0;  // keys with the bits found so far and a zero here
 #pragma unroll
-            for (int j = 0; j < J; ++j) {
-                const uint32_t o = static_cast<uint32_t>(key[j] >> 32);
-                below += __popc(__ballot_sync(kFull, (o ^ v) < bit));
-            }
+            for (int j = 0; j < J; ++j)
+                below += __popc(__ballot_sync(kFull, (o[j] ^ v) < bit));
             if (below < left) {
                 left -= below;
                 v |= bit;
             }
         }
+        unsigned keep = 0, equal = 0;  // bit j: of the lane's j-th key
         int same = 0;
 #pragma unroll
-        for (int j = 0; j < J; ++j)
-            same += __popc(__ballot_sync(kFull, static_cast<uint32_t>(key[j] >> 32) == v));
+        for (int j = 0; j < J; ++j) {
+            keep |= (o[j] < v ? 1u : 0u) << j;
+            equal |= (o[j] == v ? 1u : 0u) << j;
+            same += __popc(__ballot_sync(kFull, o[j] == v));
+        }
         uint32_t cut = 0xffffffffu;  // the last id kept of that score
         if (same > left) {
             cut = 0;
+#pragma unroll
+            for (int j = 0; j < J; ++j)
+                o[j] = equal >> j & 1 ? static_cast<uint32_t>(L[32 * j + lane]) : 0xffffffffu;  // ids are 31 bits
 #pragma unroll 1
-            for (uint32_t bit = 0x80000000u; bit; bit >>= 1) {
+            for (uint32_t bit = 0x40000000u; bit; bit >>= 1) {
                 int below = 0;
 #pragma unroll
                 for (int j = 0; j < J; ++j)
-                    below += __popc(__ballot_sync(kFull, static_cast<uint32_t>(key[j] >> 32) == v &&
-                                                             (static_cast<uint32_t>(key[j]) ^ cut) < bit));
+                    below += __popc(__ballot_sync(kFull, (o[j] ^ cut) < bit));
                 if (below < left) {
                     left -= below;
                     cut |= bit;
                 }
             }
-        }
-        const uint64_t most = static_cast<uint64_t>(v) << 32 | cut;
-        int at = 0;
 #pragma unroll
-        for (int j = 0; j < J; ++j) {
-            const bool in = key[j] <= most;
-            const unsigned m = __ballot_sync(kFull, in);
-            if (in)
-                L[at + __popc(m & lanemask_lt())] = key[j];
-            at += __popc(m);
+            for (int j = 0; j < J; ++j)
+                equal &= ~((o[j] > cut ? 1u : 0u) << j);
+        }
+        keep |= equal;
+        int at = 0;
+        constexpr int B = J % 8 ? J : 8;  // keys read before any place up to theirs is written
+#pragma unroll 1
+        for (int j0 = 0; j0 < J; j0 += B) {
+            uint64_t x[B];
+#pragma unroll
+            for (int j = 0; j < B; ++j)
+                x[j] = keep >> (j0 + j) & 1 ? L[32 * (j0 + j) + lane] : 0;
+#pragma unroll
+            for (int j = 0; j < B; ++j) {
+                const bool in = keep >> (j0 + j) & 1;
+                const unsigned m = __ballot_sync(kFull, in);
+                if (in)
+                    L[at + __popc(m & lanemask_lt())] = x[j];
+                at += __popc(m);
+            }
         }
         if (lane == r) {
             cnt = KP;
@@ -269,11 +288,11 @@ __device__ __forceinline__ void tmem_landed(uint32_t (&r)[32])
 
 // Keys that a list holds: about what a search of a million rows in random order
 // appends, and well above what a compaction leaves.
-constexpr int list_keys(int KR) { return KR == 1 ? 160 : KR <= 32 ? 256 : 512; }
+constexpr int list_keys(int KPL, int KR) { return KR == 1 ? 160 : 128 * KPL; }
 
 // P planes (1: BF16 values, 3: fp32 split), 32 KPL candidates kept of a list that
-// fills, KR >= k scores in registers, EW epilogue warps, MULTI: more than one
-// phase (128 coordinates) a tile.
+// fills, KR scores in registers (SPLIT: half as many as k), MULTI: more than
+// one phase (128 coordinates) a tile.
 // A persistent CTA per SM takes a contiguous range of the (query tile, base
 // tile) pairs in row-major order, so the ranges differ by at most one tile
 // whatever the shape, and a query tile is shared by two or three CTAs at most
@@ -286,7 +305,7 @@ constexpr int list_keys(int KR) { return KR == 1 ? 160 : KR <= 32 ? 256 : 512; }
 //               high of either chunk) in rotation: the next phase's small
 //               products go to the fourth while the epilogue reads these.  P =
 //               1 fills one, of two in turn;
-//   warps 2..   one query and (EW = 8) half of a tile's columns per thread: score,
+//   warps 2..9  one query and half of a tile's columns per thread: score,
 //               compare with the query's threshold.  The few that pass are
 //               appended to the thread's list in memory and their scores enter
 //               its k best, kept sorted in registers (KR of them), so that the
@@ -298,6 +317,12 @@ constexpr int list_keys(int KR) { return KR == 1 ? 160 : KR <= 32 ? 256 : 512; }
 //               every column that passes in some lane: 9.4 and 4.6 ms; the k
 //               smallest minima of groups of eight columns: 28.8 and 5.0 ms.)
 //               The two threads of a query share their thresholds once a tile.
+//               SPLIT, for k > 32: each keeps the k / 2 best (rounded up) of its
+//               own columns, and the larger of their last ones stands for the
+//               k-th of all: half the registers and insertions (10,000 queries
+//               among 30,000 rows of 64 coordinates: k = 64 1,179 us with all 64
+//               scores in either thread's registers, 687 us; k = 100 3,711 us with
+//               128 in those of four warps, 956 us).
 // The A images of a query tile stay in shared memory when they fit (K x P <=
 // six images: 128 fp32 or 384 uint8 coordinates), else they stream with the
 // base's.  The threshold is the k-th best score plus what the scores' errors
@@ -306,9 +331,10 @@ constexpr int list_keys(int KR) { return KR == 1 ? 160 : KR <= 32 ? 256 : 512; }
 // of scores and a pass that selects from them 23.3 ms; 4.5 ms here, six products
 // at 1,030 TFLOP/s, 55 % of the measured BF16 rate (bounded by shared-memory
 // reads of the N = 128 MMAs and the epilogue's hand-over).  960 coordinates:
-// 790 TFLOP/s, the operands streaming from L2.
-template <int P, int KPL, int KR, int EW, bool MULTI>
-__global__ void __launch_bounds__(64 + 32 * EW, 1) knn_tile_kernel(const KnnArgs a)
+// 790 TFLOP/s, the operands streaming from L2 and the epilogue's sums of several
+// phases spilling (MULTI: 304 to 720 bytes a thread up to KR = 64).
+template <int P, int KPL, int KR, bool SPLIT, bool MULTI>
+__global__ void __launch_bounds__(64 + 32 * kEpiWarps, 1) knn_tile_kernel(const KnnArgs a)
 {
     extern __shared__ __align__(1024) uint8_t smem[];
     float *sny = reinterpret_cast<float *>(smem + kOffNy);
@@ -327,7 +353,7 @@ __global__ void __launch_bounds__(64 + 32 * EW, 1) knn_tile_kernel(const KnnArgs
         }
         for (int i = 0; i < 2; ++i) {
             mbar_init(&bars->acc_full[i], 1);
-            mbar_init(&bars->acc_empty[i], EW);
+            mbar_init(&bars->acc_empty[i], kEpiWarps);
         }
         fence_mbar_init();
     }
@@ -494,7 +520,7 @@ __global__ void __launch_bounds__(64 + 32 * EW, 1) knn_tile_kernel(const KnnArgs
         }
     } else {
         // ---- epilogue: thread = query row of the tile and its columns, or half of them
-        constexpr int kHalves = EW / 4, kCap = list_keys(KR);
+        constexpr int kHalves = kEpiWarps / 4, kCap = list_keys(KPL, KR);
         constexpr int kCols = kTile / kHalves;
         const int quad = warp & 3;         // a warp reads its own quarter of the TMEM lanes
         const int half = (warp - 2) >> 2;  // warps 2..5 the first half of the columns, 6..9 the second
@@ -502,11 +528,14 @@ __global__ void __launch_bounds__(64 + 32 * EW, 1) knn_tile_kernel(const KnnArgs
         const uint32_t my_lane = tmem + (static_cast<uint32_t>(quad * 32) << 16) + half * kCols;
         const float nmax = __uint_as_float(*a.nmax);
         float coef = 0.f;
-        // the k best scores in best[KR - k .. KR), ascending; the places below
-        // never take one
+        // the `keep` best scores in best[KR - keep .. KR), ascending; the places
+        // below never take one
+        const int keep = SPLIT ? (a.k + 1) / 2 : a.k;
         float best[KR];
+        float other = INFINITY;  // SPLIT: the other half's last one
         // scores up to thr pass (all, when it is NaN), but of those equal to cut, the
-        // list's last score at its last compaction, only ids below cut_id
+        // list's last score at its last compaction, only in groups of columns that
+        // begin below cut_id (a few more than could enter)
         float thr = 0.f, slack = 0.f, cut = 0.f;
         uint32_t cut_id = 0;
         int cnt = 0;
@@ -539,7 +568,7 @@ __global__ void __launch_bounds__(64 + 32 * EW, 1) knn_tile_kernel(const KnnArgs
                 cnt = max(static_cast<int>(end.x), 0);
 #pragma unroll
                 for (int i = 0; i < KR; ++i)
-                    best[i] = i < KR - a.k ? -INFINITY : INFINITY;
+                    best[i] = i < KR - keep ? -INFINITY : INFINITY;
                 // an infinite query's products, whatever their size, stand for
                 // infinities of their sign; a NaN's scores are all NaN, so that
                 // the ids decide
@@ -547,9 +576,13 @@ __global__ void __launch_bounds__(64 + 32 * EW, 1) knn_tile_kernel(const KnnArgs
                 coef = nx == nx ? (isinf(nx) ? -FLT_MAX : a.ip ? -1.f : -2.f) : nx;
                 slack = score_slack(nx, nmax, a.dim, a.ip);
                 self = a.self ? static_cast<uint32_t>(a.row0 + row) : 0xffffffffu;
+                if constexpr (SPLIT) {  // read after the meeting below
+                    other = INFINITY;
+                    sthr[half * kTile + m] = __float_as_uint(INFINITY);
+                }
                 pad = row >= a.rows;  // a padding row: no score is below its threshold
                 thr = pad ? -INFINITY : __uint_as_float(end.y);
-                cut = pad ? thr : __int_as_float(0x7fffffff);
+                cut = __int_as_float(0x7fffffff);
                 cut_id = 0;
             }
             uint32_t *shared_thr = sthr + (seg & 1) * kTile;
@@ -618,7 +651,7 @@ __global__ void __launch_bounds__(64 + 32 * EW, 1) knn_tile_kernel(const KnnArgs
                     "{\n\t.reg .pred p, q;\n\tsetp.ne.s32 p, %1, 0;\n\t"
                     "bar.red.or.pred q, 1, %2, p;\n\tselp.s32 %0, 1, 0, q;\n\t}"
                     : "=r"(any)
-                    : "r"(dead), "n"(32 * EW)
+                    : "r"(dead), "n"(32 * kEpiWarps)
                     : "memory");
                 ok = any == 0;
                 tc_fence_after();
@@ -630,6 +663,20 @@ __global__ void __launch_bounds__(64 + 32 * EW, 1) knn_tile_kernel(const KnnArgs
                 if (lane == 0)
                     mbar_arrive(&bars->acc_empty[ph & 1]);
                 ++ph;
+            };
+            // short of k scores, everything passes still
+            auto lower_thr = [&]() {
+                const float kth = SPLIT ? fmaxf(best[KR - 1], other) : best[KR - 1];
+                thr = kth < INFINITY ? fminf(thr, kth + slack) : thr;
+            };
+            // SPLIT, any time after the tile's first meeting: the halves' last scores.
+            // A half sets its word back before the next query tile's first meeting,
+            // at which this one must be too.
+            auto exchange = [&]() {
+                volatile uint32_t *word = sthr;
+                word[half * kTile + m] = __float_as_uint(best[KR - 1]);
+                other = fminf(other, __uint_as_float(word[(half ^ 1) * kTile + m]));
+                lower_thr();
             };
             auto score = [&](int cc, float (&s)[32]) {
                 const float4 *ny4 = reinterpret_cast<const float4 *>(sny + b * kTile + half * kCols + cc);
@@ -645,23 +692,18 @@ __global__ void __launch_bounds__(64 + 32 * EW, 1) knn_tile_kernel(const KnnArgs
                 }
                 if (!__any_sync(kFull, !(lo > thr)))
                     return;
+                if constexpr (SPLIT)
+                    exchange();
                 // the columns that pass, then every lane its own one after
                 // another: a few turns, not one for every column that passes
                 // in some lane
                 const uint32_t id0 = static_cast<uint32_t>(a.col0 + c0) + half * kCols + cc;
+                // past cut_id, scores below the cut: up to the float before it
+                const float most = thr == cut && id0 >= cut_id && thr > -INFINITY ? ord_to_f32(f32_to_ord(thr) - 1) : thr;
                 unsigned todo = 0;
 #pragma unroll
                 for (int j = 0; j < 32; ++j)
-                    todo |= (s[j] > thr ? 0u : 1u) << j;
-                if (__any_sync(kFull, thr == cut)) {
-                    unsigned equal = 0;
-#pragma unroll
-                    for (int j = 0; j < 32; ++j)
-                        equal |= (s[j] == cut ? 1u : 0u) << j;
-                    const uint32_t ids = cut_id > id0 ? cut_id - id0 : 0;
-                    if (thr == cut && ids < 32)
-                        todo &= ~(equal & ~((1u << ids) - 1u));
-                }
+                    todo |= (s[j] > most ? 0u : 1u) << j;
                 if (width - cc < 32)
                     todo &= width > cc ? (1u << (width - cc)) - 1u : 0u;
                 if (self - id0 < 32)
@@ -699,16 +741,17 @@ __global__ void __launch_bounds__(64 + 32 * EW, 1) knn_tile_kernel(const KnnArgs
                             x = fmaxf(best[i], x);
                             best[i] = lower;
                         }
-                        // short of k scores, everything passes still
-                        thr = best[KR - 1] < INFINITY ? fminf(thr, best[KR - 1] + slack) : thr;
+                        lower_thr();
                     }
                     todo &= todo - 1;
                 }
             };
-            // after the tile's first meeting: nobody reads the other copy of
-            // the shared thresholds any more, the next query tile's
+            // After the tile's first meeting: nobody reads the other copy of the
+            // shared thresholds any more, the next query tile's.
             auto begin = [&]() {
-                if constexpr (kHalves > 1) {
+                if constexpr (SPLIT) {
+                    exchange();
+                } else {
                     if (fresh && half == 0)
                         sthr[((seg & 1) ^ 1) * kTile + m] = 0xffffffffu;
                     if (thr == thr && !pad)
@@ -840,17 +883,22 @@ __global__ void __launch_bounds__(256) norms_kernel(const S *x, int64_t rows, in
     float mx = 0.f;
     for (int64_t r = blockIdx.x * 8ll + w; r < rows; r += gridDim.x * 8ll) {
         float s = 0.f;
-        bool inf = false;
         for (int c = lane; c < dim; c += 32) {
             const float v = static_cast<float>(x[r * dim + c]);
             s = fmaf(v, v, s);
-            inf |= isinf(v);
         }
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1)
             s += __shfl_xor_sync(kFull, s, o);
-        if (!__any_sync(kFull, inf))
-            s = s > FLT_MAX ? FLT_MAX : s;
+        if constexpr (sizeof(S) == 4) {
+            if (isinf(s)) {  // every lane has the sum
+                bool inf = false;
+                for (int c = lane; c < dim; c += 32)
+                    inf |= isinf(x[r * dim + c]);
+                if (!__any_sync(kFull, inf))
+                    s = FLT_MAX;
+            }
+        }
         if (lane == 0)
             out[r] = s;
         mx = fmaxf(mx, isfinite(s) ? s : 0.f);
@@ -1090,17 +1138,17 @@ unsigned pack_grid(int64_t rows, int chunks)
         std::min<int64_t>(((rows + kTile - 1) / kTile * chunks * (kTile * 8) + 255) / 256, 152 * 32));
 }
 
-template <typename S, int P, int KPL, int KR, int EW>
+template <typename S, int P, int KPL, int KR, bool SPLIT>
 ann_status knn_typed(const S *base, int64_t n, int dim, int metric, const S *queries, int64_t nq, int k,
                      bool exclude_self, int32_t *d_ids, void *d_dists, cudaStream_t s)
 {
-    constexpr int kCap = list_keys(KR), kShare = 16;
+    constexpr int kCap = list_keys(KPL, KR), kShare = 16;
     const int chunks = (dim + 63) / 64;
     const size_t tile_bytes = static_cast<size_t>(chunks) * P * kImage;
     int dev = 0, sms = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    auto kern = chunks > 2 ? knn_tile_kernel<P, KPL, KR, EW, true> : knn_tile_kernel<P, KPL, KR, EW, false>;
+    auto kern = chunks > 2 ? knn_tile_kernel<P, KPL, KR, SPLIT, true> : knn_tile_kernel<P, KPL, KR, SPLIT, false>;
     KNN_CK(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kKnnSmem));
     // blocks of base rows and of queries whose packed images stay within 1 GB
     // and 256 MB, and of queries whose lists stay within 512 MB
@@ -1120,7 +1168,7 @@ ann_status knn_typed(const S *base, int64_t n, int dim, int metric, const S *que
         if (unit_of(tm, tn) == 1)
             for (int64_t i = 0; i < tm; ++i)
                 most = std::max(most, cta_of_tile((i + 1) * tn - 1, T, G) - cta_of_tile(i * tn, T, G) + 1);
-        return most * (EW / 4);
+        return most * (kEpiWarps / 4);
     };
     // Base tiles are met by the golden section of their number, all CTAs alike (they
     // share them in L2).  In their own order, rows that lie along a path would
@@ -1206,7 +1254,7 @@ ann_status knn_typed(const S *base, int64_t n, int dim, int metric, const S *que
             a.ends = ends.as<uint2>();
             a.slots = static_cast<int>(slots);
             a.status = status;
-            kern<<<static_cast<unsigned>(grid_of(tm, tn)), 64 + 32 * EW, kKnnSmem, s>>>(a);
+            kern<<<static_cast<unsigned>(grid_of(tm, tn)), 64 + 32 * kEpiWarps, kKnnSmem, s>>>(a);
             KNN_CK(cudaGetLastError());
         }
         const int rowbytes = dim * static_cast<int>(sizeof(S));
@@ -1214,9 +1262,9 @@ ann_status knn_typed(const S *base, int64_t n, int dim, int metric, const S *que
         const uint8_t *qq = reinterpret_cast<const uint8_t *>(queries + q0 * dim);
         int32_t *oi = d_ids + q0 * k;
         void *od = static_cast<uint8_t *>(d_dists) + q0 * k * 4;
-        // up to four queries an SM, sixteen warps each: below, one warp a query
-        // leaves most of the chip idle
-        const bool few = rows <= 4 * int64_t{sms};
+        // up to a query an SM, where one warp a query leaves the chip idle (500
+        // queries, k = 100: 118 us by one warp each, 150 by sixteen)
+        const bool few = rows <= sms;
         auto rescore = [&](auto one, auto shared) {
             (few ? shared : one)<<<static_cast<unsigned>(few ? rows : (rows + 3) / 4), few ? 32 * kShare : 128, 0, s>>>(
                 bb, rowbytes, qq, rowbytes, dim, rows, lists.as<uint64_t>(), ends.as<uint2>(), static_cast<int>(slots),
@@ -1236,22 +1284,22 @@ ann_status knn_typed(const S *base, int64_t n, int dim, int metric, const S *que
     return failed ? ANN_ERR_TIMEOUT : ANN_OK;
 }
 
-// k nearest by the kernel with as many scores in registers as k needs; k > 64
-// takes half the epilogue warps, whose threads then have registers for 128.
+// k nearest by the kernel with as many scores in registers as k needs, past 32 as
+// half of it needs.
 template <typename S, int P>
 ann_status knn_by_k(const S *base, int64_t n, int dim, int metric, const S *queries, int64_t nq, int k,
                     bool exclude_self, int32_t *d_ids, void *d_dists, cudaStream_t s)
 {
     auto run = [&](auto fn) { return fn(base, n, dim, metric, queries, nq, k, exclude_self, d_ids, d_dists, s); };
     if (k == 1)
-        return run(knn_typed<S, P, 2, 1, 8>);
+        return run(knn_typed<S, P, 2, 1, false>);
     if (k <= 16)
-        return run(knn_typed<S, P, 2, 16, 8>);
+        return run(knn_typed<S, P, 2, 16, false>);
     if (k <= 32)
-        return run(knn_typed<S, P, 2, 32, 8>);
+        return run(knn_typed<S, P, 2, 32, false>);
     if (k <= 64)
-        return run(knn_typed<S, P, 4, 64, 8>);
-    return run(knn_typed<S, P, 4, 128, 4>);
+        return run(knn_typed<S, P, 4, 32, true>);
+    return run(knn_typed<S, P, 4, 64, true>);
 }
 
 }  // namespace

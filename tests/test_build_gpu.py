@@ -304,10 +304,10 @@ def test_knn_time_grows_with_the_base():
     assert ms[1] <= 1.25 * 6 * ms[0], ms
 
 
-@pytest.mark.parametrize("nq,k", [(1, 64), (5, 128), (609, 33), (608, 10)])
+@pytest.mark.parametrize("nq,k", [(1, 64), (5, 128), (153, 33), (152, 10)])
 def test_knn_few_queries(nq, k):
     # their lists, one or two of every CTA, are shared by the warps of a CTA (up
-    # to 608 queries, four an SM), whole numbers as in test_knn_edges_exact
+    # to 152 queries, one an SM), whole numbers as in test_knn_edges_exact
     rng = np.random.default_rng(nq)
     base = rng.integers(-3, 4, size=(30_000, 96)).astype(np.float32)
     q = rng.integers(-3, 4, size=(nq, 96)).astype(np.float32)
@@ -449,3 +449,17 @@ def test_builders_give_their_scratch_back():
     assert torch.equal(out[0], first)
     with pytest.raises(ann.AnnError):
         ann.ann_release_scratch(99)
+
+
+@pytest.mark.parametrize("n,nq,d,k", [(20_001, 300, 100, 65), (20_001, 129, 132, 127), (128, 40, 64, 128),
+                                      (200, 1_300, 64, 128), (20_001, 257, 64, 33), (150, 1_300, 260, 64)])
+def test_knn_neighbours_split_over_the_halves(n, nq, d, k):
+    # k > 32: either half of a tile's columns keeps half of the k best scores; the
+    # near rows of a query lie in one half of their tiles
+    rng = np.random.default_rng(n + d)
+    base = rng.integers(-3, 4, size=(n, d)).astype(np.float32)
+    base[:, 0] = np.arange(n) // 64 % 2 * 40
+    q = rng.integers(-3, 4, size=(nq, d)).astype(np.float32)
+    ids, dd = _knn_gpu(base, q, k)
+    oi, od = oracle.knn(base, q.astype(np.float64), k)
+    assert np.array_equal(ids, oi) and np.array_equal(dd.astype(np.float64), od)
