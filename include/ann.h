@@ -110,10 +110,11 @@ typedef struct {
  *   W         pool entries expanded per step, 1..ANN_MAX_W, W*degree <= 128
  *   hash_bits log2 of the per-query shared-memory visited-table capacity,
  *             0 = chosen: the largest up to 32 KB that leaves every SM its
- *             share of the queries, else none; 8..15; -1 = no shared table (the
+ *             share of the queries, else none (but never none where spill_bits
+ *             asks for global tables that hold less); 8..15; -1 = no shared table (the
  *             visited set lives in the global spill tables from the first step)
  *   stage_rows neighbour rows gathered into shared memory per round, 0 =
- *             chosen from the row size and nq; 1..32.  hash_bits and stage_rows change
+ *             chosen from the row size, team and nq; 1..32.  hash_bits and stage_rows change
  *             speed only, never results (see ann_autotune)
  *   team      lanes that compute one distance together (the warp evaluates
  *             32/team staged rows at a time), 0 = chosen from the row size;
@@ -344,7 +345,8 @@ ann_status ann_plan_free(ann_plan *plan);
  * *best the copy of *p with the fastest combination (*best_ms: its time per
  * batch).  The stages:
  *   1. hash_bits (no shared table, and sizes around and below the default)
- *      x stage_rows 4, 6, 8, 12, 16;
+ *      x stage_rows 4, 6, 8, 12, 16, with bulk copies (gather 1 where 0 would
+ *      mean 4) unless p fixes the mode;
  *   2. team 2 to 32, where a lane gets 1 to 16 16-byte chunks of the row;
  *   3. spill_bits up to two either side of the default;
  *   4. gather 4 (when the index's rows allow TMA tensor gathers) with
@@ -703,8 +705,8 @@ ann_status ann_topo_tokens(ann_index *idx, const int32_t *d_hubs, int32_t H, int
  *   d_centroids  out (optional): k^levels x dim fp32 final centroids
  *   d_label      out (optional): n int32 final cluster of every row
  * Blocking.  Errors: ANN_ERR_INVALID_ARG for a NULL input or output, bad
- * sizes or alignment; ANN_ERR_UNSUPPORTED when k x dim floats do not fit in
- * one block's shared memory.
+ * sizes or alignment; ANN_ERR_UNSUPPORTED when k x dim floats are more than 227
+ * KB.
  */
 ann_status ann_hbkm(const float *d_x, int64_t n, int32_t dim, int32_t k, int32_t levels, double lambda, int32_t T,
                     const uint32_t *d_keys, int32_t *d_hubs, float *d_centroids, int32_t *d_label, void *stream);
@@ -780,9 +782,12 @@ ann_status ann_merge_shards(const int32_t *d_ids, const void *d_dists, int32_t P
 /*
  * Exact k nearest neighbours (Sec. 2.1, Problem 1; the ground truth R of
  * recall@k): for each of nq query rows, the k base rows with the smallest
- * (distance, id).  Candidate scores come from the tensor cores; every candidate
- * that their error leaves in question is re-scored exactly (int32 for uint8,
- * fp32 direct differences otherwise) and sorted.
+ * (distance, id).  Candidate scores come from the tensor cores; of the best 64 (k
+ * <= 32) or 128 by score, those that the scores' error leaves in question are
+ * re-scored exactly (int32 for uint8, fp32 direct differences otherwise) and
+ * sorted.  So the answer is exact while the k nearest are among those: scores
+ * are within about 1e-7 |x| |y| (fp32), which neighbours at the last places of a
+ * large k, or rows far from the origin, can come closer than.
  *   d_base       n*dim base rows (dtype ANN_U8 or ANN_F32), 16-byte aligned
  *   d_queries    nq*dim rows of the same dtype; equal to d_base when
  *                exclude_self != 0 (then row i never returns id i)

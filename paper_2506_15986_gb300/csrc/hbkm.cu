@@ -782,10 +782,12 @@ ann_status ann_hbkm(const float *d_x, int64_t n, int32_t dim, int32_t k, int32_t
                                                                        cent.as<float>(), cent2.as<float>());
         // large clusters: position tiles (a tile spans one or two clusters)
         // and the visit by rounds of 512 members; below, pairs and warps.
-        // A visit by rounds assumes sizes up to 512 members old: its
-        // uncertain members grow as the round's share of a cluster.  At 1 % of a
-        // cluster it is 6.6 times as fast as one by one, at 27 % (1,875 members)
-        // 2.3 times as slow; the line lies between, at 6 %.
+        // A visit by rounds assumes sizes up to 512 members old: its uncertain
+        // members grow as the round's share of a cluster.  One cluster, k = 32, ten
+        // iterations (ms, by rounds | one by one): 32,768 members 6.1 | 28.7, 8,192
+        // 4.0 | 7.5, 4,096 3.3 | 4.0, 1,024 1.2 | 1.3; with lambda = 10, where rounds
+        // end one by one, 6.9 | 7.5 at 8,192.  Below the line a level has many
+        // clusters, of which a warp each fills the chip with fewer registers.
         const bool tiles = n / P >= kDistTile;
         const bool rounds = n / P >= kVisitMinMembers;
         for (int it = 0; it < T; ++it) {
