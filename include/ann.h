@@ -111,7 +111,8 @@ typedef struct {
  *   hash_bits log2 of the per-query shared-memory visited-table capacity,
  *             0 = chosen: the largest up to 32 KB that leaves every SM its
  *             share of the queries, else none (but never none where spill_bits
- *             asks for global tables that hold less); 8..15; -1 = no shared table (the
+ *             asks for global tables that hold less); 8..15 (at most the first
+ *             global table's, where the second one holds as much); -1 = no shared table (the
  *             visited set lives in the global spill tables from the first step)
  *   stage_rows neighbour rows gathered into shared memory per round, 0 =
  *             chosen from the row size, team and nq; 1..32.  hash_bits and stage_rows change

@@ -419,7 +419,11 @@ ann_status launch_search(ann_index *idx, const SearchLaunch &L, cudaStream_t s)
         // without it the visited set has the global tables only, which must hold as
         // much (they do unless the caller asks for small ones)
         const int none = sb + 2 >= table ? -1 : table;
-        const int tables[2] = {p->hash_bits ? p->hash_bits : table, p->hash_bits ? p->hash_bits : none};
+        // a full shared table hands its keys to the first global one, which must
+        // have room for them; the second one then holds what it would have held
+        // itself (if not, the query fails, as it says)
+        auto within = [&](int hb) { return hb > sb && hb <= sb + 2 ? sb : hb; };
+        const int tables[2] = {within(p->hash_bits ? p->hash_bits : table), within(p->hash_bits ? p->hash_bits : none)};
         const int kRows[] = {32, 24, 16, 12, 8, 4};
         int r0 = want < kFullTeams ? 0 : 1, r1 = a.stage_stride > 1024 ? 6 : 5;
         while (r1 > 1 && kRows[r1 - 1] < 32 >> a.team_lg)

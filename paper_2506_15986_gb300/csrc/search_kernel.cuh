@@ -509,8 +509,9 @@ __global__ void __launch_bounds__(32 * kMaxSearchWarps, 16) beam_search_kernel(c
         // the first global table's size: the launch's, or the query's own L's,
         // so that a small query of a mixed batch clears and touches a small
         // table (the second one keeps the launch's size, so no query's
-        // capacity shrinks)
-        const int qbits = a.spill_by_query ? min(spill_bits_for(max(Lq, 1)), a.spill_bits) : a.spill_bits;
+        // capacity shrinks), never smaller than the shared one, whose keys it takes
+        const int qbits =
+            a.spill_by_query ? min(max(spill_bits_for(max(Lq, 1)), a.hash_bits), a.spill_bits) : a.spill_bits;
         int level = shared_tab ? 0 : 1, used = 0, gbits = qbits;
         int limit = shared_tab ? hlimit : (1 << qbits) * 3 / 4;
         uint32_t *gtab = gtab1;

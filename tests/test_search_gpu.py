@@ -538,3 +538,33 @@ def test_short_rounds_keep_every_team_busy():
         assert torch.equal(ia, ib) and a <= 1.27 * b, (a, b)
     finally:
         ann.ann_free_index(h)
+
+
+@pytest.mark.parametrize("R,L,W,knobs,mixed", [(32, 512, 4, dict(hash_bits=13, spill_bits=12), False),
+                                               (32, 512, 2, dict(hash_bits=11, spill_bits=10), False),
+                                               (128, 282, 1, {}, True), (128, 282, 1, dict(hash_bits=13), True)])
+def test_visited_keys_survive_a_smaller_first_table(R, L, W, knobs, mixed):
+    # a shared table that outgrows the first global one: asked for so, or by a query
+    # whose own L is small; no node is evaluated twice, as with tables that are
+    # never left
+    rng = np.random.default_rng(R)
+    n = 12_000
+    x = rng.standard_normal((n, 16)).astype(np.float32)
+    g = rng.integers(0, n, size=(n, R)).astype(np.int32)
+    q = rng.standard_normal((200, 16)).astype(np.float32)
+    own = dict(Ls=rng.integers(10, L + 1, size=200), ks=np.full(200, 10)) if mixed else {}
+    h = make_index(x, g, 0)
+    try:
+        a = search(h, q, 10, L, W=W, hash_bits=-1, spill_bits=16, **own)
+        b = search(h, q, 10, L, W=W, **knobs, **own)
+    finally:
+        ann.ann_free_index(h)
+    small = own["Ls"] <= 76 if mixed else slice(None)
+    assert a[4] == ann.OK and a[2][small].max() > (1536 if knobs.get("hash_bits") == 11 else 6144)
+    if knobs.get("spill_bits") == 10:  # 3,072 keys at most: failed queries say so
+        assert b[4] in (ann.OK, ann.ERR_CAPACITY)
+        done = b[0][:, 0] >= 0
+    else:
+        assert b[4] == ann.OK
+        done = np.ones(200, bool)
+    assert all(np.array_equal(u[done], v[done]) for u, v in zip(a[:4], b[:4]))
