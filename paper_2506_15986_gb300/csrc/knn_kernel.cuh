@@ -157,7 +157,7 @@ __device__ __forceinline__ void merge_sorted(uint64_t (&T)[KPL], uint64_t v, int
 // which bounds what a list takes in when the slack hides every
 // difference between the scores (rows far from the origin, or one row farther
 // than the rest): 10,000 queries among 300,000 rows of 128 coordinates, k = 10,
-// one row of 1e20: 148 ms without the cut, 8.9 ms with it; 4.7 ms without that
+// one row of 1e20: 148 ms without the cut, 8.6 ms with it; 4.6 ms without that
 // row.  The KP-th smallest score is found bit by bit over the keys in
 // registers, and where it cuts equal scores their ids'; sorting the list 32 keys
 // at a time instead took 12.8 ms, its warp's chain of shuffles holding up the
@@ -332,7 +332,7 @@ constexpr int list_keys(int KPL, int KR) { return KR == 1 ? 160 : 128 * KPL; }
 // at 1,030 TFLOP/s, 55 % of the measured BF16 rate (bounded by shared-memory
 // reads of the N = 128 MMAs and the epilogue's hand-over).  960 coordinates:
 // 790 TFLOP/s, the operands streaming from L2 and the epilogue's sums of several
-// phases spilling (MULTI: 304 to 720 bytes a thread up to KR = 64).
+// phases spilling (MULTI: 324 to 536 bytes a thread).
 template <int P, int KPL, int KR, bool SPLIT, bool MULTI>
 __global__ void __launch_bounds__(64 + 32 * kEpiWarps, 1) knn_tile_kernel(const KnnArgs a)
 {
