@@ -134,6 +134,13 @@ MEASURED_TRAFFIC = {
         dict(digest="38c0a0976680fa9a", entry="exhaustive", L=93, nq=10_000, hash_bits=-1, stage_rows=8,
              team=4, spill_bits=12, gather=4, visited_l2=True, group_entries=False,
              bytes=((3.4414e9 + 0.0111e9) + (3.4380e9 + 0.0158e9) + (3.4343e9 + 0.0204e9)) / 3),
+        # and both orders with a bulk copy per row
+        dict(digest="38c0a0976680fa9a", entry="exhaustive", L=93, nq=10_000, hash_bits=-1, stage_rows=8,
+             team=4, spill_bits=12, gather=0, visited_l2=True, group_entries=True,
+             bytes=((2.9231e9 + 0.0051e9) + (2.9208e9 + 0.0080e9) + (2.9196e9 + 0.0107e9)) / 3),
+        dict(digest="38c0a0976680fa9a", entry="exhaustive", L=93, nq=10_000, hash_bits=-1, stage_rows=8,
+             team=4, spill_bits=12, gather=0, visited_l2=True, group_entries=False,
+             bytes=((3.3623e9 + 0.0054e9) + (3.3601e9 + 0.0087e9) + (3.3578e9 + 0.0121e9)) / 3),
     ],
 }
 
